@@ -211,31 +211,33 @@ constexpr int TRI_UNROLL = 4;
 constexpr int TW_HASH = 2 * TRI_WARP_MAX;   // slots of a warp's table (load <= 1/2)
 constexpr int TM_HASH = 2 * TRI_MID_MAX;    // slots of a block's table
 
-template <int HS, typename IdxT>
-__device__ __forceinline__ int tri_lookup(const int32_t *hk, const IdxT *hp, int32_t w) {
-    uint32_t h = hash32((uint32_t)w) & (HS - 1);
-    for (int probe = 0; probe < HS; ++probe) {
+// (hm: slots - 1; the slots are a power of two, at least twice the ids)
+template <typename IdxT>
+__device__ __forceinline__ int tri_lookup(const int32_t *hk, const IdxT *hp, uint32_t hm, int32_t w) {
+    uint32_t h = hash32((uint32_t)w) & hm;
+    for (uint32_t probe = 0; probe <= hm; ++probe) {
         const int32_t k = hk[h];
         if (k == w) return (int)hp[h];
         if (k == -1) return -1;
-        h = (h + 1) & (HS - 1);
+        h = (h + 1) & hm;
     }
     return -1;
 }
 
-template <int HS, typename IdxT>
-__device__ __forceinline__ void tri_insert(int32_t *hk, IdxT *hp, int32_t v, int k) {
-    uint32_t h = hash32((uint32_t)v) & (HS - 1);
-    while (atomicCAS(&hk[h], -1, v) != -1) h = (h + 1) & (HS - 1);
+template <typename IdxT>
+__device__ __forceinline__ void tri_insert(int32_t *hk, IdxT *hp, uint32_t hm, int32_t v, int k) {
+    uint32_t h = hash32((uint32_t)v) & hm;
+    while (atomicCAS(&hk[h], -1, v) != -1) h = (h + 1) & hm;
     hp[h] = (IdxT)k;
 }
 
 // Elements [e_begin, e_end) of a node's flattened stream, walked by one warp
 // from position p (pre[p] <= e_begin).  Returns this lane's triangle count.
-template <int HS, typename IdxT>
+template <typename IdxT>
 __device__ __forceinline__ int tri_stream(int e_begin, int e_end, int p, const int32_t *pre, const long long *base,
                                           const int32_t *__restrict__ oadj, int32_t lo_id, int32_t hi_id,
-                                          const int32_t *hk, const IdxT *hp, int *cnt, uint8_t *sup, int lane) {
+                                          const int32_t *hk, const IdxT *hp, uint32_t hm, int *cnt, uint8_t *sup,
+                                          int lane) {
     int tu = 0;
     for (int e0 = e_begin; e0 < e_end; e0 += 32 * TRI_UNROLL) {
         int pp[TRI_UNROLL];
@@ -257,7 +259,7 @@ __device__ __forceinline__ int tri_stream(int e_begin, int e_end, int p, const i
 #pragma unroll
         for (int j = 0; j < TRI_UNROLL; ++j) {
             if (pp[j] >= 0 && x[j] >= lo_id && x[j] <= hi_id) {
-                const int idx = tri_lookup<HS, IdxT>(hk, hp, x[j]);
+                const int idx = tri_lookup<IdxT>(hk, hp, hm, x[j]);
                 if (idx >= 0) {
                     atomicAdd(&cnt[idx], 1);
                     atomicAdd(&cnt[pp[j]], 1);
@@ -271,67 +273,182 @@ __device__ __forceinline__ int tri_stream(int e_begin, int e_end, int p, const i
     return tu;
 }
 
-// One warp per node u with 2 <= d+(u) <= TRI_WARP_MAX.
+// Lane holding element e of 32 lists laid end to end (inc: this lane's
+// inclusive prefix sum of their lengths, e below the last one).
+__device__ __forceinline__ int flat_owner(int inc, int e) {
+    int j = 0;
+#pragma unroll
+    for (int b = 16; b > 0; b >>= 1)
+        if (__shfl_sync(FULL, inc, j + b - 1) <= e) j += b;
+    return j;
+}
+
+__device__ __forceinline__ int warp_scan_inclusive(int x, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+// Nodes with 2 <= d+(u) <= TRI_FLAT_MAX.  Their streams are a few elements
+// long, so a warp per node spends its time in the node's chain of dependent
+// loads and in clearing a hash table.  Here a warp lays the out-edges of up to
+// 32 consecutive nodes end to end over its lanes, then the out-lists of 32 such
+// edges, so every lane has an element whatever the lists' lengths, and tests it
+// by a binary search of N+(u) (at most five loads, in the first-level cache: the
+// warp has just read that row).  Triangles are credited by global atomics; the
+// rows are short, so there are few per element.
+// 335k nodes, 0.93M edges: 133 (a warp and a hash table per node) -> 39 us.
+constexpr int TRI_FLAT_MAX = 32;
+
+__global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int32_t *__restrict__ oadj, int64_t n,
+                                                  int run, unsigned long long *tri, uint8_t *sup, DevScalars *ds) {
+    __shared__ unsigned long long s_found[8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    unsigned long long found = 0;
+    for (int64_t u0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * run; u0 < n; u0 += warps * run) {
+        const int64_t u = min(n, u0 + lane);
+        const int64_t s = ooff[u];
+        const int64_t dl = ooff[min(n, u + 1)] - s;
+        const int du = lane < run && dl >= 2 && dl <= TRI_FLAT_MAX ? (int)dl : 0;
+        const int inc = warp_scan_inclusive(du, lane);
+        const int edges = __shfl_sync(FULL, inc, 31);
+        for (int e0 = 0; e0 < edges; e0 += 32) {
+            const int e = e0 + lane;
+            const int j = flat_owner(inc, e);
+            const int64_t us = __shfl_sync(FULL, s, j);
+            const int ud = __shfl_sync(FULL, du, j);
+            const int k = e - (__shfl_sync(FULL, inc, j) - ud);   // position of the edge in N+(u)
+            int32_t v = 0;
+            int64_t vs = 0;
+            int len = 0;
+            if (e < edges) {
+                v = oadj[us + k];
+                vs = ooff[v];
+                len = (int)(ooff[v + 1] - vs);
+            }
+            const int inc2 = warp_scan_inclusive(len, lane);
+            const int total = __shfl_sync(FULL, inc2, 31);
+            int mine = 0;   // triangles closed by this lane's elements
+            for (int f0 = 0; f0 < total; f0 += 32) {
+                const int f = f0 + lane;
+                const int q = flat_owner(inc2, f);
+                const int64_t at = __shfl_sync(FULL, vs, q) + (f - (__shfl_sync(FULL, inc2, q) - __shfl_sync(FULL, len, q)));
+                const int64_t rs = __shfl_sync(FULL, us, q);
+                const int rd = __shfl_sync(FULL, ud, q);
+                const int rk = __shfl_sync(FULL, k, q);
+                const int32_t rv = __shfl_sync(FULL, v, q);
+                const int64_t ru = u0 + __shfl_sync(FULL, j, q);
+                if (f < total) {
+                    const int32_t x = oadj[at];
+                    const int idx = find_sorted(oadj + rs, rd, x);
+                    if (idx >= 0) {
+                        atomicAdd(&tri[ru], 1ull);
+                        atomicAdd(&tri[rv], 1ull);
+                        atomicAdd(&tri[x], 1ull);
+                        sup[at] = 1;
+                        sup[rs + rk] = 1;
+                        sup[rs + idx] = 1;
+                        ++mine;
+                    }
+                }
+                __syncwarp();
+            }
+            found += (unsigned long long)__reduce_add_sync(FULL, mine);
+        }
+    }
+    if (lane == 0) s_found[w] = found;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) found += s_found[k];
+        if (found) atomicAdd(&ds->num_tri, found);
+    }
+}
+
+// One warp per node u with TRI_FLAT_MAX < d+(u) <= TRI_WARP_MAX; warps of a
+// resident grid take runs of up to 32 consecutive nodes, whose offsets load
+// together and of which one ballot picks the ones to do.
 __global__ void __launch_bounds__(256) k_tri_warp(const int64_t *ooff, const int32_t *__restrict__ oadj, int64_t n,
-                                                  unsigned long long *tri, uint8_t *sup, DevScalars *ds) {
+                                                  int run, unsigned long long *tri, uint8_t *sup, DevScalars *ds) {
     __shared__ long long s_base[8][TRI_WARP_MAX];
     __shared__ int32_t s_list[8][TRI_WARP_MAX];
     __shared__ int32_t s_pre[8][TRI_WARP_MAX + 1];
     __shared__ int32_t s_cnt[8][TRI_WARP_MAX];
     __shared__ int32_t s_hk[8][TW_HASH];
     __shared__ uint8_t s_hp[8][TW_HASH];
+    __shared__ unsigned long long s_found[8];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int32_t *list = s_list[w], *pre = s_pre[w], *cnt = s_cnt[w], *hk = s_hk[w];
     long long *base = s_base[w];
     uint8_t *hp = s_hp[w];
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     unsigned long long found = 0;
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
-        const int64_t s = ooff[u];
-        const int du = (int)(ooff[u + 1] - s);
-        if (du < 2 || du > TRI_WARP_MAX) continue;
-        for (int k = lane; k < TW_HASH; k += 32) hk[k] = -1;
-        int carry = 0;
-        for (int k0 = 0; k0 < du; k0 += 32) {
-            const int k = k0 + lane;
-            int len = 0;
-            if (k < du) {
-                const int32_t v = oadj[s + k];
-                const int64_t b = ooff[v];
-                list[k] = v;
-                base[k] = b;
-                len = (int)(ooff[v + 1] - b);
-                cnt[k] = 0;
-            }
-            int x = len;   // inclusive warp scan of the lengths
+    for (int64_t u0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * run; u0 < n; u0 += warps * run) {
+        const int64_t ul = min(n, u0 + lane);
+        const int64_t sl = ooff[ul], dl = ooff[min(n, ul + 1)] - sl;
+        unsigned todo = __ballot_sync(FULL, lane < run && dl > TRI_FLAT_MAX && dl <= TRI_WARP_MAX);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int64_t u = u0 + src;
+            const int64_t s = __shfl_sync(FULL, sl, src);
+            const int du = (int)__shfl_sync(FULL, dl, src);
+            const uint32_t hs = max(32u, 2u << (31 - __clz(2 * du - 1)));   // pow2 >= 2 du
+            for (uint32_t k = lane; k < hs; k += 32) hk[k] = -1;
+            int carry = 0;
+            for (int k0 = 0; k0 < du; k0 += 32) {
+                const int k = k0 + lane;
+                int len = 0;
+                if (k < du) {
+                    const int32_t v = oadj[s + k];
+                    const int64_t b = ooff[v];
+                    list[k] = v;
+                    base[k] = b;
+                    len = (int)(ooff[v + 1] - b);
+                    cnt[k] = 0;
+                }
+                int x = len;   // inclusive warp scan of the lengths
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(FULL, x, o);
-                if (lane >= o) x += y;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (k < du) pre[k + 1] = carry + x;
+                carry += __shfl_sync(FULL, x, 31);
             }
-            if (k < du) pre[k + 1] = carry + x;
-            carry += __shfl_sync(FULL, x, 31);
-        }
-        if (lane == 0) pre[0] = 0;
-        __syncwarp();
-        for (int k = lane; k < du; k += 32) tri_insert<TW_HASH, uint8_t>(hk, hp, list[k], k);
-        __syncwarp();
-        int tu = tri_stream<TW_HASH, uint8_t>(0, pre[du], 0, pre, base, oadj, list[0], list[du - 1], hk, hp, cnt,
-                                              sup, lane);
-        __syncwarp();
-        for (int k = lane; k < du; k += 32) {
-            const int c = cnt[k];
-            if (c > 0) {
-                atomicAdd(&tri[list[k]], (unsigned long long)c);
-                sup[s + k] = 1;
+            if (carry == 0) {   // no out-neighbour has one of its own
+                __syncwarp();
+                continue;
             }
+            if (lane == 0) pre[0] = 0;
+            __syncwarp();
+            for (int k = lane; k < du; k += 32) tri_insert<uint8_t>(hk, hp, hs - 1, list[k], k);
+            __syncwarp();
+            int tu = tri_stream<uint8_t>(0, pre[du], 0, pre, base, oadj, list[0], list[du - 1], hk, hp, hs - 1, cnt,
+                                         sup, lane);
+            __syncwarp();
+            for (int k = lane; k < du; k += 32) {
+                const int c = cnt[k];
+                if (c > 0) {
+                    atomicAdd(&tri[list[k]], (unsigned long long)c);
+                    sup[s + k] = 1;
+                }
+            }
+            tu = __reduce_add_sync(FULL, tu);
+            if (lane == 0 && tu > 0) atomicAdd(&tri[u], (unsigned long long)tu);
+            found += (unsigned long long)tu;
+            __syncwarp();
         }
-        tu = __reduce_add_sync(FULL, tu);
-        if (lane == 0 && tu > 0) atomicAdd(&tri[u], (unsigned long long)tu);
-        found += (unsigned long long)tu;
-        __syncwarp();
     }
-    if (lane == 0 && found) atomicAdd(&ds->num_tri, found);
+    if (lane == 0) s_found[w] = found;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) found += s_found[k];
+        if (found) atomicAdd(&ds->num_tri, found);
+    }
 }
 
 // One 256-thread block per node with TRI_WARP_MAX < d+(u) <= TRI_MID_MAX: the
@@ -391,7 +508,7 @@ __global__ void __launch_bounds__(TRI_MID_THREADS) k_tri_mid(const int64_t *ooff
             run += lens[j];
         }
         if (threadIdx.x == TRI_MID_THREADS - 1) pre[du] = run;
-        for (int k = threadIdx.x; k < du; k += TRI_MID_THREADS) tri_insert<TM_HASH, uint16_t>(hk, hp, list[k], k);
+        for (int k = threadIdx.x; k < du; k += TRI_MID_THREADS) tri_insert<uint16_t>(hk, hp, TM_HASH - 1, list[k], k);
         __syncthreads();
         const int total = pre[du];
         const int eb = (int)((long long)total * w / NW), ee = (int)((long long)total * (w + 1) / NW);
@@ -403,8 +520,8 @@ __global__ void __launch_bounds__(TRI_MID_THREADS) k_tri_mid(const int64_t *ooff
                 const int mid = (lo + hi) >> 1;
                 if (pre[mid + 1] <= eb) lo = mid + 1; else hi = mid;
             }
-            tu = tri_stream<TM_HASH, uint16_t>(eb, ee, lo, pre, base, oadj, list[0], list[du - 1], hk, hp, cnt, sup,
-                                               lane);
+            tu = tri_stream<uint16_t>(eb, ee, lo, pre, base, oadj, list[0], list[du - 1], hk, hp, TM_HASH - 1, cnt,
+                                      sup, lane);
         }
         tu = __reduce_add_sync(FULL, tu);
         if (lane == 0 && tu) atomicAdd(&s_tu, (unsigned long long)tu);
@@ -516,6 +633,15 @@ void set_triangle_attrs() {
     LF_CUDA(cudaFuncSetAttribute(k_tri_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRI_MID_SMEM));
 }
 
+// lf_graph_create takes this path up to this mean out-degree m / n, the
+// middle-vertex kernels above it.  Measured (ms; this path / the other):
+// m/n 2.8 and 335k nodes 0.06 / 0.19, 7.9 and 300k nodes 0.23 / 0.34, 9.1
+// (planted) and 300k nodes 0.21 / 0.30, 11.6 and 200k nodes 0.30 / 0.40, 15 and
+// 100k nodes 0.76 / 0.64, 19 (planted) and 61k nodes 0.22 / 0.25, 28 and 100k nodes
+// 1.82 / 1.04: the streams of the lowest vertices grow faster with the mean
+// degree and its spread.
+constexpr int64_t FLAT_MAX_MEAN = 10;
+
 // Triangle counts and support marks of an oriented graph with n > 0 nodes.
 // `hubs` holds n ints of scratch and `nh` two counters that start at zero.
 // Returns the number of kernels launched.
@@ -524,13 +650,16 @@ int launch_triangles(const int64_t *ooff, const int32_t *oadj, int64_t n, int32_
     const int sms = 152;
     k_select_hubs<<<grid_for(n, 256, 8192), 256, 0, st>>>(ooff, n, hubs, nh);
     LF_LAUNCHED();
-    k_tri_warp<<<grid_for(n * 32, 256, 1 << 16), 256, 0, st>>>(ooff, oadj, n, tri, sup, ds);
+    const int run = (int)std::min<int64_t>(32, std::max<int64_t>(1, n / (2 * 8 * 6 * sms)));
+    k_tri_flat<<<grid_for(n, 8 * run, 6 * sms), 256, 0, st>>>(ooff, oadj, n, run, tri, sup, ds);
+    LF_LAUNCHED();
+    k_tri_warp<<<grid_for(n, 8 * run, 6 * sms), 256, 0, st>>>(ooff, oadj, n, run, tri, sup, ds);
     LF_LAUNCHED();
     k_tri_mid<<<sms * 8, TRI_MID_THREADS, TRI_MID_SMEM, st>>>(ooff, oadj, hubs, nh, tri, sup, ds);
     LF_LAUNCHED();
     k_tri_block<<<2 * sms, TRI_BLOCK_THREADS, TRI_BIG_SMEM, st>>>(ooff, oadj, hubs + n, nh + 1, tri, sup, ds);
     LF_LAUNCHED();
-    return 4;
+    return 5;
 }
 
 
@@ -778,16 +907,18 @@ __device__ __forceinline__ int tv_compact(const int32_t *adj, const int32_t *deg
 }
 
 // One warp per node v with 1 <= d+(v) <= TV_WARP_DPLUS and deg(v) <= TV_WARP_DEG.
-// A resident grid; each warp takes runs of TV_WARP_BATCH node ids from a
-// counter, so that a block is not held by one long node while its other warps
-// idle.
+// A resident grid; each warp takes runs of `batch` node ids from a counter, so
+// that a block is not held by one long node while its other warps idle.  The
+// batch is the largest that still gives every warp about four runs, at most
+// TV_WARP_BATCH: with 64 ids a run always, graphs below 400k nodes left most
+// warps without one (61k nodes: 609 -> 131 us).
 constexpr int TV_WARP_BATCH = 64;
 
 template <typename Idx>
 __global__ void __launch_bounds__(256, 5) k_tv_warp(const int64_t *off, const int32_t *adj, const int32_t *deg,
                                                     const int64_t *ooff, const int32_t *__restrict__ oadj,
-                                                    int64_t n, uint32_t *next, unsigned long long *tri, uint8_t *sup,
-                                                    DevScalars *ds) {
+                                                    int64_t n, int batch, uint32_t *next, unsigned long long *tri,
+                                                    uint8_t *sup, DevScalars *ds) {
     __shared__ Idx s_shift[8][TV_ROUND];
     __shared__ int32_t s_ul[8][TV_ROUND];
     __shared__ int32_t s_pre[8][TV_ROUND + 1];
@@ -809,11 +940,11 @@ __global__ void __launch_bounds__(256, 5) k_tv_warp(const int64_t *off, const in
     for (;;) {
         if (vv == vend) {
             unsigned long long b0 = 0;
-            if (lane == 0) b0 = (unsigned long long)atomicAdd(next, 1u) * TV_WARP_BATCH;
+            if (lane == 0) b0 = (unsigned long long)atomicAdd(next, 1u) * (unsigned)batch;
             b0 = __shfl_sync(FULL, b0, 0);
             if ((int64_t)b0 >= n) break;
             vv = (int64_t)b0;
-            vend = min(n, vv + TV_WARP_BATCH);
+            vend = min(n, vv + batch);
         }
         const int32_t v = (int32_t)(vv++);
         const int64_t vs = ooff[v];
@@ -1121,7 +1252,9 @@ int launch_tv(const int64_t *off, const int32_t *adj, const int32_t *deg, const 
     k_tv_items<true, Idx><<<sms * 2, TV_THREADS, bs, st>>>(off, adj, deg, ooff, oadj, items + cap, cnt + 1, cnt + 3,
                                                            tri, sup, ds);
     LF_LAUNCHED();
-    k_tv_warp<Idx><<<sms * std::max(1, per_sm), 256, 0, st>>>(off, adj, deg, ooff, oadj, n, cnt + 4, tri, sup, ds);
+    const int64_t grid = sms * std::max(1, per_sm);
+    const int batch = (int)std::min<int64_t>(TV_WARP_BATCH, std::max<int64_t>(1, n / (4 * 8 * grid)));
+    k_tv_warp<Idx><<<(unsigned)grid, 256, 0, st>>>(off, adj, deg, ooff, oadj, n, batch, cnt + 4, tri, sup, ds);
     LF_LAUNCHED();
     return 4;
 }
@@ -1131,29 +1264,44 @@ int launch_tv(const int64_t *off, const int32_t *adj, const int32_t *deg, const 
 int64_t tv_item_cap(int64_t m) { return 2 * m / (TV_WARP_DPLUS + 1) + 2 * m / TV_ITEM + 2; }
 
 // ---- a4 --------------------------------------------------------------------
-__global__ void k_vt(const int64_t *ooff, const int32_t *oadj, const uint8_t *sup, int64_t n, int32_t *vt,
-                     DevScalars *ds) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+// vt: groups of eight lanes take a node each (mean out-degrees are small), on a
+// resident grid.  The merge-stream byte count leaves a block as one atomic:
+// one per node's warp queued hundreds of thousands of atomics on one address,
+// which was nearly all of the kernel's time (335k nodes: 231 -> 23 us).
+__global__ void __launch_bounds__(256) k_vt(const int64_t *ooff, const int32_t *oadj, const uint8_t *sup, int64_t n,
+                                            int32_t *vt, DevScalars *ds) {
+    __shared__ unsigned long long s_mb[8];
+    const int sub = threadIdx.x & 7, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> 3;
+    const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     unsigned long long mb = 0;
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
-        const int64_t s = ooff[u], e = ooff[u + 1];
-        const int64_t du = e - s;
+    for (int64_t b = 0; b < n; b += groups) {   // the whole warp stays together for the shuffles
+        const int64_t u = b + g0;
         int cnt = 0;
-        for (int64_t p = s + lane; p < e; p += 32) {
-            int32_t v = oadj[p];
-            mb += 4ull * (unsigned long long)(du + (ooff[v + 1] - ooff[v]));
-            if (sup[p]) {
-                ++cnt;
-                atomicAdd(&vt[v], 1);
+        if (u < n) {
+            const int64_t s = ooff[u], e = ooff[u + 1];
+            const int64_t du = e - s;
+            for (int64_t p = s + sub; p < e; p += 8) {
+                const int32_t v = oadj[p];
+                mb += 4ull * (unsigned long long)(du + (ooff[v + 1] - ooff[v]));
+                if (sup[p]) {
+                    ++cnt;
+                    atomicAdd(&vt[v], 1);
+                }
             }
         }
-        cnt = __reduce_add_sync(FULL, cnt);
-        if (lane == 0 && cnt) atomicAdd(&vt[u], cnt);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
+        if (sub == 0 && cnt) atomicAdd(&vt[u], cnt);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mb += __shfl_down_sync(FULL, mb, o);
-    if (lane == 0 && mb) atomicAdd(&ds->merge_bytes, mb);
+    if (lane == 0) s_mb[w] = mb;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) mb += s_mb[k];
+        if (mb) atomicAdd(&ds->merge_bytes, mb);
+    }
 }
 
 // ---- a5 --------------------------------------------------------------------
@@ -1459,7 +1607,14 @@ void build_graph(lf_graph *g, const int32_t *src, const int32_t *dst, int64_t E,
     LF_CUDA(cudaMemsetAsync(g->vt, 0, (size_t)(n > 0 ? n : 1) * 4, st));
     LF_CUDA(cudaMemsetAsync(sup, 0, (size_t)(m > 0 ? m : 1), st));
     unsigned long long *utri = reinterpret_cast<unsigned long long *>(g->tri);
-    if (n > 0) {
+    if (n > 0 && m <= FLAT_MAX_MEAN * n) {
+        int32_t *hubs = dalloc_n<int32_t>(g, n);
+        uint32_t *nh = reinterpret_cast<uint32_t *>(tmp64);
+        LF_CUDA(cudaMemsetAsync(nh, 0, 2 * sizeof(uint32_t), st));
+        set_triangle_attrs();
+        g->launches += launch_triangles(g->ooff, g->oadj, n, hubs, nh, utri, sup, ds, st);
+        dfree(g, hubs);
+    } else if (n > 0) {
         const int64_t cap = tv_item_cap(m);
         unsigned long long *items = dalloc_n<unsigned long long>(g, cap);
         // [0..1] item counts, [2..3] item counters, [4] node-run counter
@@ -1475,7 +1630,7 @@ void build_graph(lf_graph *g, const int32_t *src, const int32_t *dst, int64_t E,
     }
     pt.mark();   // 3
     if (n > 0) {
-        k_vt<<<grid_for(n * 32, 256, 1 << 16), 256, 0, st>>>(g->ooff, g->oadj, sup, n, g->vt, ds); ++g->launches;
+        k_vt<<<grid_for(n * 8, 256, 8 * sm_count()), 256, 0, st>>>(g->ooff, g->oadj, sup, n, g->vt, ds); ++g->launches;
         LF_LAUNCHED();
     }
     dfree(g, sup);
@@ -1664,7 +1819,7 @@ void triangles_noalloc(const int64_t *ooff, const int32_t *oadj, int64_t n, int6
     LF_CUDA(cudaMemsetAsync(vt, 0, (size_t)n * sizeof(int32_t), st));
     unsigned long long *utri = reinterpret_cast<unsigned long long *>(t);
     launch_triangles(ooff, oadj, n, hubs, nh, utri, sup, ds, st);
-    k_vt<<<grid_for(n * 32, 256, 1 << 16), 256, 0, st>>>(ooff, oadj, sup, n, vt, ds);
+    k_vt<<<grid_for(n * 8, 256, 8 * sm_count()), 256, 0, st>>>(ooff, oadj, sup, n, vt, ds);
     LF_LAUNCHED();
 }
 
