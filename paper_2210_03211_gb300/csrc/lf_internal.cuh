@@ -319,17 +319,22 @@ __device__ __forceinline__ double binom2(double z) {
 //   E[t(x,C)] / E[t(x,V)] * d / (|C \ {x}| + deg(x, V \ C)),
 //   E[t(x,C)] = C(k,2) p, p = m2 / (n (n-1)),  E[t(x,V)] = C(d,2) cc.
 // (Heuristic Counting of Triangles; zero when n < 2 or E[t(x,V)] = 0.)
-__device__ __forceinline__ double wcchat_member(int64_t k, int64_t d, int64_t n, uint32_t m2,
-                                                double cc) {
+// wcchat_term takes p, which members of one community share.
+__device__ __forceinline__ double wcchat_term(int64_t k, int64_t d, int64_t n, double p, double cc) {
     if (n < 2) return 0.0;
     double nd = (double)n;
-    double p = __ddiv_rn((double)m2, __dmul_rn(nd, __dsub_rn(nd, 1.0)));
     double ec = __dmul_rn(binom2((double)k), p);
     double ev = __dmul_rn(binom2((double)d), cc);
     if (!(ev > 0.0)) return 0.0;
     double dd = (double)d;
     return __dmul_rn(__ddiv_rn(ec, ev),
                      __ddiv_rn(dd, __dadd_rn(__dsub_rn(nd, 1.0), __dsub_rn(dd, (double)k))));
+}
+
+__device__ __forceinline__ double wcchat_member(int64_t k, int64_t d, int64_t n, uint32_t m2, double cc) {
+    if (n < 2) return 0.0;
+    const double nd = (double)n;
+    return wcchat_term(k, d, n, __ddiv_rn((double)m2, __dmul_rn(nd, __dsub_rn(nd, 1.0))), cc);
 }
 
 // Mean-field community score: every member given the mean internal degree

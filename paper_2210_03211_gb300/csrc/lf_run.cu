@@ -1848,65 +1848,93 @@ __device__ __forceinline__ void ssacc_add(unsigned long long *acc, double v) {
         if (d[t]) atomicAdd(&acc[c + t], neg ? (unsigned long long)(-(long long)d[t]) : d[t]);
 }
 
-// The double nearest (ties to even) to the non-negative value held in 32-bit
-// digits dg (bit 0 = 2^-1074).
-__device__ inline double round_digits(const uint32_t *dg) {
-    int top = -1;
-    for (int i = SACC_CHUNKS - 1; i >= 0; --i)
-        if (dg[i]) {
-            top = i;
-            break;
-        }
-    if (top < 0) return 0.0;
-    int P = 32 * top + (31 - __clz((int)dg[top]));
-    auto bit = [&](int q) -> unsigned long long {
-        return q < 0 ? 0ull : (unsigned long long)((dg[q >> 5] >> (q & 31)) & 1u);
-    };
-    if (P <= 52) {
-        unsigned long long v = 0;
-        for (int q = P; q >= 0; --q) v = (v << 1) | bit(q);
-        return __longlong_as_double((long long)v);
+// A warp's values v >= 0 (zero for lanes without one) added to (or, with neg,
+// subtracted from) its own accumulator: the words from the lowest to the
+// highest digit any lane has are summed over the lanes by integer reductions of
+// their 16-bit halves, then added by one lane.  32 lanes adding their digits
+// with 64-bit shared atomics queue up on the same two or three words.
+__device__ __forceinline__ void ssacc_add_warp(unsigned long long *acc, double v, bool neg) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    const unsigned long long mant = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    const int p = e ? (int)e - 1 : 0;
+    const int c = p >> 5, sh = p & 31;
+    const unsigned long long lo = mant << sh;
+    const uint32_t d0 = (uint32_t)lo, d1 = (uint32_t)(lo >> 32), d2 = sh ? (uint32_t)(mant >> (64 - sh)) : 0u;
+    const int c0 = __reduce_min_sync(FULL, b ? c : SACC_CHUNKS);
+    const int c1 = __reduce_max_sync(FULL, b ? c : -1);
+    for (int t = c0; t <= c1 + 2 && t < SACC_CHUNKS; ++t) {   // none if no lane has a value
+        const uint32_t dg = b == 0ull ? 0u : t == c ? d0 : t == c + 1 ? d1 : t == c + 2 ? d2 : 0u;
+        const unsigned l16 = __reduce_add_sync(FULL, dg & 0xffffu), h16 = __reduce_add_sync(FULL, dg >> 16);
+        const unsigned long long sum = (unsigned long long)l16 + ((unsigned long long)h16 << 16);
+        if ((threadIdx.x & 31) == 0) acc[t] += neg ? (unsigned long long)(-(long long)sum) : sum;
     }
-    unsigned long long mant = 0;
-    for (int q = P; q >= P - 52; --q) mant = (mant << 1) | bit(q);
-    const int r = P - 53;
-    const bool round_bit = bit(r) != 0;
-    bool sticky = false;
-    for (int i = 0; i < (r >> 5) && !sticky; ++i) sticky = dg[i] != 0u;
-    if (!sticky && (r & 31)) sticky = (dg[r >> 5] & ((1u << (r & 31)) - 1u)) != 0u;
-    if (round_bit && (sticky || (mant & 1ull))) ++mant;
-    if (mant == (1ull << 53)) {
-        mant >>= 1;
-        ++P;
-    }
-    const long long biased = (long long)P - 51;
-    if (biased >= 2047) return __longlong_as_double(0x7ff0000000000000ll);
-    return __longlong_as_double((long long)(((unsigned long long)biased << 52) | (mant & 0xfffffffffffffull)));
+    __syncwarp();
 }
 
-// Round the signed accumulated value to the nearest double and clear the
-// accumulator.  One thread.
-__device__ inline double ssacc_round_and_clear(unsigned long long *acc) {
-    uint32_t dg[SACC_CHUNKS];
-    long long carry = 0;
-    for (int i = 0; i < SACC_CHUNKS; ++i) {
-        const long long v = (long long)acc[i] + carry;
-        acc[i] = 0ull;
-        const uint32_t low = (uint32_t)(unsigned long long)v;
-        dg[i] = low;
-        carry = (v - (long long)low) / 4294967296ll;   // exact: v - low is a multiple of 2^32
-    }
-    const bool neg = carry < 0;   // the value is (digits) - 2^(32 * SACC_CHUNKS)
-    if (neg) {
-        unsigned long long c = 1;
-        for (int i = 0; i < SACC_CHUNKS; ++i) {
-            const unsigned long long t = (unsigned long long)(uint32_t)~dg[i] + c;
-            dg[i] = (uint32_t)t;
-            c = t >> 32;
+// The accumulated signed value rounded to the nearest double (ties to even),
+// and the accumulator cleared: one warp, the result on every lane.  Only the
+// words between the lowest and the highest non-zero one are walked (the terms
+// of a gain reach over a handful), in place.
+__device__ __noinline__ double ssacc_round_warp(unsigned long long *acc) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const unsigned m0 = __ballot_sync(FULL, acc[lane] != 0ull), m1 = __ballot_sync(FULL, acc[lane + 32] != 0ull);
+    const unsigned m2 = __ballot_sync(FULL, lane + 64 < SACC_CHUNKS && acc[min(lane + 64, SACC_CHUNKS - 1)] != 0ull);
+    if (!(m0 | m1 | m2)) return 0.0;
+    const int first = m0 ? __ffs(m0) - 1 : m1 ? 31 + __ffs(m1) : 63 + __ffs(m2);
+    const int last0 = m2 ? 95 - __clz(m2) : m1 ? 63 - __clz(m1) : 31 - __clz(m0);
+    double r = 0.0;
+    if (lane == 0) {
+        const int last = min(last0 + 1, SACC_CHUNKS - 1);   // the carry out of the top word
+        long long carry = 0;
+        for (int i = first; i <= last; ++i) {
+            const long long v = (long long)acc[i] + carry;
+            acc[i] = (unsigned long long)(uint32_t)v;
+            carry = v >> 32;   // rounds down: the digit just stored is v mod 2^32
         }
+        const bool neg = carry < 0;   // the value is (digits) - 2^(32 (last + 1))
+        int top = -1;
+        uint32_t c = 1;
+        for (int i = first; i <= last; ++i) {
+            uint32_t d = (uint32_t)acc[i];
+            if (neg) {
+                const unsigned long long t = (unsigned long long)(uint32_t)~d + c;
+                d = (uint32_t)t;
+                c = (uint32_t)(t >> 32);
+                acc[i] = d;
+            }
+            if (d) top = i;
+        }
+        if (top >= 0) {
+            const uint32_t a2 = (uint32_t)acc[top], a1 = top >= 1 ? (uint32_t)acc[top - 1] : 0u,
+                           a0 = top >= 2 ? (uint32_t)acc[top - 2] : 0u;
+            const int z = __clz((int)a2), P = 32 * top + 31 - z;   // P: index of the leading bit
+            const unsigned long long h = ((unsigned long long)a2 << 32) | a1;
+            unsigned long long bits;
+            if (P <= 52) {   // fewer than 54 significant bits: exact
+                bits = top == 1 ? h : (unsigned long long)a2;
+            } else {
+                const unsigned long long w = z ? (h << z) | (a0 >> (32 - z)) : h;   // the leading 64 bits
+                bool sticky = (w & 0x3ffull) != 0ull || (z ? (a0 << z) != 0u : a0 != 0u);
+                for (int i = first; i < top - 2 && !sticky; ++i) sticky = acc[i] != 0ull;
+                unsigned long long mant = w >> 11;
+                long long biased = (long long)P - 51;
+                if (((w >> 10) & 1ull) && (sticky || (mant & 1ull))) ++mant;
+                if (mant == (1ull << 53)) {
+                    mant >>= 1;
+                    ++biased;
+                }
+                bits = biased >= 2047 ? 0x7ff0000000000000ull
+                                      : ((unsigned long long)biased << 52) | (mant & 0xfffffffffffffull);
+            }
+            r = __longlong_as_double((long long)bits);
+            if (neg) r = -r;
+        }
+        for (int i = first; i <= last; ++i) acc[i] = 0ull;
     }
-    const double r = round_digits(dg);
-    return neg ? -r : r;
+    __syncwarp();
+    return __shfl_sync(FULL, r, 0);
 }
 
 // Bounds-checked mode (lf_options.debug_checks): a value read from device
@@ -1931,6 +1959,55 @@ __device__ __forceinline__ int row_find(const int32_t *row, int32_t cnt, int32_t
     return -1;
 }
 
+// The first eight ids of node y's membership row (rows start on 16-byte
+// boundaries; K is 4 or a multiple of 8): loads that do not wait for the row's
+// count, so that count, ids and whatever else of y is wanted arrive together.
+struct RowHead {
+    int4 a, b;
+};
+
+__device__ __forceinline__ RowHead row_head8(const int32_t *rows, int64_t y, int32_t K) {
+    const int4 *p = reinterpret_cast<const int4 *>(rows + y * K);
+    RowHead h;
+    h.a = __ldcg(p);
+    h.b = K >= 8 ? __ldcg(p + 1) : make_int4(0, 0, 0, 0);
+    return h;
+}
+
+// Position of C in y's row of cnt ids, -1 if absent: the head's ids are
+// compared directly, only longer rows are searched.
+__device__ __forceinline__ int head_find(const RowHead &h, const int32_t *row, int32_t cnt, int32_t C) {
+    int s = -1;
+    s = cnt > 0 && h.a.x == C ? 0 : s;
+    s = cnt > 1 && h.a.y == C ? 1 : s;
+    s = cnt > 2 && h.a.z == C ? 2 : s;
+    s = cnt > 3 && h.a.w == C ? 3 : s;
+    s = cnt > 4 && h.b.x == C ? 4 : s;
+    s = cnt > 5 && h.b.y == C ? 5 : s;
+    s = cnt > 6 && h.b.z == C ? 6 : s;
+    s = cnt > 7 && h.b.w == C ? 7 : s;
+    if (s < 0 && cnt > 8) {
+        s = row_find(row + 8, cnt - 8, C);
+        if (s >= 0) s += 8;
+    }
+    return s;
+}
+
+// Entry s of a row whose head is h.
+__device__ __forceinline__ int32_t head_entry(const RowHead &h, const int32_t *row, int s) {
+    switch (s) {
+    case 0: return h.a.x;
+    case 1: return h.a.y;
+    case 2: return h.a.z;
+    case 3: return h.a.w;
+    case 4: return h.b.x;
+    case 5: return h.b.y;
+    case 6: return h.b.z;
+    case 7: return h.b.w;
+    }
+    return __ldcg(&row[s]);
+}
+
 // y in the ascending adjacency list adj[beg, end)?
 __device__ __forceinline__ bool adj_has(const int32_t *adj, int64_t beg, int64_t end, int32_t y) {
     int64_t lo = beg, hi = end - 1;
@@ -1944,18 +2021,9 @@ __device__ __forceinline__ bool adj_has(const int32_t *adj, int64_t beg, int64_t
     return false;
 }
 
-// g_y(nu) = C(k,2) d / (C(d,2) (nu - 1 + d - k)): a member's estimator
-// without the factor (2m / (nu (nu - 1))) / cc.  Zero where the estimator is
-// (k < 2, or d < 2 so that E[t(x,V)] = 0).
-__device__ __forceinline__ double lit_g(int64_t k, int64_t d, int64_t nu) {
-    if (k < 2 || d < 2) return 0.0;
-    const int64_t den = nu - 1 + d - k;
-    if (den <= 0) return 0.0;
-    const double bk = 0.5 * ((double)k * (double)(k - 1));
-    const double bd = 0.5 * ((double)d * (double)(d - 1));
-    return (bk * (double)d) / (bd * (double)den);
-}
-
+// With g_y(nu) = C(k,2) d / (C(d,2) (nu - 1 + d - k)) a member's estimator
+// without the factor (2m / (nu (nu - 1))) / cc, zero where the estimator is
+// (k < 2, or d < 2 so that E[t(x,V)] = 0):
 // The neighbours' corrections:
 //   h+ = g(n+1; k+1) - g(n+1; k) = d (k D + C(k,2)) / (C(d,2) D (D-1)), D = n + d - k
 //        (a neighbour y of a joining x; y is not x, so k <= d - 1 and D - 1 >= n >= 1),
@@ -2021,6 +2089,15 @@ __device__ __forceinline__ void lit_screen(const RunArgs &a, int32_t C, uint32_t
     if (!isfinite(X) || !isfinite(E)) {   // out of float range: only the exact sum can decide
         X = 0.f;
         E = INFINITY;
+    }
+    // Every term after the move is exactly zero (no density left, or no member
+    // with two neighbours inside: sums of non-negative floats far above
+    // underflow, so the sum is zero only if each term is): the gain is at most
+    // zero and cannot be chosen.  Without this every such candidate of a node
+    // that gains nothing passed the bracket and was summed exactly.
+    if (A == 0.f || (own ? f.x : Sm) == 0.f) {
+        X = -f.z;
+        E = 0.f;
     }
 }
 
@@ -2127,29 +2204,50 @@ __device__ double lit_exact_gain(const RunArgs &a, int32_t x, int32_t d, int32_t
     const int64_t n1 = own ? n0 - 1 : n0 + 1;
     const uint32_t m21 = own ? m20 - (uint32_t)(2 * k) : m20 + (uint32_t)(2 * k);
     const int64_t xb = a.off[x], xe = a.off[x + 1];
-    auto member = [&](int32_t y) {
+    // the densities of wcchat_member, the same for every member
+    const double nd0 = (double)n0, nd1 = (double)n1;
+    const double p0 = __ddiv_rn((double)m20, __dmul_rn(nd0, __dsub_rn(nd0, 1.0)));
+    const double p1 = __ddiv_rn((double)m21, __dmul_rn(nd1, __dsub_rn(nd1, 1.0)));
+    auto member = [&](int32_t y, double &after, double &before) {
         if (y == x) return;
         if (!dbg_ok(a, y >= 0 && y < a.nnodes)) return;
+        const RowHead ids = row_head8(a.mem, y, a.K), ks = row_head8(a.kmem, y, a.K);
         const int32_t cy = __ldcg(&a.nmem[y]);
-        if (!dbg_ok(a, cy >= 0 && cy <= a.K)) return;
-        const int s = row_find(a.mem + (int64_t)y * a.K, cy, C);
-        if (s < 0) return;   // left C earlier in this iteration
-        const int64_t ky = __ldcg(&a.kmem[(int64_t)y * a.K + s]);
         const int64_t dy = a.deg[y];
+        const bool near = adj_has_fenced(a.adj, xb, xe, fence, nf, step, y);
+        if (!dbg_ok(a, cy >= 0 && cy <= a.K)) return;
+        const int s = head_find(ids, a.mem + (int64_t)y * a.K, cy, C);
+        if (s < 0) return;   // left C earlier in this iteration
+        const int64_t ky = head_entry(ks, a.kmem + (int64_t)y * a.K, s);
         if (!dbg_ok(a, ky >= 0 && ky <= dy)) return;
-        const int64_t k1 = adj_has_fenced(a.adj, xb, xe, fence, nf, step, y) ? (own ? ky - 1 : ky + 1) : ky;
-        ssacc_add(wacc, wcchat_member(k1, dy, n1, m21, cc));
-        ssacc_add(wacc, -wcchat_member(ky, dy, n0, m20, cc));
+        const int64_t k1 = near ? (own ? ky - 1 : ky + 1) : ky;
+        after = wcchat_term(k1, dy, n1, p1, cc);
+        before = wcchat_term(ky, dy, n0, p0, cc);
     };
-    lit_members(a, C, tid, nthreads, member);
-    if (tid == 0) ssacc_add(wacc, own ? -wcchat_member(k, d, n0, m20, cc) : wcchat_member(k, d, n1, m21, cc));
-    if (!block) {
-        __syncwarp();
-        double g = 0.0;
-        if (lane == 0) g = ssacc_round_and_clear(acc);
-        __syncwarp();
-        return __shfl_sync(FULL, g, 0);
+    {
+        const int64_t b0 = (int64_t)a.cm_off[C], cap = (int64_t)a.cm_off[C + 1] - b0;
+        const int64_t used = (int64_t)__ldcg(&a.cm_cnt[C]);
+        const int64_t b1 = b0 + (used < cap ? used : cap);
+        for (int64_t q0 = b0 + (tid - lane); q0 < b1; q0 += nthreads) {   // a warp's lanes stay together
+            double after = 0.0, before = 0.0;
+            if (q0 + lane < b1) member(__ldcg(&a.cm_node[q0 + lane]), after, before);
+            __syncwarp();
+            ssacc_add_warp(wacc, after, false);
+            ssacc_add_warp(wacc, before, true);
+        }
+        if (used > cap) {   // joiners beyond the region
+            int idx = 0;
+            for (int32_t e = __ldcg(&a.jl_head[C]); e >= 0; e = __ldcg(&a.jl_next[e]), ++idx)
+                if (idx % nthreads == tid) {
+                    double after = 0.0, before = 0.0;
+                    member(__ldcg(&a.jl_node[e]), after, before);
+                    ssacc_add(wacc, after);
+                    ssacc_add(wacc, -before);
+                }
+        }
     }
+    if (tid == 0) ssacc_add(wacc, own ? -wcchat_term(k, d, n0, p0, cc) : wcchat_term(k, d, n1, p1, cc));
+    if (!block) return ssacc_round_warp(acc);
     __syncthreads();
     const int nw = (int)(blockDim.x >> 5);
     for (int c = threadIdx.x; c < SACC_CHUNKS; c += blockDim.x) {
@@ -2161,7 +2259,10 @@ __device__ double lit_exact_gain(const RunArgs &a, int32_t x, int32_t d, int32_t
         acc[c] = t;
     }
     __syncthreads();
-    if (threadIdx.x == 0) *s_g = ssacc_round_and_clear(acc);
+    if (threadIdx.x < 32) {
+        const double g = ssacc_round_warp(acc);
+        if (threadIdx.x == 0) *s_g = g;
+    }
     __syncthreads();
     const double g = *s_g;
     __syncthreads();
@@ -3036,97 +3137,154 @@ __global__ void __launch_bounds__(AP_THREADS) k_lit_kupd(RunArgs a, int64_t bsta
 }
 
 // F(n-1), F(n), F(n+1) of communities: list[0 .. *count) (or every id below
-// ncount when list is null).  Blocks take eight entries at a time: each warp
-// sums a community of up to LIT_FSUM_WARP members alone, larger ones are then
-// summed by the whole block, one after the other.
+// ncount when list is null).  Bound by latency for short queues and by the FP64
+// pipe for long ones (ncu, 16,384-node queue of the 767k-node graph: FP64 48% busy
+// with 17 of 32 lanes on, 84 us).  So a group of eight lanes takes a
+// community (they mostly have 5-50 members; a warp each left most lanes of the
+// FP64 pipe empty), whole warps take the ones of more than LIT_FSUM_GROUP
+// members, and the block those above LIT_FSUM_WARP; a member's count, ids,
+// deg(y,C) and degree load together, not one after another; its three terms
+// share one division; and the stored factors are formed by three lanes at once.
+// Mean over the queues: 767k nodes, q 16,384: 112 -> 59 us; 3.07M nodes, q 65,536:
+// 460 -> 111 us; 335k nodes, q 1,024: 23 -> 20 us (cold caches).
+constexpr int LIT_FSUM_GROUP = 64;
 constexpr int LIT_FSUM_WARP = 512;
 
-__device__ __forceinline__ void lit_fsum_member(const RunArgs &a, int32_t C, int64_t n, int32_t y, double &f0,
+// g_y(n-1), g_y(n), g_y(n+1) added to f0, f1, f2: with D = n - 1 + d - k they are
+// k (k-1) / (d-1) over D-1, D and D+1, so one quotient q = k (k-1) / ((d-1) (D-1) D
+// (D+1)) times D (D+1), (D-1) (D+1) and (D-1) D.  FP64 as before (eight roundings a
+// term against six, 2^-53 each, under a sum kept as a float); members have
+// k <= n-1, hence D >= d >= 2.
+__device__ __forceinline__ void lit_g3(int32_t k, int32_t d, int32_t n, double &f0, double &f1, double &f2) {
+    if (k < 2 || d < 2 || (int64_t)n - 1 + d - k < 2) return;
+    const double D = __uint2double_rn((uint32_t)(n - 1) + (uint32_t)(d - k));
+    const double kd = __int2double_rn(k), dm = __int2double_rn(d - 1);
+    const double lo = D - 1.0, hi = D + 1.0;
+    const double lh = lo * hi;
+    const double q = (kd * (kd - 1.0)) / ((dm * D) * lh);
+    f0 = fma(q, D * hi, f0);
+    f1 = fma(q, lh, f1);
+    f2 = fma(q, lo * D, f2);
+}
+
+__device__ __forceinline__ void lit_fsum_member(const RunArgs &a, int32_t C, int32_t n, int32_t y, double &f0,
                                                 double &f1, double &f2) {
     if (!dbg_ok(a, y >= 0 && y < a.nnodes)) return;
+    const RowHead ids = row_head8(a.mem, y, a.K), ks = row_head8(a.kmem, y, a.K);
     const int32_t cy = __ldcg(&a.nmem[y]);
+    const int32_t dy = a.deg[y];
     if (!dbg_ok(a, cy >= 0 && cy <= a.K)) return;
-    const int s = row_find(a.mem + (int64_t)y * a.K, cy, C);
+    const int s = head_find(ids, a.mem + (int64_t)y * a.K, cy, C);
     if (s < 0) return;   // left C earlier in this iteration
-    const int64_t ky = __ldcg(&a.kmem[(int64_t)y * a.K + s]);
-    const int64_t dy = a.deg[y];
+    const int32_t ky = head_entry(ks, a.kmem + (int64_t)y * a.K, s);
     if (!dbg_ok(a, ky >= 0 && ky <= dy)) return;
-    f0 += lit_g(ky, dy, n - 1);
-    f1 += lit_g(ky, dy, n);
-    f2 += lit_g(ky, dy, n + 1);
+    lit_g3(ky, dy, n, f0, f1, f2);
 }
 
 // The per-community values of the bracket from the member sums (rounded
-// to float; the bound E allows for it).
-__device__ __forceinline__ void lit_fsum_store(const RunArgs &a, int32_t C, double f0, double f1, double f2) {
+// to float; the bound E allows for it).  Lane t of the first three of a group
+// (all of which hold the sums) forms the t-th factor.
+__device__ __forceinline__ void lit_fsum_store(const RunArgs &a, int32_t C, int t, double f0, double f1, double f2) {
+    if (t > 2) return;
     const int4 r = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C]));
-    const int64_t n = r.x;
-    const double m2 = (double)(uint32_t)r.y;
+    const int32_t n = r.x;
     const double cc = a.gcc ? a.gcc[r.w] : a.cc;
-    const bool on = cc > 0.0 && n >= 1;
+    const double nd = __int2double_rn(n);
+    const bool on = cc > 0.0 && (t == 0 ? n >= 2 : t == 1 ? n >= 1 : n >= 3);
+    // t = 0: n (n-1), 1: (n+1) n, 2: (n-1)(n-2)
+    const double den = (t == 1 ? nd + 1.0 : nd - 1.0) * (t == 2 ? nd - 2.0 : nd);
+    double v = on ? (t == 0 ? __uint2double_rn((uint32_t)r.y) : 1.0) / (den * cc) : 0.0;
     float *f = a.litF + 8 * (int64_t)C;
-    f[0] = (float)f0;
-    f[1] = (float)f2;
-    f[2] = on && n >= 2 ? (float)(((m2 / ((double)n * (double)(n - 1))) / cc) * f1) : 0.f;
-    f[3] = on ? (float)((1.0 / ((double)(n + 1) * (double)n)) / cc) : 0.f;
-    f[4] = on && n - 1 >= 2 ? (float)((1.0 / ((double)(n - 1) * (double)(n - 2))) / cc) : 0.f;
+    if (t == 0) {
+        f[0] = (float)f0;
+        f[1] = (float)f2;
+        v *= f1;
+    }
+    f[2 + t] = (float)v;
 }
 
-__global__ void __launch_bounds__(256) k_lit_fsum(RunArgs a, const int32_t *list, const uint32_t *count,
-                                                  int64_t ncount) {
-    __shared__ double red[3][8];
-    __shared__ int32_t big[8];
-    __shared__ int nbig;
-    const int64_t total = list ? (int64_t)__ldcg(count) : ncount;
+__device__ __forceinline__ void lit_fsum_reduce(double &f0, double &f1, double &f2, int width) {
+    for (int o = width >> 1; o > 0; o >>= 1) {
+        f0 += __shfl_xor_sync(FULL, f0, o);
+        f1 += __shfl_xor_sync(FULL, f1, o);
+        f2 += __shfl_xor_sync(FULL, f2, o);
+    }
+}
+
+struct FsumShared {
+    double red[3][EV_WARPS];
+    int32_t big[4 * EV_WARPS];
+    int nbig;
+};
+
+// Entries t0 .. t0 + 4 x warps - 1 of the list, by one block of EV_WARPS warps.
+__device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0, int64_t total, FsumShared &fs) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int64_t t0 = (int64_t)blockIdx.x * 8; t0 < total; t0 += (int64_t)gridDim.x * 8) {
-        if (threadIdx.x == 0) nbig = 0;
-        __syncthreads();
-        const int64_t t = t0 + w;
-        if (t < total) {
-            const int32_t C = list ? __ldcg(&list[t]) : (int32_t)t;
-            const int64_t n = __ldcg(&a.comm[C].n);
-            if (n > LIT_FSUM_WARP) {
-                if (lane == 0) big[atomicAdd(&nbig, 1)] = C;
-            } else {
-                double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-                if (n > 0)
-                    lit_members(a, C, lane, 32, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    f0 += __shfl_xor_sync(FULL, f0, o);
-                    f1 += __shfl_xor_sync(FULL, f1, o);
-                    f2 += __shfl_xor_sync(FULL, f2, o);
-                }
-                if (lane == 0) lit_fsum_store(a, C, f0, f1, f2);
-            }
+    const int sub = lane & 7, grp = lane >> 3;
+    if (threadIdx.x == 0) fs.nbig = 0;
+    __syncthreads();
+    const int64_t t = t0 + 4 * w + grp;
+    int32_t C = 0, n = -1;
+    if (t < total) {
+        C = list ? __ldcg(&list[t]) : (int32_t)t;
+        n = __ldcg(&a.comm[C].n);
+    }
+    {
+        double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+        const bool mine = n >= 0 && n <= LIT_FSUM_GROUP;
+        if (mine && n > 0)
+            lit_members(a, C, sub, 8, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
+        __syncwarp();
+        lit_fsum_reduce(f0, f1, f2, 8);
+        if (mine) lit_fsum_store(a, C, sub, f0, f1, f2);
+    }
+    unsigned mid = __ballot_sync(FULL, sub == 0 && n > LIT_FSUM_GROUP);
+    while (mid) {
+        const int src = __ffs(mid) - 1;
+        mid &= mid - 1;
+        const int32_t C1 = __shfl_sync(FULL, C, src), n1 = __shfl_sync(FULL, n, src);
+        if (n1 > LIT_FSUM_WARP) {
+            if (lane == 0) fs.big[atomicAdd(&fs.nbig, 1)] = C1;
+            continue;
+        }
+        double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+        lit_members(a, C1, lane, 32, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
+        __syncwarp();
+        lit_fsum_reduce(f0, f1, f2, 32);
+        lit_fsum_store(a, C1, lane, f0, f1, f2);
+    }
+    __syncthreads();
+    const int nbig = fs.nbig;
+    for (int b = 0; b < nbig; ++b) {
+        const int32_t C1 = fs.big[b];
+        const int32_t n1 = __ldcg(&a.comm[C1].n);
+        double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+        lit_members(a, C1, threadIdx.x, blockDim.x, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
+        __syncwarp();
+        lit_fsum_reduce(f0, f1, f2, 32);
+        if (lane == 0) {
+            fs.red[0][w] = f0;
+            fs.red[1][w] = f1;
+            fs.red[2][w] = f2;
         }
         __syncthreads();
-        for (int b = 0; b < nbig; ++b) {
-            const int32_t C = big[b];
-            const int64_t n = __ldcg(&a.comm[C].n);
-            double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-            lit_members(a, C, threadIdx.x, blockDim.x, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                f0 += __shfl_xor_sync(FULL, f0, o);
-                f1 += __shfl_xor_sync(FULL, f1, o);
-                f2 += __shfl_xor_sync(FULL, f2, o);
-            }
-            if (lane == 0) {
-                red[0][w] = f0;
-                red[1][w] = f1;
-                red[2][w] = f2;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double sum[3] = {0.0, 0.0, 0.0};
-                for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2)
-                    for (int t2 = 0; t2 < 3; ++t2) sum[t2] += red[t2][k2];
-                lit_fsum_store(a, C, sum[0], sum[1], sum[2]);
-            }
-            __syncthreads();
+        if (w == 0) {
+            double sum[3] = {0.0, 0.0, 0.0};
+            for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2)
+                for (int t2 = 0; t2 < 3; ++t2) sum[t2] += fs.red[t2][k2];
+            lit_fsum_store(a, C1, lane, sum[0], sum[1], sum[2]);
         }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(EV_THREADS) k_lit_fsum(RunArgs a, const int32_t *list, const uint32_t *count,
+                                                         int64_t ncount) {
+    __shared__ FsumShared fs;
+    const int64_t total = list ? (int64_t)__ldcg(count) : ncount;
+    for (int64_t t0 = (int64_t)blockIdx.x * (4 * EV_WARPS); t0 < total; t0 += (int64_t)gridDim.x * (4 * EV_WARPS)) {
+        lit_fsum_block(a, list, t0, total, fs);
+        __syncthreads();
     }
 }
 
@@ -4367,7 +4525,7 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         const unsigned ag = grid_for((int64_t)blen * 32, AP_THREADS, 1 << 30);
         launch_pdl(k_lit_apply, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
         k_lit_kupd<<<ag, AP_THREADS, 0, g->stream>>>(ab, bstart, blen);
-        k_lit_fsum<<<(unsigned)std::min<int64_t>((2 * (int64_t)blen + 7) / 8, 8 * (int64_t)num_sms()), 256, 0,
+        k_lit_fsum<<<(unsigned)std::min<int64_t>((2 * (int64_t)blen + 31) / 32, 8 * (int64_t)num_sms()), EV_THREADS, 0,
                      g->stream>>>(ab, g->touched, ctr + 2, 0);
         g->launches += 5;
     }
@@ -4474,8 +4632,8 @@ void lit_iteration_start(lf_graph *g, const RunArgs &a) {
     // count changes between iterations, so serials of different iterations
     // may coincide): clear them
     LF_CUDA(cudaMemsetAsync(g->tstamp, 0, (size_t)n * 4, st));
-    k_lit_fsum<<<(unsigned)std::min<int64_t>((nc + 7) / 8, 16 * (int64_t)num_sms()), 256, 0, st>>>(a, nullptr, nullptr,
-                                                                                                   nc);
+    k_lit_fsum<<<(unsigned)std::min<int64_t>((nc + 31) / 32, 16 * (int64_t)num_sms()), EV_THREADS, 0, st>>>(
+        a, nullptr, nullptr, nc);
     g->launches += 4;
     LF_LAUNCHED();
 }
