@@ -231,7 +231,7 @@ struct lf_graph {
     // membership, the member index of the current iteration (members at its
     // start, by community; its joiners as per-community lists), per-community
     // sums F(n-1), F(n), F(n+1), per-queue counters (overflow count, overflow
-    // next, touched count), the overflow list, the touched list and stamps
+    // next, touched count, apply items), the overflow list, the touched list and stamps
     int32_t *kmem = nullptr;              // n*K
     unsigned long long *cm_off = nullptr; // n+1
     unsigned long long *cm_cur = nullptr; // n+1
@@ -242,7 +242,9 @@ struct lf_graph {
     uint32_t *lit_misc = nullptr;         // [0]: joiners listed in this iteration
     float *litF = nullptr;                // 8n: F(n-1), F(n+1), WCC-hat(C), 1/((n+1)n cc), 1/((n-1)(n-2) cc)
     uint32_t *tstamp = nullptr;           // n
-    uint32_t *lit_ctr = nullptr;          // 3 per queue
+    uint32_t *lit_ctr = nullptr;          // 4 per queue
+    unsigned long long *lit_items = nullptr;   // movers of a queue, in pieces
+    int32_t *lit_apacc = nullptr;         // 4 qcap, zero between queues
     int64_t lit_ctr_cap = 0;
     int32_t *lit_over = nullptr;          // qcap
     int32_t *touched = nullptr;           // 2 qcap

@@ -99,6 +99,12 @@ struct RunArgs {
     int32_t *touched;
     uint32_t *ntouched;
     uint32_t *tstamp;
+    // a queue's movers in pieces of AP_CHUNK neighbours (position, piece), and
+    // per position the sums and finished pieces of a node of several (zero
+    // between queues)
+    int2 *items;
+    uint32_t *nitems;
+    int32_t *apacc;
     // tables in global memory for nodes with more entries than a block's
     // shared table holds (bump-allocated per queue, lg_cap slots)
     int32_t *lg_keys;
@@ -2269,6 +2275,8 @@ __device__ double lit_exact_gain(const RunArgs &a, int32_t x, int32_t d, int32_t
     return g;
 }
 
+__device__ __forceinline__ void lit_write_action(const RunArgs &a, int i, int32_t d, const Best &bj, const Best &bl);
+
 // Per-warp values a literal team exchanges.
 struct LitScratch {
     float lbj[EV_WARPS], lbl[EV_WARPS];
@@ -2581,7 +2589,7 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
         for (int o = 16; o > 0; o >>= 1) pb += __shfl_down_sync(FULL, pb, o);
         if (lane == 0) atomicAdd(&a.ds->prof_bytes, pb + (w_in == 0 ? 44ull + 8ull * (unsigned long long)ln.cx : 0ull));
     }
-    if (w_in == 0 && lane == 0) write_action(a, i, bj, bl, 0ull);
+    if (w_in == 0 && lane == 0) lit_write_action(a, i, ln.d, bj, bl);
     team_sync<T>(tm);
     return true;
 }
@@ -2991,7 +2999,7 @@ __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int
             }
     }
     if (threadIdx.x == 0) {
-        write_action(a, i, bj, bl, 0ull);
+        lit_write_action(a, i, d, bj, bl);
         if (a.profile) atomicAdd(&a.ds->prof_bytes, 44ull + 8ull * (unsigned long long)__ldcg(&a.nmem[x]));
         hp.ns[h] = 0u;   // ready for the hub's next queue
         hp.lb[2 * h] = f2ord(-INFINITY);
@@ -2999,44 +3007,150 @@ __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int
     }
 }
 
-// Apply of one queue under the paper's gain: as apply_node (rows, n_C,
-// vol_C, 2m_C with the same in-queue corrections), and in addition each
-// membership's deg(x,C) moves with the row, a joiner's starts at its count
-// before the queue (k_lit_kupd adds the queue's other moves), the joiner is
-// appended to C's list of this iteration's joiners, and every community a
-// move touches is listed once for k_lit_fsum.
-__device__ void lit_apply_node(const RunArgs &a, int64_t bstart, int32_t blen, int64_t i, uint32_t serial,
+// ---------------------------------------------------------------------------
+// Apply of one queue under the paper's gain: rows, n_C, vol_C and 2m_C with the
+// in-queue corrections of apply_node, and deg(y,C) of every membership a move
+// concerns, in one pass over the moving nodes' neighbours.
+//
+// For a mover x (joins j, leaves l) and a neighbour y without a move of its own,
+// x's warp finds j (l) in y's row, which nobody rewrites, and adds one to
+// (takes one from) deg(y,j) (deg(y,l)).  A neighbour y that moves too is left
+// alone: its own warp meets x among its neighbours and corrects its own row,
+// which only it writes, before it rewrites it; its new membership starts at
+// its count before the queue + (neighbours joining with it) - (neighbours leaving
+// that community).  So no pass has to wait for all rows to be final: the former
+// second kernel (every mover's neighbours read again after the apply) and the
+// barrier before it are gone.
+//
+// The evaluation lists the movers (lit_write_action), a piece of at most
+// AP_CHUNK neighbours per item: idle nodes cost nothing, and a hub's
+// neighbours are spread over many warps (one warp walking 30,000 neighbours
+// alone held its queue for 2 ms); the warp that finishes a node's last piece
+// rewrites its row.
+// Mean over the queues, both steps together: 767k nodes, q 16,384: 142 -> 57 us;
+// 84k nodes, q 64: 15.3 -> 10.8 us and one launch less (cold caches).
+// ---------------------------------------------------------------------------
+constexpr int AP_CHUNK = 512;
+
+// The decision of queue position i, and its pieces of work if it moves.  One thread.
+__device__ __forceinline__ void lit_write_action(const RunArgs &a, int i, int32_t d, const Best &bj, const Best &bl) {
+    write_action(a, i, bj, bl, 0ull);
+    if (bj.c < 0 && bl.c < 0) return;
+    const uint32_t pieces = d > AP_CHUNK ? (uint32_t)(d + AP_CHUNK - 1) / AP_CHUNK : 1u;
+    const uint32_t at = atomicAdd(a.nitems, pieces);
+    for (uint32_t c = 0; c < pieces; ++c) a.items[at + c] = make_int2(i, (int)c);
+}
+
+__device__ void lit_apply_item(const RunArgs &a, int64_t bstart, int32_t blen, int2 item, uint32_t serial,
                                unsigned long long &nj, unsigned long long &nl) {
     const int lane = threadIdx.x & 31;
+    const int i = item.x;
     const int32_t j = __ldcg(&a.act[i]), l = __ldcg(&a.act[a.qcap + i]);
-    if (j < 0 && l < 0) return;
     if (!dbg_ok(a, j < a.nnodes && l < a.nnodes && (j < 0 || j != l))) return;
     const int32_t x = a.order[bstart + i];
+    const int32_t kjoin = __ldcg(&a.act[2 * a.qcap + i]), kl = __ldcg(&a.act[3 * a.qcap + i]);
+    int32_t *row = a.mem + (int64_t)x * a.K;
+    int32_t *krow = a.kmem + (int64_t)x * a.K;
+    const int32_t c = __ldcg(&a.nmem[x]);
+    const int64_t xb = a.off[x], xe = a.off[x + 1];
+    const int32_t d = (int32_t)(xe - xb);
+    if (!dbg_ok(a, c >= 0 && c <= a.K && (j < 0 || (kjoin >= 0 && kjoin <= d)))) return;
     int jj = 0, jl = 0, ll = 0;
-    for (int64_t p = a.off[x] + lane; p < a.off[x + 1]; p += 32) {
+    const int64_t pe = min(xe, xb + (int64_t)(item.y + 1) * AP_CHUNK);
+    for (int64_t p = xb + (int64_t)item.y * AP_CHUNK + lane; p < pe; p += 32) {
         const int32_t y = a.adj[p];
-        const int64_t py = a.pos[y];
-        if (py >= bstart && py < bstart + blen) {
-            const int64_t iy = py - bstart;
-            const int32_t aj = __ldcg(&a.act[iy]), al = __ldcg(&a.act[a.qcap + iy]);
+        const RowHead ids = row_head8(a.mem, y, a.K);
+        const int32_t cy = __ldcg(&a.nmem[y]);
+        const int64_t iy = (int64_t)a.pos[y] - bstart;
+        int32_t aj = -1, al = -1;
+        if (iy >= 0 && iy < blen) {
+            aj = __ldcg(&a.act[iy]);
+            al = __ldcg(&a.act[a.qcap + iy]);
+        }
+        if (aj >= 0 || al >= 0) {   // y moves too: what its move means for x
             if (j >= 0) {
                 jj += aj == j;
                 jl += al == j;
             }
             if (l >= 0) ll += al == l;
+            if (aj >= 0 && aj != l) {
+                const int s = row_find(row, c, aj);
+                if (s >= 0) {
+                    const int32_t was = atomicAdd(&krow[s], 1);
+                    dbg_ok(a, was >= 0 && was < d);
+                }
+            }
+            if (al >= 0 && al != l) {
+                const int s = row_find(row, c, al);
+                if (s >= 0) dbg_ok(a, atomicAdd(&krow[s], -1) >= 1);
+            }
+            continue;
+        }
+        if (!dbg_ok(a, cy >= 0 && cy <= a.K)) continue;
+        const int32_t *rowy = a.mem + (int64_t)y * a.K;
+        int32_t *krowy = a.kmem + (int64_t)y * a.K;
+        if (j >= 0) {
+            const int s = head_find(ids, rowy, cy, j);
+            if (s >= 0) {
+                const int32_t was = atomicAdd(&krowy[s], 1);
+                dbg_ok(a, was >= 0 && was < a.deg[y]);
+            }
+        }
+        if (l >= 0) {
+            const int s = head_find(ids, rowy, cy, l);
+            if (s >= 0) dbg_ok(a, atomicAdd(&krowy[s], -1) >= 1);
         }
     }
+    __syncwarp();
     jj = __reduce_add_sync(FULL, jj);
     jl = __reduce_add_sync(FULL, jl);
     ll = __reduce_add_sync(FULL, ll);
-    const int32_t d = a.deg[x];
-    const int32_t kjoin = __ldcg(&a.act[2 * a.qcap + i]);
-    int32_t *row = a.mem + (int64_t)x * a.K;
-    int32_t *krow = a.kmem + (int64_t)x * a.K;
-    const int32_t c = __ldcg(&a.nmem[x]);
-    if (!dbg_ok(a, c >= 0 && c <= a.K && (j < 0 || (kjoin >= 0 && kjoin <= d)))) return;
+    if (d > AP_CHUNK) {   // several pieces: the last to finish goes on with the sums of all
+        int32_t *acc = a.apacc + 4 * (int64_t)i;
+        const int pieces = (d + AP_CHUNK - 1) / AP_CHUNK;
+        int last = 0;
+        if (lane == 0) {
+            if (jj) atomicAdd(&acc[0], jj);
+            if (jl) atomicAdd(&acc[1], jl);
+            if (ll) atomicAdd(&acc[2], ll);
+        }
+        __threadfence();   // every lane's corrections before the piece is counted
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(&acc[3], 1) == pieces - 1;
+        if (!__shfl_sync(FULL, last, 0)) return;
+        __threadfence();
+        jj = __ldcg(&acc[0]);
+        jl = __ldcg(&acc[1]);
+        ll = __ldcg(&acc[2]);
+        __syncwarp();
+        if (lane < 4) acc[lane] = 0;   // ready for the next queue
+    }
+    const int32_t kstart = kjoin + jj - jl;
     int32_t c_new = c;
-    if (lane == 0) {
+    if (c <= 32) {
+        // the whole row in one load per array: leave l, insert j, ascending
+        const int32_t v = lane < c ? __ldcg(&row[lane]) : 0;
+        const int32_t kv = lane < c ? __ldcg(&krow[lane]) : 0;
+        const bool keep = lane < c && v != l;
+        const unsigned km = __ballot_sync(FULL, keep);
+        const int kept = __popc(km);
+        const int ins = j >= 0 ? __popc(__ballot_sync(FULL, keep && v < j)) : kept;
+        if (j >= 0 && kept >= a.K) {
+            if (lane == 0) atomicOr(&a.ds->err, DERR_CAPACITY);
+        } else {
+            if (keep) {
+                const int s = __popc(km & lanemask_lt());
+                const int t = s + (j >= 0 && s >= ins ? 1 : 0);
+                row[t] = v;
+                krow[t] = kv;
+            }
+            if (j >= 0 && lane == 0) {
+                row[ins] = j;
+                krow[ins] = kstart;
+            }
+            c_new = kept + (j >= 0 ? 1 : 0);
+        }
+    } else if (lane == 0) {
         int32_t cc2 = c;
         if (l >= 0) {
             int32_t o = 0;
@@ -3062,78 +3176,47 @@ __device__ void lit_apply_node(const RunArgs &a, int64_t bstart, int32_t blen, i
                     --s;
                 }
                 row[s] = j;
-                krow[s] = kjoin;
+                krow[s] = kstart;
                 ++cc2;
             }
         }
         c_new = cc2;
-        if (l >= 0) {
-            const int32_t kl = __ldcg(&a.act[3 * a.qcap + i]);
-            atomicAdd(&a.comm[l].n, -1);
-            atomicAdd(&a.comm[l].vol, (uint32_t)(-d));
-            atomicAdd(&a.comm[l].m2, (uint32_t)(-2 * kl + ll));
-            ++nl;
-            if (atomicExch(&a.tstamp[l], serial) != serial) a.touched[atomicAdd(a.ntouched, 1u)] = l;
-        }
-        if (j >= 0) {
-            atomicAdd(&a.comm[j].n, 1);
-            atomicAdd(&a.comm[j].vol, (uint32_t)d);
-            atomicAdd(&a.comm[j].m2, (uint32_t)(2 * kjoin + jj - 2 * jl));
+    }
+    // lane 0: the community left, lane 1: the one joined
+    const int32_t C = lane == 0 ? l : lane == 1 ? j : -1;
+    if (C >= 0) {
+        const bool in = lane == 1;
+        atomicAdd(&a.comm[C].n, in ? 1 : -1);
+        atomicAdd(&a.comm[C].vol, in ? (uint32_t)d : (uint32_t)(-d));
+        atomicAdd(&a.comm[C].m2, (uint32_t)(in ? 2 * kjoin + jj - 2 * jl : -2 * kl + ll));
+        if (in) {
             ++nj;
-            const unsigned long long slot = atomicAdd(&a.cm_cnt[j], 1u);
-            if ((long long)slot < (long long)(a.cm_off[j + 1] - a.cm_off[j])) {
-                a.cm_node[a.cm_off[j] + slot] = x;
+            const unsigned long long slot = atomicAdd(&a.cm_cnt[C], 1u);
+            if ((long long)slot < (long long)(a.cm_off[C + 1] - a.cm_off[C])) {
+                a.cm_node[a.cm_off[C] + slot] = x;
             } else {
                 const int32_t e = (int32_t)atomicAdd(a.jl_count, 1u);
                 a.jl_node[e] = x;
-                a.jl_next[e] = atomicExch(&a.jl_head[j], e);
+                a.jl_next[e] = atomicExch(&a.jl_head[C], e);
             }
-            if (atomicExch(&a.tstamp[j], serial) != serial) a.touched[atomicAdd(a.ntouched, 1u)] = j;
+        } else {
+            ++nl;
         }
-        a.nmem[x] = c_new;
+        if (atomicExch(&a.tstamp[C], serial) != serial) a.touched[atomicAdd(a.ntouched, 1u)] = C;
     }
+    if (lane == 0) a.nmem[x] = c_new;
 }
 
+// A resident grid at most; warps stride over the queue's items.
 __global__ void __launch_bounds__(AP_THREADS) k_lit_apply(RunArgs a, int64_t bstart, int32_t blen, int64_t bidx) {
     pdl_trigger();
     pdl_wait();
     const uint32_t serial = (uint32_t)queue_serial(a, bidx);
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t count = __ldcg(a.nitems);
     unsigned long long nj = 0, nl = 0;
-    if (i < blen) lit_apply_node(a, bstart, blen, i, serial, nj, nl);
+    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < count; t += (gridDim.x * blockDim.x) >> 5)
+        lit_apply_item(a, bstart, blen, __ldcg(&a.items[t]), serial, nj, nl);
     flush_counts(a, nj, nl);
-}
-
-// Every neighbour y of a node that joined (left) C and is in C after the
-// queue has one more (fewer) neighbour in C.  Summed over the queue this
-// turns each membership's count before the queue into its count after it,
-// for stayers and joiners alike (leavers' memberships are gone).
-__global__ void __launch_bounds__(AP_THREADS) k_lit_kupd(RunArgs a, int64_t bstart, int32_t blen) {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= blen) return;
-    const int32_t j = __ldcg(&a.act[i]), l = __ldcg(&a.act[a.qcap + i]);
-    if (j < 0 && l < 0) return;
-    const int32_t x = a.order[bstart + i];
-    for (int64_t p = a.off[x] + lane; p < a.off[x + 1]; p += 32) {
-        const int32_t y = a.adj[p];
-        const int32_t cy = __ldcg(&a.nmem[y]);
-        const int32_t *row = a.mem + (int64_t)y * a.K;
-        if (j >= 0) {
-            const int s = row_find(row, cy, j);
-            if (s >= 0) {
-                const int32_t was = atomicAdd(&a.kmem[(int64_t)y * a.K + s], 1);
-                dbg_ok(a, was >= 0 && was < a.deg[y]);
-            }
-        }
-        if (l >= 0) {
-            const int s = row_find(row, cy, l);
-            if (s >= 0) {
-                const int32_t was = atomicAdd(&a.kmem[(int64_t)y * a.K + s], -1);
-                dbg_ok(a, was >= 1);
-            }
-        }
-    }
 }
 
 // F(n-1), F(n), F(n+1) of communities: list[0 .. *count) (or every id below
@@ -4093,6 +4176,9 @@ RunArgs make_args(lf_graph *g, Readback *rbd) {
     a.touched = g->touched;
     a.ntouched = g->lit_ctr;
     a.tstamp = g->tstamp;
+    a.items = reinterpret_cast<int2 *>(g->lit_items);
+    a.nitems = g->lit_ctr;
+    a.apacc = g->lit_apacc;
     a.lg_cap = g->lg_cap;
     a.lg_dv = static_cast<float *>(g->lg_area);
     a.lg_keys = reinterpret_cast<int32_t *>(a.lg_dv + g->lg_cap);
@@ -4486,7 +4572,7 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
     const int T0 = choose_team(g, q);
     static const int per_sm_big = blocks_per_sm(k_lit_big, EV_THREADS, LIT_SMEM);
     const unsigned big_grid = (unsigned)(num_sms() * std::max(1, per_sm_big));
-    LF_CUDA(cudaMemsetAsync(g->lit_ctr + 3 * first, 0, (size_t)(3 * count) * sizeof(uint32_t), g->stream));
+    LF_CUDA(cudaMemsetAsync(g->lit_ctr + 4 * first, 0, (size_t)(4 * count) * sizeof(uint32_t), g->stream));
     LF_CUDA(cudaMemsetAsync(g->lit_used + first, 0, (size_t)count * sizeof(unsigned long long), g->stream));
     const bool prof = g->profile && (int64_t)g->prof_ev.size() >= 2 * (first + count);
     for (int64_t b = first; b < first + count; ++b) {
@@ -4495,9 +4581,10 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         queue_bounds(g, q, b, bstart, blen);
         const int T = sched ? choose_team(g, blen) : T0;
         const int teams = EV_WARPS / T;
-        uint32_t *ctr = g->lit_ctr + 3 * b;
+        uint32_t *ctr = g->lit_ctr + 4 * b;
         RunArgs ab = a;
         ab.ntouched = ctr + 2;
+        ab.nitems = ctr + 3;
         if (prof) record_event(g, g->prof_ev[2 * b], capturing);
         const unsigned grid = (unsigned)((blen + teams - 1) / teams);
         switch (T) {
@@ -4522,12 +4609,12 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
             g->launches += 5;
         }
         if (prof) record_event(g, g->prof_ev[2 * b + 1], capturing);
-        const unsigned ag = grid_for((int64_t)blen * 32, AP_THREADS, 1 << 30);
+        const int64_t longest = g->max_deg / AP_CHUNK + 1;   // pieces of one node at most
+        const unsigned ag = grid_for((int64_t)blen * longest * 32, AP_THREADS, 6 * (int64_t)num_sms());
         launch_pdl(k_lit_apply, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
-        k_lit_kupd<<<ag, AP_THREADS, 0, g->stream>>>(ab, bstart, blen);
         k_lit_fsum<<<(unsigned)std::min<int64_t>((2 * (int64_t)blen + 31) / 32, 8 * (int64_t)num_sms()), EV_THREADS, 0,
                      g->stream>>>(ab, g->touched, ctr + 2, 0);
-        g->launches += 5;
+        g->launches += 4;
     }
     LF_LAUNCHED();
 }
@@ -4555,16 +4642,24 @@ void ensure_lit(lf_graph *g, int64_t q, int64_t nb) {
     if (g->lit_qcap < q) {
         if (g->lit_over) dfree(g, g->lit_over);
         if (g->touched) dfree(g, g->touched);
+        if (g->lit_items) dfree(g, g->lit_items);
+        if (g->lit_apacc) dfree(g, g->lit_apacc);
+        g->lit_over = g->touched = g->lit_apacc = nullptr;
+        g->lit_items = nullptr;
+        // a node of degree d brings at most 1 + d / AP_CHUNK items
+        g->lit_items = dalloc_n<unsigned long long>(g, q + 2 * g->m / AP_CHUNK + 1);
+        g->lit_apacc = dalloc_n<int32_t>(g, 4 * q);
+        LF_CUDA(cudaMemsetAsync(g->lit_apacc, 0, (size_t)(4 * q) * 4, g->stream));
         g->lit_qcap = q;
         g->lit_over = dalloc_n<int32_t>(g, q);
         g->touched = dalloc_n<int32_t>(g, 2 * q);
         drop_graph(g);
     }
-    if (g->lit_ctr_cap < 3 * nb) {
+    if (g->lit_ctr_cap < 4 * nb) {
         if (g->lit_ctr) dfree(g, g->lit_ctr);
         if (g->lit_used) dfree(g, g->lit_used);
-        g->lit_ctr_cap = 3 * nb;
-        g->lit_ctr = dalloc_n<uint32_t>(g, 3 * nb);
+        g->lit_ctr_cap = 4 * nb;
+        g->lit_ctr = dalloc_n<uint32_t>(g, 4 * nb);
         g->lit_used = dalloc_n<unsigned long long>(g, nb);
         drop_graph(g);
     }
@@ -5043,7 +5138,10 @@ void free_run_state(lf_graph *g) {
     g->bar_flags_cap = 0;
     for (auto e : g->prof_ev) cudaEventDestroy(e);
     g->prof_ev.clear();
-    for (int32_t **pp : {&g->kmem, &g->cm_node, &g->jl_head, &g->jl_next, &g->jl_node, &g->lit_over, &g->touched})
+    if (g->lit_items) dfree(g, g->lit_items);
+    g->lit_items = nullptr;
+    for (int32_t **pp : {&g->kmem, &g->cm_node, &g->jl_head, &g->jl_next, &g->jl_node, &g->lit_over, &g->touched,
+                         &g->lit_apacc})
         if (*pp) {
             dfree(g, *pp);
             *pp = nullptr;
