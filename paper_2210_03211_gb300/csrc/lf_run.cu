@@ -2309,6 +2309,32 @@ __device__ __forceinline__ int lit_insert(int32_t *keys, uint32_t *vals, uint32_
     return -1;
 }
 
+// The bracket of every candidate in the table: dv <- X, aux <- E, and per
+// lane the largest lower ends of the two kinds.
+template <int T>
+__device__ __forceinline__ void lit_screen_table(const RunArgs &a, int32_t d, int32_t *keys, uint32_t *vals, int32_t *aux,
+                                                 float *dv, uint32_t H, int tm, int w_in, float &lbj, float &lbl,
+                                                 unsigned long long &pb, bool count_bytes) {
+    const float *hs = reinterpret_cast<const float *>(aux);
+    for (uint32_t s = (uint32_t)w_in * 32 + (threadIdx.x & 31); s < H; s += T * 32) {
+        const int32_t C = keys[s];
+        if (C == EMPTY_KEY) continue;
+        const uint32_t v = vals[s];
+        float X, E;
+        lit_screen(a, C, v, d, hs[s], X, E);
+        dv[s] = X;
+        aux[s] = __float_as_int(E);
+        const float L = X - E;
+        if (v & OWN_FLAG) lbl = fmaxf(lbl, L);
+        else lbj = fmaxf(lbj, L);
+        if (count_bytes) {
+            pb += 40ull;
+            atomicAdd(&a.ds->prof_cands, 1ull);
+        }
+    }
+    team_sync<T>(tm);
+}
+
 // One pass over the node's candidates of part p (of P): the table gets x's
 // own communities (own flag), then every neighbour membership (y, C) adds
 // one to C's count and its correction h(y) (by C's size before the queue and
@@ -2363,23 +2389,7 @@ __device__ bool lit_pass(const RunArgs &a, const LitNode &ln, int P, int p, int3
         ok = __all_sync(FULL, ok);
     }
     if (!ok) return false;
-    for (uint32_t s = tl; s < H; s += NT) {
-        const int32_t C = keys[s];
-        if (C == EMPTY_KEY) continue;
-        const uint32_t v = vals[s];
-        float X, E;
-        lit_screen(a, C, v, ln.d, hs[s], X, E);
-        dv[s] = X;
-        aux[s] = __float_as_int(E);
-        const float L = X - E;
-        if (v & OWN_FLAG) lbl = fmaxf(lbl, L);
-        else lbj = fmaxf(lbj, L);
-        if (count_bytes) {
-            pb += 40ull;
-            atomicAdd(&a.ds->prof_cands, 1ull);
-        }
-    }
-    team_sync<T>(tm);
+    lit_screen_table<T>(a, ln.d, keys, vals, aux, dv, H, tm, w_in, lbj, lbl, pb, count_bytes);
     return true;
 }
 
@@ -2523,67 +2533,42 @@ __device__ void lit_exact_survivors(const RunArgs &a, const LitNode &ln, const i
     }
 }
 
-// A node's decision with the paper's gain, by a team of T warps over a table
-// of H slots (P parts of the candidates, one pass each).  False if a part
-// overflowed the table (the caller retries with more parts).
+// One kind's survivors: none or a lone one with a positive lower end settles
+// it; true if exact sums have to.
+__device__ __forceinline__ bool lit_settle(const RunArgs &a, int count, int32_t C, int32_t k, float L, Best &b) {
+    if (count == 0) return false;
+    if (a.screen && count == 1 && L > 0.f) {
+        b = Best{INFINITY, C, k};
+        return false;
+    }
+    return true;
+}
+
+// The best exact gains of a team's warps, on its first warp.
 template <int T>
-__device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P, int32_t *keys, uint32_t *vals,
-                              int32_t *aux, float *dv, uint32_t H, LitScratch &ls, unsigned long long *acc,
-                              int tm, int w_in) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned long long pb = 0;
-    float lbj = -INFINITY, lbl = -INFINITY;
-    for (int p = 0; p < P; ++p)
-        if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, a.profile != 0))
-            return false;
-    team_max2<T>(ls, tm, lbj, lbl);
-    int cj = 0, cl = 0;
-    int32_t Cj = -1, Cl = -1, kj = 0, kl = 0;
-    float Lj = 0.f, Ll = 0.f;
-    for (int p = 0; p < P; ++p) {
-        if (P > 1 && !lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, false))
-            return false;
-        lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, cj, cl, Cj, Cl, kj, kl, Lj, Ll);
-    }
-    Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
-    bool do_j = cj > 0, do_l = cl > 0;
-    if (a.screen && cj == 1 && Lj > 0.f) {
-        bj = Best{INFINITY, Cj, kj};
-        do_j = false;
-    }
-    if (a.screen && cl == 1 && Ll > 0.f) {
-        bl = Best{INFINITY, Cl, kl};
-        do_l = false;
-    }
-    if (do_j || do_l) {
-        for (int p = 0; p < P; ++p) {
-            if (P > 1) {
-                float d1 = -INFINITY, d2 = -INFINITY;
-                if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, d1, d2, pb, false)) return false;
-                int c1 = 0, c2 = 0;
-                int32_t e1 = -1, e2 = -1, e3 = 0, e4 = 0;
-                float e5 = 0.f, e6 = 0.f;
-                lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, c1, c2, e1, e2, e3, e4, e5, e6);
-            }
-            lit_exact_survivors<T>(a, ln, keys, vals, H, do_j, do_l, acc, w_in, bj, bl);
-            team_sync<T>(tm);
+__device__ __forceinline__ void lit_team_best(LitScratch &ls, int tm, int w_in, Best &bj, Best &bl) {
+    if constexpr (T > 1) {
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        if (lane == 0) {
+            ls.bgj[w] = bj.g; ls.bcj[w] = bj.c; ls.bkj[w] = bj.k;
+            ls.bgl[w] = bl.g; ls.bcl[w] = bl.c; ls.bkl[w] = bl.k;
         }
-        if constexpr (T > 1) {
-            if (lane == 0) {
-                ls.bgj[w] = bj.g; ls.bcj[w] = bj.c; ls.bkj[w] = bj.k;
-                ls.bgl[w] = bl.g; ls.bcl[w] = bl.c; ls.bkl[w] = bl.k;
+        team_sync<T>(tm);
+        if (w_in == 0) {
+            for (int k2 = 1; k2 < T; ++k2) {
+                const int q = tm * T + k2;
+                if (better(ls.bgj[q], ls.bcj[q], bj.g, bj.c)) bj = Best{ls.bgj[q], ls.bcj[q], ls.bkj[q]};
+                if (better(ls.bgl[q], ls.bcl[q], bl.g, bl.c)) bl = Best{ls.bgl[q], ls.bcl[q], ls.bkl[q]};
             }
-            team_sync<T>(tm);
-            if (w_in == 0) {
-                for (int k2 = 1; k2 < T; ++k2) {
-                    const int q = tm * T + k2;
-                    if (better(ls.bgj[q], ls.bcj[q], bj.g, bj.c)) bj = Best{ls.bgj[q], ls.bcj[q], ls.bkj[q]};
-                    if (better(ls.bgl[q], ls.bcl[q], bl.g, bl.c)) bl = Best{ls.bgl[q], ls.bcl[q], ls.bkl[q]};
-                }
-            }
-            team_sync<T>(tm);
         }
+        team_sync<T>(tm);
     }
+}
+
+template <int T>
+__device__ __forceinline__ void lit_finish(const RunArgs &a, int i, const LitNode &ln, const Best &bj, const Best &bl,
+                                           int tm, int w_in, unsigned long long pb) {
+    const int lane = threadIdx.x & 31;
     if (a.profile) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) pb += __shfl_down_sync(FULL, pb, o);
@@ -2591,6 +2576,139 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
     }
     if (w_in == 0 && lane == 0) lit_write_action(a, i, ln.d, bj, bl);
     team_sync<T>(tm);
+}
+
+// The decision from one bracketed table (all candidates in it): survivors,
+// their exact gains where the bracket cannot tell, the action written.
+template <int T>
+__device__ __forceinline__ void lit_decide(const RunArgs &a, int i, const LitNode &ln, int32_t *keys, uint32_t *vals,
+                                           const int32_t *aux, const float *dv, uint32_t H, float lbj, float lbl,
+                                           LitScratch &ls, unsigned long long *acc, int tm, int w_in,
+                                           unsigned long long pb) {
+    const int lane = threadIdx.x & 31;
+    int cj = 0, cl = 0;
+    int32_t Cj = -1, Cl = -1, kj = 0, kl = 0;
+    float Lj = 0.f, Ll = 0.f;
+    lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, cj, cl, Cj, Cl, kj, kl, Lj, Ll);
+    Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
+    const bool do_j = lit_settle(a, cj, Cj, kj, Lj, bj), do_l = lit_settle(a, cl, Cl, kl, Ll, bl);
+    if (do_j || do_l) {
+        lit_exact_survivors<T>(a, ln, keys, vals, H, do_j, do_l, acc, w_in, bj, bl);
+        team_sync<T>(tm);
+        lit_team_best<T>(ls, tm, w_in, bj, bl);
+    }
+    lit_finish<T>(a, i, ln, bj, bl, tm, w_in, pb);
+}
+
+// A node's decision with the paper's gain, by a team of T warps over a table
+// of H slots (P parts of the candidates, one pass each).  False if a part
+// overflowed the table (the caller retries with more parts).
+template <int T>
+__device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P, int32_t *keys, uint32_t *vals,
+                              int32_t *aux, float *dv, uint32_t H, LitScratch &ls, unsigned long long *acc,
+                              int tm, int w_in) {
+    unsigned long long pb = 0;
+    float lbj = -INFINITY, lbl = -INFINITY;
+    for (int p = 0; p < P; ++p)
+        if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, a.profile != 0))
+            return false;
+    team_max2<T>(ls, tm, lbj, lbl);
+    if (P == 1) {
+        lit_decide<T>(a, i, ln, keys, vals, aux, dv, H, lbj, lbl, ls, acc, tm, w_in, pb);
+        return true;
+    }
+    int cj = 0, cl = 0;
+    int32_t Cj = -1, Cl = -1, kj = 0, kl = 0;
+    float Lj = 0.f, Ll = 0.f;
+    for (int p = 0; p < P; ++p) {
+        if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, false)) return false;
+        lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, cj, cl, Cj, Cl, kj, kl, Lj, Ll);
+    }
+    Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
+    const bool do_j = lit_settle(a, cj, Cj, kj, Lj, bj), do_l = lit_settle(a, cl, Cl, kl, Ll, bl);
+    if (do_j || do_l) {
+        for (int p = 0; p < P; ++p) {
+            float d1 = -INFINITY, d2 = -INFINITY;
+            if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, d1, d2, pb, false)) return false;
+            int c1 = 0, c2 = 0;
+            int32_t e1 = -1, e2 = -1, e3 = 0, e4 = 0;
+            float e5 = 0.f, e6 = 0.f;
+            lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, c1, c2, e1, e2, e3, e4, e5, e6);
+            lit_exact_survivors<T>(a, ln, keys, vals, H, do_j, do_l, acc, w_in, bj, bl);
+            team_sync<T>(tm);
+        }
+        lit_team_best<T>(ls, tm, w_in, bj, bl);
+    }
+    lit_finish<T>(a, i, ln, bj, bl, tm, w_in, pb);
+    return true;
+}
+
+// A node of at most 32 neighbours, by one warp over a table of up to hcap slots:
+// a neighbour per lane, whose count, degree, ids and deg(y,C) load together, so
+// the chain of dependent loads is neighbour -> rows -> community sizes ->
+// bracket values, half of the general path's (which counts the entries first
+// to size its table, then reads the rows).  y0: this lane's neighbour.  False if
+// the entries could fill more than half of the table.
+constexpr int LIT_SMALL_DEG = 32;
+
+__device__ bool lit_eval_small(const RunArgs &a, int i, LitNode &ln, int32_t y0, int32_t *keys, uint32_t *vals,
+                               int32_t *aux, float *dv, uint32_t hcap, LitScratch &ls, unsigned long long *acc) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool on = lane < ln.d && dbg_ok(a, y0 >= 0 && y0 < a.nnodes);
+    const int32_t y = on ? y0 : ln.x;
+    const RowHead ids = row_head8(a.mem, y, a.K), ks = row_head8(a.kmem, y, a.K), own = row_head8(a.mem, ln.x, a.K);
+    int32_t cy = on ? __ldcg(&a.nmem[y]) : 0;
+    const int32_t dy = a.deg[y];
+    ln.cx = __ldcg(&a.nmem[ln.x]);
+    if (!dbg_ok(a, cy >= 0 && cy <= a.K)) cy = 0;
+    if (!dbg_ok(a, ln.cx >= 0 && ln.cx <= a.K)) ln.cx = 0;
+    const int32_t entries = __reduce_add_sync(FULL, cy) + ln.cx;
+    const int32_t cmax = __reduce_max_sync(FULL, cy);
+    uint32_t H = 32;
+    while (H < 2u * (uint32_t)entries) H <<= 1;
+    if (H > hcap) return false;
+    const uint32_t hm = H - 1;
+    float *hs = reinterpret_cast<float *>(aux);
+    for (uint32_t s = lane; s < H; s += 32) {
+        keys[s] = EMPTY_KEY;
+        vals[s] = 0u;
+        hs[s] = 0.f;
+    }
+    __syncwarp();
+    const int32_t *rowx = a.mem + (int64_t)ln.x * a.K;
+    for (int j = lane; j < ln.cx; j += 32) ht_insert(keys, vals, hm, head_entry(own, rowx, j), 0u, true);
+    __syncwarp();
+    const int32_t *rowy = a.mem + (int64_t)y * a.K, *krowy = a.kmem + (int64_t)y * a.K;
+    for (int s0 = 0; s0 < cmax; s0 += 4) {
+        int32_t C[4], k[4], n[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {   // four communities' sizes in flight
+            C[t] = -1;
+            n[t] = 0;
+            k[t] = 0;
+            if (s0 + t < cy) {
+                C[t] = head_entry(ids, rowy, s0 + t);
+                k[t] = head_entry(ks, krowy, s0 + t);
+                if (!dbg_ok(a, C[t] >= 0 && C[t] < a.nnodes && k[t] >= 0 && k[t] <= dy)) C[t] = -1;
+                if (C[t] >= 0) n[t] = __ldcg(&a.comm[C[t]].n);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (C[t] < 0) continue;
+            const int slot = lit_insert(keys, vals, hm, C[t]);   // has room: H >= 2 x entries
+            if (slot < 0) continue;
+            const float h = (vals[slot] & OWN_FLAG) ? lit_h_leave32(k[t], dy, n[t]) : lit_h_join32(k[t], dy, n[t]);
+            if (h != 0.f) atomicAdd(&hs[slot], h);
+        }
+    }
+    __syncwarp();
+    unsigned long long pb = a.profile && on ? 12ull + 8ull * (unsigned long long)cy : 0ull;
+    float lbj = -INFINITY, lbl = -INFINITY;
+    lit_screen_table<1>(a, ln.d, keys, vals, aux, dv, H, w, 0, lbj, lbl, pb, a.profile != 0);
+    lbj = warp_max_f(lbj);
+    lbl = warp_max_f(lbl);
+    lit_decide<1>(a, i, ln, keys, vals, aux, dv, H, lbj, lbl, ls, acc, w, 0, pb);
     return true;
 }
 
@@ -2603,32 +2721,38 @@ __device__ __forceinline__ void lit_smem(double *base, float *&dv, int32_t *&key
     acc = reinterpret_cast<unsigned long long *>(aux + LB_SLOTS);
 }
 
-// Teams of T warps, one queued node each.  A node whose entries (own rows
-// plus its neighbours' rows) could fill more than half of the team's table
-// is listed for k_lit_big.  Counters: over[0] = listed nodes, over[1] = next.
-template <int T>
-__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t bstart, int32_t blen, uint32_t *over,
-                                                           int32_t *over_list) {
-    extern __shared__ double lit_dyn[];
-    __shared__ LitScratch ls;
-    float *dv;
+struct LitTables {   // a block's shared tables and per-warp accumulators
     int32_t *keys, *aux;
     uint32_t *vals;
+    float *dv;
     unsigned long long *acc;
-    lit_smem(lit_dyn, dv, keys, vals, aux, acc);
+};
+
+// One queued node by a team of T warps (index i in the queue; its static data and
+// this warp's first neighbours prefetched in pf).  False if its entries (own row
+// plus its neighbours' rows) could fill more than half of the team's table: a
+// whole block has to take it.
+template <int T>
+__device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const NodePrefetch &pf, const LitTables &t,
+                                              LitScratch &ls, int tm, int w_in) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int c = lane; c < SACC_CHUNKS; c += 32) acc[w * SACC_CHUNKS + c] = 0ull;
-    pdl_trigger();
-    pdl_wait();
-    const int tm = w / T, w_in = w % T;
-    const int i = (int)blockIdx.x * (EV_WARPS / T) + tm;
-    if (i >= blen) return;   // the whole team leaves together
     LitNode ln;
-    ln.x = a.order[bstart + i];
-    ln.beg = a.off[ln.x];
-    ln.end = a.off[ln.x + 1];
-    ln.d = (int32_t)(ln.end - ln.beg);
-    if (ln.d > a.lit_hub_deg) return;   // the hub kernels decide it
+    ln.x = pf.x;
+    ln.beg = pf.beg;
+    ln.end = pf.end;
+    ln.d = pf.d;
+    const int base = tm * T * LW;
+    if (ln.d <= LIT_SMALL_DEG) {
+        if constexpr (T == 1) {
+            return lit_eval_small(a, i, ln, pf.y0, t.keys + base, t.vals + base, t.aux + base, t.dv + base, LW, ls,
+                                  t.acc + w * SACC_CHUNKS);
+        } else if (2 * (ln.d + 1) * a.K <= T * LW) {   // the table holds it whatever its rows
+            if (w_in == 0)
+                lit_eval_small(a, i, ln, pf.y0, t.keys + base, t.vals + base, t.aux + base, t.dv + base, T * LW, ls,
+                               t.acc + w * SACC_CHUNKS);
+            return true;
+        }
+    }
     ln.cx = __ldcg(&a.nmem[ln.x]);
     long long bound = w_in == 0 && lane == 0 ? ln.cx : 0;
     for (int64_t q = ln.beg + w_in * 32 + lane; q < ln.end; q += T * 32) bound += __ldcg(&a.nmem[a.adj[q]]);
@@ -2643,93 +2767,120 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t b
     }
     uint32_t H = 32;
     while ((long long)H < 2 * bound) H <<= 1;
-    if (H > (uint32_t)(T * LW)) {
-        if (w_in == 0 && lane == 0) {
-            const uint32_t slot = atomicAdd(&over[0], 1u);
-            over_list[slot] = i;
-        }
-        return;
-    }
-    const int base = tm * T * LW;
-    if (!lit_eval_node<T>(a, i, ln, 1, keys + base, vals + base, aux + base, dv + base, H, ls, acc + w * SACC_CHUNKS,
-                          tm, w_in)) {
+    if (H > (uint32_t)(T * LW)) return false;
+    if (!lit_eval_node<T>(a, i, ln, 1, t.keys + base, t.vals + base, t.aux + base, t.dv + base, H, ls,
+                          t.acc + w * SACC_CHUNKS, tm, w_in)) {
         if (w_in == 0 && lane == 0) atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: H >= 2 x entries
+    }
+    return true;
+}
+
+__device__ __forceinline__ LitTables lit_tables(double *dyn) {
+    LitTables t;
+    lit_smem(dyn, t.dv, t.keys, t.vals, t.aux, t.acc);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int c = lane; c < SACC_CHUNKS; c += 32) t.acc[w * SACC_CHUNKS + c] = 0ull;
+    __syncwarp();
+    return t;
+}
+
+// Teams of T warps, one queued node each.  A node too large for its team is listed
+// for k_lit_big.  Counters: over[0] = listed nodes, over[1] = next.  The
+// order, offsets and neighbour ids never change in a run, so they are read
+// before the wait for the previous kernel.
+template <int T>
+__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t bstart, int32_t blen, uint32_t *over,
+                                                           int32_t *over_list) {
+    extern __shared__ double lit_dyn[];
+    __shared__ LitScratch ls;
+    const LitTables t = lit_tables(lit_dyn);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int tm = w / T, w_in = w % T;
+    const int i = (int)blockIdx.x * (EV_WARPS / T) + tm;
+    NodePrefetch pf;
+    prefetch_node(a, bstart, blen, i, w_in, pf);
+    pdl_trigger();
+    pdl_wait();
+    if (i >= blen) return;   // the whole team leaves together
+    if (pf.d > a.lit_hub_deg) return;   // the hub kernels decide it
+    if (!lit_eval_team<T>(a, i, pf, t, ls, tm, w_in) && w_in == 0 && lane == 0) over_list[atomicAdd(&over[0], 1u)] = i;
+}
+
+// One node by the whole block: over the block's table in as many parts as needed
+// (a part that overflows doubles the parts), or over a table of its own in
+// global memory if the queue's area has room.
+__device__ void lit_big_node(const RunArgs &a, int64_t bstart, int i, const LitTables &t, LitScratch &ls,
+                             long long &s_base, unsigned long long *used) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    LitNode ln;
+    ln.x = a.order[bstart + i];
+    ln.beg = a.off[ln.x];
+    ln.end = a.off[ln.x + 1];
+    ln.d = (int32_t)(ln.end - ln.beg);
+    ln.cx = __ldcg(&a.nmem[ln.x]);
+    long long bound = threadIdx.x == 0 ? ln.cx : 0;
+    for (int64_t q = ln.beg + threadIdx.x; q < ln.end; q += EV_THREADS) bound += __ldcg(&a.nmem[a.adj[q]]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) bound += __shfl_xor_sync(FULL, bound, o);
+    if (lane == 0) ls.part[w] = bound;
+    __syncthreads();
+    bound = 0;
+    for (int k2 = 0; k2 < EV_WARPS; ++k2) bound += ls.part[k2];
+    __syncthreads();
+    if (2 * bound > LB_SLOTS) {   // a table of its own in global memory, if the queue's area has room
+        unsigned long long H = 32;
+        while ((long long)H < 2 * bound) H <<= 1;
+        if (threadIdx.x == 0) {
+            const unsigned long long base = atomicAdd(used, H);
+            s_base = base + H <= a.lg_cap ? (long long)base : -1ll;
+        }
+        __syncthreads();
+        const long long base = s_base;
+        __syncthreads();
+        if (base >= 0) {
+            lit_eval_node<EV_WARPS>(a, i, ln, 1, a.lg_keys + base, a.lg_vals + base, a.lg_aux + base, a.lg_dv + base,
+                                    (uint32_t)H, ls, t.acc + w * SACC_CHUNKS, 0, w);
+            return;
+        }
+    }
+    int P = (int)((bound + LIT_PART_ENTRIES - 1) / LIT_PART_ENTRIES);
+    uint32_t Hs = (uint32_t)LB_SLOTS;
+    if (P < 1 || 2 * bound <= LB_SLOTS) {   // one pass over a table of pow2 >= 2 x entries
+        P = 1;
+        Hs = 32;
+        while ((long long)Hs < 2 * bound) Hs <<= 1;
+    }
+    while (!lit_eval_node<EV_WARPS>(a, i, ln, P, t.keys, t.vals, t.aux, t.dv, Hs, ls, t.acc + w * SACC_CHUNKS, 0, w)) {
+        Hs = (uint32_t)LB_SLOTS;
+        P *= 2;
+        if (P > (1 << 22)) {   // cannot happen for < 2^31 entries; leave an error, not a loop
+            if (threadIdx.x == 0) atomicOr(&a.ds->err, DERR_CHECK);
+            break;
+        }
     }
 }
 
-// Listed nodes, one block each, over the block's whole table in as many
-// parts as needed (a part that overflows doubles the parts).
+// Listed nodes, one block each, taken from a counter.
 __global__ void __launch_bounds__(EV_THREADS, 3) k_lit_big(RunArgs a, int64_t bstart, uint32_t *over,
                                                           const int32_t *over_list, unsigned long long *used) {
     extern __shared__ double lit_dyn[];
     __shared__ LitScratch ls;
     __shared__ int s_i;
     __shared__ long long s_base;
-    float *dv;
-    int32_t *keys, *aux;
-    uint32_t *vals;
-    unsigned long long *acc;
-    lit_smem(lit_dyn, dv, keys, vals, aux, acc);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int c = lane; c < SACC_CHUNKS; c += 32) acc[w * SACC_CHUNKS + c] = 0ull;
+    const LitTables t = lit_tables(lit_dyn);
     pdl_trigger();
     pdl_wait();
     const uint32_t count = __ldcg(&over[0]);
     for (;;) {
         if (threadIdx.x == 0) {
-            const uint32_t t = atomicAdd(&over[1], 1u);
-            s_i = t < count ? over_list[t] : -1;
+            const uint32_t n = atomicAdd(&over[1], 1u);
+            s_i = n < count ? over_list[n] : -1;
         }
         __syncthreads();
         const int i = s_i;
         __syncthreads();
         if (i < 0) break;
-        LitNode ln;
-        ln.x = a.order[bstart + i];
-        ln.beg = a.off[ln.x];
-        ln.end = a.off[ln.x + 1];
-        ln.d = (int32_t)(ln.end - ln.beg);
-        ln.cx = __ldcg(&a.nmem[ln.x]);
-        long long bound = threadIdx.x == 0 ? ln.cx : 0;
-        for (int64_t q = ln.beg + threadIdx.x; q < ln.end; q += EV_THREADS) bound += __ldcg(&a.nmem[a.adj[q]]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) bound += __shfl_xor_sync(FULL, bound, o);
-        if (lane == 0) ls.part[w] = bound;
-        __syncthreads();
-        bound = 0;
-        for (int k2 = 0; k2 < EV_WARPS; ++k2) bound += ls.part[k2];
-        __syncthreads();
-        if (2 * bound > LB_SLOTS) {   // a table of its own in global memory, if the queue's area has room
-            unsigned long long H = 32;
-            while ((long long)H < 2 * bound) H <<= 1;
-            if (threadIdx.x == 0) {
-                const unsigned long long base = atomicAdd(used, H);
-                s_base = base + H <= a.lg_cap ? (long long)base : -1ll;
-            }
-            __syncthreads();
-            const long long base = s_base;
-            __syncthreads();
-            if (base >= 0) {
-                lit_eval_node<EV_WARPS>(a, i, ln, 1, a.lg_keys + base, a.lg_vals + base, a.lg_aux + base,
-                                        a.lg_dv + base, (uint32_t)H, ls, acc + w * SACC_CHUNKS, 0, w);
-                continue;
-            }
-        }
-        int P = (int)((bound + LIT_PART_ENTRIES - 1) / LIT_PART_ENTRIES);
-        uint32_t Hs = (uint32_t)LB_SLOTS;
-        if (P < 1 || 2 * bound <= LB_SLOTS) {   // one pass over a table of pow2 >= 2 x entries
-            P = 1;
-            Hs = 32;
-            while ((long long)Hs < 2 * bound) Hs <<= 1;
-        }
-        while (!lit_eval_node<EV_WARPS>(a, i, ln, P, keys, vals, aux, dv, Hs, ls, acc + w * SACC_CHUNKS, 0, w)) {
-            Hs = (uint32_t)LB_SLOTS;
-            P *= 2;
-            if (P > (1 << 22)) {   // cannot happen for < 2^31 entries; leave an error, not a loop
-                if (threadIdx.x == 0) atomicOr(&a.ds->err, DERR_CHECK);
-                break;
-            }
-        }
+        lit_big_node(a, bstart, i, t, ls, s_base, used);
     }
 }
 
@@ -3035,29 +3186,28 @@ constexpr int AP_CHUNK = 512;
 // The decision of queue position i, and its pieces of work if it moves.  One thread.
 __device__ __forceinline__ void lit_write_action(const RunArgs &a, int i, int32_t d, const Best &bj, const Best &bl) {
     write_action(a, i, bj, bl, 0ull);
-    if (bj.c < 0 && bl.c < 0) return;
+    if ((bj.c < 0 && bl.c < 0) || !a.items) return;   // the persistent loop's blocks apply their own nodes
     const uint32_t pieces = d > AP_CHUNK ? (uint32_t)(d + AP_CHUNK - 1) / AP_CHUNK : 1u;
     const uint32_t at = atomicAdd(a.nitems, pieces);
     for (uint32_t c = 0; c < pieces; ++c) a.items[at + c] = make_int2(i, (int)c);
 }
 
-__device__ void lit_apply_item(const RunArgs &a, int64_t bstart, int32_t blen, int2 item, uint32_t serial,
-                               unsigned long long &nj, unsigned long long &nl) {
+// One piece of queue position i (node x, neighbours adj[xb, xe)), by one warp.
+__device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, int i, int piece, int32_t x, int64_t xb,
+                                int64_t xe, uint32_t serial, unsigned long long &nj, unsigned long long &nl) {
     const int lane = threadIdx.x & 31;
-    const int i = item.x;
     const int32_t j = __ldcg(&a.act[i]), l = __ldcg(&a.act[a.qcap + i]);
+    if (j < 0 && l < 0) return;
     if (!dbg_ok(a, j < a.nnodes && l < a.nnodes && (j < 0 || j != l))) return;
-    const int32_t x = a.order[bstart + i];
     const int32_t kjoin = __ldcg(&a.act[2 * a.qcap + i]), kl = __ldcg(&a.act[3 * a.qcap + i]);
     int32_t *row = a.mem + (int64_t)x * a.K;
     int32_t *krow = a.kmem + (int64_t)x * a.K;
     const int32_t c = __ldcg(&a.nmem[x]);
-    const int64_t xb = a.off[x], xe = a.off[x + 1];
     const int32_t d = (int32_t)(xe - xb);
     if (!dbg_ok(a, c >= 0 && c <= a.K && (j < 0 || (kjoin >= 0 && kjoin <= d)))) return;
     int jj = 0, jl = 0, ll = 0;
-    const int64_t pe = min(xe, xb + (int64_t)(item.y + 1) * AP_CHUNK);
-    for (int64_t p = xb + (int64_t)item.y * AP_CHUNK + lane; p < pe; p += 32) {
+    const int64_t pe = min(xe, xb + (int64_t)(piece + 1) * AP_CHUNK);
+    for (int64_t p = xb + (int64_t)piece * AP_CHUNK + lane; p < pe; p += 32) {
         const int32_t y = a.adj[p];
         const RowHead ids = row_head8(a.mem, y, a.K);
         const int32_t cy = __ldcg(&a.nmem[y]);
@@ -3214,8 +3364,11 @@ __global__ void __launch_bounds__(AP_THREADS) k_lit_apply(RunArgs a, int64_t bst
     const uint32_t serial = (uint32_t)queue_serial(a, bidx);
     const uint32_t count = __ldcg(a.nitems);
     unsigned long long nj = 0, nl = 0;
-    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < count; t += (gridDim.x * blockDim.x) >> 5)
-        lit_apply_item(a, bstart, blen, __ldcg(&a.items[t]), serial, nj, nl);
+    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < count; t += (gridDim.x * blockDim.x) >> 5) {
+        const int2 item = __ldcg(&a.items[t]);
+        const int32_t x = a.order[bstart + item.x];
+        lit_apply_piece(a, bstart, blen, item.x, item.y, x, a.off[x], a.off[x + 1], serial, nj, nl);
+    }
     flush_counts(a, nj, nl);
 }
 
@@ -3232,6 +3385,7 @@ __global__ void __launch_bounds__(AP_THREADS) k_lit_apply(RunArgs a, int64_t bst
 // 460 -> 111 us; 335k nodes, q 1,024: 23 -> 20 us (cold caches).
 constexpr int LIT_FSUM_GROUP = 64;
 constexpr int LIT_FSUM_WARP = 512;
+constexpr int LIT_FSUM_FEW = 128;    // the same where entries are few
 
 // g_y(n-1), g_y(n), g_y(n+1) added to f0, f1, f2: with D = n - 1 + d - k they are
 // k (k-1) / (d-1) over D-1, D and D+1, so one quotient q = k (k-1) / ((d-1) (D-1) D
@@ -3300,33 +3454,39 @@ struct FsumShared {
     int nbig;
 };
 
-// Entries t0 .. t0 + 4 x warps - 1 of the list, by one block of EV_WARPS warps.
-__device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0, int64_t total, FsumShared &fs) {
+// Entries t0, t0 + step, ... (4 x warps of them) of the list, by one block of
+// EV_WARPS warps.
+__device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0, int64_t step, int64_t total,
+                               FsumShared &fs) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int sub = lane & 7, grp = lane >> 3;
     if (threadIdx.x == 0) fs.nbig = 0;
     __syncthreads();
-    const int64_t t = t0 + 4 * w + grp;
+    // few entries (the longest stride reaches past them): a warp each, the block for
+    // the larger ones; latency counts, not the lanes of the FP64 pipe
+    const bool few = step * EV_WARPS >= total;
+    const int group = few ? -1 : LIT_FSUM_GROUP, warp = few ? LIT_FSUM_FEW : LIT_FSUM_WARP;
+    const int64_t t = t0 + (few ? w : 4 * w + grp) * step;
     int32_t C = 0, n = -1;
-    if (t < total) {
+    if (t < total && (!few || grp == 0)) {
         C = list ? __ldcg(&list[t]) : (int32_t)t;
         n = __ldcg(&a.comm[C].n);
     }
-    {
+    if (!few) {
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-        const bool mine = n >= 0 && n <= LIT_FSUM_GROUP;
+        const bool mine = n >= 0 && n <= group;
         if (mine && n > 0)
             lit_members(a, C, sub, 8, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 8);
         if (mine) lit_fsum_store(a, C, sub, f0, f1, f2);
     }
-    unsigned mid = __ballot_sync(FULL, sub == 0 && n > LIT_FSUM_GROUP);
+    unsigned mid = __ballot_sync(FULL, sub == 0 && n > group);
     while (mid) {
         const int src = __ffs(mid) - 1;
         mid &= mid - 1;
         const int32_t C1 = __shfl_sync(FULL, C, src), n1 = __shfl_sync(FULL, n, src);
-        if (n1 > LIT_FSUM_WARP) {
+        if (n1 > warp) {
             if (lane == 0) fs.big[atomicAdd(&fs.nbig, 1)] = C1;
             continue;
         }
@@ -3365,8 +3525,11 @@ __global__ void __launch_bounds__(EV_THREADS) k_lit_fsum(RunArgs a, const int32_
                                                          int64_t ncount) {
     __shared__ FsumShared fs;
     const int64_t total = list ? (int64_t)__ldcg(count) : ncount;
-    for (int64_t t0 = (int64_t)blockIdx.x * (4 * EV_WARPS); t0 < total; t0 += (int64_t)gridDim.x * (4 * EV_WARPS)) {
-        lit_fsum_block(a, list, t0, total, fs);
+    // a list's first entries go to a block each (short lists spread over the SMs'
+    // FP64 pipes); all communities: neighbours' records to one block
+    const int64_t step = list ? gridDim.x : 1;
+    for (int64_t r = 0; r < total; r += (int64_t)gridDim.x * (4 * EV_WARPS)) {
+        lit_fsum_block(a, list, r + (list ? 1 : 4 * EV_WARPS) * (int64_t)blockIdx.x, step, total, fs);
         __syncthreads();
     }
 }
@@ -3727,6 +3890,102 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_iterate(RunArgs a, int64_t q,
         }
         for (int64_t i = gw; i < blen; i += warps) apply_node(a, bstart, blen, i, serial, nj, nl);
         if (!grid_sync(flags, nblocks, ++epoch, spin_limit, a.ds, &s_ok, bar_mode)) return;
+        if (a.qtimes && blockIdx.x == 0 && threadIdx.x == 0) a.qtimes[b - first + 1] = global_ns();
+    }
+    flush_counts(a, nj, nl);
+}
+
+// ---------------------------------------------------------------------------
+// Persistent queue loop under the paper's gain: one cooperative launch runs
+// queues first .. first + count - 1 of an iteration, each evaluate | apply | member
+// sums of the touched communities, with a grid barrier after each step (a
+// __syncthreads when one block holds the queue: Fox).  A short queue's time is
+// the latency of its chain of dependent loads; per-queue launches add four launch
+// boundaries to it, reload what a block has just had (a block applies the nodes it
+// evaluated, the next queue's static data load while a barrier completes) and
+// read lists to find their work.
+// Only for graphs without hubs (degree above LIT_HUB_DEG), which need the many-block
+// kernels.
+// ---------------------------------------------------------------------------
+struct LitIterShared {
+    LitScratch ls;
+    FsumShared fs;
+    int32_t over[EV_WARPS];
+    int nover, ok;
+    long long base;
+};
+
+template <int T>
+__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, const int64_t *qstart, int64_t q, int64_t first,
+                                                              int64_t count, uint32_t *ctr, unsigned long long *used,
+                                                              long long spin_limit, int inject_stall, unsigned *flags,
+                                                              unsigned epoch, int bar_mode) {
+    extern __shared__ double lit_dyn[];
+    __shared__ LitIterShared sh;
+    const LitTables t = lit_tables(lit_dyn);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int tm = w / T, w_in = w % T;
+    constexpr int TEAMS = EV_WARPS / T;
+    const int64_t round = (int64_t)gridDim.x * TEAMS;
+    unsigned long long nj = 0, nl = 0;
+    if (inject_stall && blockIdx.x == 0 && gridDim.x > 1) return;   // test hook: a block that never arrives
+    auto bounds = [&](int64_t b, int64_t &start, int32_t &len) {
+        start = qstart ? qstart[b] : b * q;
+        len = (int32_t)((qstart ? qstart[b + 1] : min(start + q, a.nnodes)) - start);
+    };
+    auto meet = [&]() {
+        if (gridDim.x == 1) {
+            __syncthreads();
+            return true;
+        }
+        return grid_sync(flags, gridDim.x, ++epoch, spin_limit, a.ds, &sh.ok, bar_mode);
+    };
+    int64_t bstart;
+    int32_t blen;
+    bounds(first, bstart, blen);
+    NodePrefetch pf;
+    const int base0 = (int)blockIdx.x * TEAMS;
+    prefetch_node(a, bstart, blen, base0 + tm, w_in, pf);
+    if (a.qtimes && blockIdx.x == 0 && threadIdx.x == 0) a.qtimes[0] = global_ns();
+    for (int64_t b = first; b < first + count; ++b) {
+        const uint32_t serial = (uint32_t)queue_serial(a, b);
+        a.ntouched = ctr + 4 * b + 2;
+        // evaluate
+        NodePrefetch cur = pf;
+        for (int64_t base = base0; base < blen; base += round) {
+            const int i = (int)base + tm;
+            if (base != base0) prefetch_node(a, bstart, blen, i, w_in, cur);
+            if (threadIdx.x == 0) sh.nover = 0;
+            __syncthreads();
+            if (i < blen && !lit_eval_team<T>(a, i, cur, t, sh.ls, tm, w_in) && w_in == 0 && lane == 0)
+                sh.over[atomicAdd(&sh.nover, 1)] = i;
+            __syncthreads();
+            const int nover = sh.nover;
+            for (int h = 0; h < nover; ++h) lit_big_node(a, bstart, sh.over[h], t, sh.ls, sh.base, used + b);
+        }
+        if (!meet()) return;
+        // apply: each team's first warp, its own nodes
+        for (int64_t base = base0; base < blen; base += round) {
+            const int i = (int)base + tm;
+            if (base != base0) prefetch_node(a, bstart, blen, i, w_in, cur);
+            else cur = pf;
+            if (i >= blen || w_in != 0) continue;
+            for (int piece = 0; piece == 0 || piece * AP_CHUNK < cur.d; ++piece)
+                lit_apply_piece(a, bstart, blen, i, piece, cur.x, cur.beg, cur.end, serial, nj, nl);
+        }
+        // the next queue's static data load while the barrier completes
+        const bool more = b + 1 < first + count;
+        if (more) {
+            bounds(b + 1, bstart, blen);
+            prefetch_node(a, bstart, blen, base0 + tm, w_in, pf);
+        }
+        if (!meet()) return;
+        const int64_t total = __ldcg(a.ntouched);
+        for (int64_t r = 0; r < total; r += (int64_t)gridDim.x * (4 * EV_WARPS)) {
+            lit_fsum_block(a, a.touched, r + blockIdx.x, gridDim.x, total, sh.fs);
+            __syncthreads();
+        }
+        if (more && !meet()) return;
         if (a.qtimes && blockIdx.x == 0 && threadIdx.x == 0) a.qtimes[b - first + 1] = global_ns();
     }
     flush_counts(a, nj, nl);
@@ -4441,6 +4700,12 @@ void free_lit_hub_plan(lf_graph *g) {
     g->lh_plan_K = 0;
 }
 
+// Queues up to this size run in the persistent loop under the paper's gain: one
+// block and no grid barrier at queue size 1. Measured, us a queue, loop / launches:
+// 1,000 nodes (planted) q 1 13.0 / 18.1, q 4 19.8 / 21.3, q 16 22.9 / 24.3; 84k nodes
+// q 16 18.3 / 18.8, q 64 25.2 / 24.1, q 256 36.1 / 30.1.
+constexpr int64_t LIT_LOOP_MAX_Q = 16;
+
 // The hubs of every queue (degree > LIT_HUB_DEG): worst-case tables of
 // pow2 >= 2 (d+1) K slots (K bounds every row), fill items of LH_CHUNK
 // neighbours, slot items of LH_SLOTS slots.  Queues run one after the other,
@@ -4612,7 +4877,7 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         const int64_t longest = g->max_deg / AP_CHUNK + 1;   // pieces of one node at most
         const unsigned ag = grid_for((int64_t)blen * longest * 32, AP_THREADS, 6 * (int64_t)num_sms());
         launch_pdl(k_lit_apply, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
-        k_lit_fsum<<<(unsigned)std::min<int64_t>((2 * (int64_t)blen + 31) / 32, 8 * (int64_t)num_sms()), EV_THREADS, 0,
+        k_lit_fsum<<<(unsigned)std::min<int64_t>(2 * (int64_t)blen, 4 * (int64_t)num_sms()), EV_THREADS, 0,
                      g->stream>>>(ab, g->touched, ctr + 2, 0);
         g->launches += 4;
     }
@@ -4899,6 +5164,50 @@ void launch_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int64_t
     void *args[] = {&a, &q, &first, &count, &spin, &inject, &flags, &epoch, &bar_mode};
     if (e0) LF_CUDA(cudaEventRecord(e0, g->stream));
     LF_CUDA(cudaLaunchCooperativeKernel(iterate_kernel_for(T), dim3(grid), dim3(EV_THREADS), args, EV_DYN_SMEM,
+                                        g->stream));
+    ++g->launches;
+    if (e1) LF_CUDA(cudaEventRecord(e1, g->stream));
+}
+
+const void *lit_iterate_kernel_for(int T) {
+    switch (T) {
+    case 1: return (const void *)k_lit_iterate<1>;
+    case 2: return (const void *)k_lit_iterate<2>;
+    case 4: return (const void *)k_lit_iterate<4>;
+    default: return (const void *)k_lit_iterate<8>;
+    }
+}
+
+int lit_persistent_grid_max(int T) {
+    int per_sm = 0;
+    const void *k = lit_iterate_kernel_for(T);
+    LF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, EV_THREADS, LIT_SMEM));
+    return std::max(1, per_sm) * num_sms();
+}
+
+// One cooperative launch runs queues first .. first+count-1 under the paper's gain.
+void launch_lit_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int64_t count, int grid_max, int T,
+                           cudaEvent_t e0, cudaEvent_t e1) {
+    if (count <= 0) return;
+    const int64_t teams = EV_WARPS / T;
+    const int64_t want = (q + teams - 1) / teams;
+    unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, grid_max));
+    long long spin = (long long)g->barrier_timeout_ms * 4000ll;   // >= ~250 ns per poll of the flags
+    int inject = g->inject_stall;
+    unsigned *flags = g->bar_flags;
+    unsigned epoch = g->bar_epoch;
+    g->bar_epoch += (unsigned)(3 * count);
+    int bar_mode = g->barrier_mode;
+    uint32_t *ctr = g->lit_ctr;
+    unsigned long long *used = g->lit_used;
+    const int64_t *qstart = nullptr;
+    a.items = nullptr;
+    LF_CUDA(cudaMemsetAsync(ctr + 4 * first, 0, (size_t)(4 * count) * sizeof(uint32_t), g->stream));
+    LF_CUDA(cudaMemsetAsync(used + first, 0, (size_t)count * sizeof(unsigned long long), g->stream));
+    void *args[] = {&a, &qstart, &q, &first, &count, &ctr, &used, &spin, &inject, &flags, &epoch, &bar_mode};
+    if (e0) LF_CUDA(cudaEventRecord(e0, g->stream));
+    LF_CUDA(cudaLaunchCooperativeKernel(lit_iterate_kernel_for(T), dim3(grid), dim3(EV_THREADS), args, LIT_SMEM,
                                         g->stream));
     ++g->launches;
     if (e1) LF_CUDA(cudaEventRecord(e1, g->stream));
@@ -5345,9 +5654,11 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
     else if (!lit && use_dyn(g, q)) ensure_dyn(g, q, nb);
     // measured on GB300: the persistent loop wins for small queues (grid
     // barriers over few blocks), launches per queue for large ones
-    const bool persistent = !batch && !lit && (g->per_queue == 0 || (g->per_queue < 0 && q <= 256));
+    const bool loop_ok = !batch && (!lit || g->max_deg <= LIT_HUB_DEG);
+    const bool persistent =
+        loop_ok && (g->per_queue == 0 || (g->per_queue < 0 && q <= (lit ? LIT_LOOP_MAX_Q : 256)));
     const int team = choose_team(g, q);
-    const int grid_max = persistent ? persistent_grid_max(g, team) : 0;
+    const int grid_max = !persistent ? 0 : lit ? lit_persistent_grid_max(team) : persistent_grid_max(g, team);
     if (persistent) {
         if (g->bar_flags_cap < grid_max + 1) {
             if (g->bar_flags) dfree(g, g->bar_flags);
@@ -5389,7 +5700,9 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
         if (lit) lit_iteration_start(g, a);
         const bool partial = max_batches >= 0 && batches + nb > max_batches;
         if (partial) {
-            if (persistent) launch_persistent(g, a, q, 0, max_batches - batches, grid_max, team, nullptr, nullptr);
+            if (persistent && lit)
+                launch_lit_persistent(g, a, q, 0, max_batches - batches, grid_max, team, nullptr, nullptr);
+            else if (persistent) launch_persistent(g, a, q, 0, max_batches - batches, grid_max, team, nullptr, nullptr);
             else if (lit) launch_batches_lit(g, a, q, 0, max_batches - batches);
             else launch_batches(g, a, q, 0, max_batches - batches);
             batches = max_batches;
@@ -5400,7 +5713,8 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
             break;
         }
         if (persistent) {
-            launch_persistent(g, a, q, 0, nb, grid_max, team, pev[0], pev[1]);
+            if (lit) launch_lit_persistent(g, a, q, 0, nb, grid_max, team, pev[0], pev[1]);
+            else launch_persistent(g, a, q, 0, nb, grid_max, team, pev[0], pev[1]);
             launch_iteration_end(g, a);
         } else if (g->use_graphs > 0 && max_batches < 0) {
             if (!g->iter_exec || g->graph_q != q || g->graph_K != g->K || g->graph_sched != g->sched_version ||
