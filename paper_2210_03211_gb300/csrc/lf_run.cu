@@ -1827,7 +1827,7 @@ constexpr int LW = 512;                            // table slots of one warp
 constexpr int LB_SLOTS = EV_WARPS * LW;            // table slots of a block
 constexpr uint32_t SURV_FLAG = 0x40000000u;        // candidate survives the bracket test
 constexpr uint32_t CNT_MASK = 0x3fffffffu;
-constexpr size_t LIT_SMEM = (size_t)LB_SLOTS * 16 + (size_t)EV_WARPS * SACC_CHUNKS * 8;
+constexpr size_t LIT_SMEM = (size_t)LB_SLOTS * 16 + (size_t)EV_WARPS * SACC_CHUNKS * 8 + (size_t)LB_SLOTS;   // tables, accumulators, candidate lists
 constexpr int LIT_PART_ENTRIES = 1024;             // entries per pass of a multi-pass node
 
 // Signed exact accumulation: like sacc_add, with negative values added as
@@ -2038,28 +2038,31 @@ __device__ __forceinline__ bool adj_has(const int32_t *adj, int64_t beg, int64_t
 // and x's own g, in FP32 (about ten roundings each, relative error
 // < 16 x 2^-24; a sum of k of them adds k roundings): used only in the
 // bracket, whose bound E carries a term for them.
-__device__ __forceinline__ float lit_h_join32(int64_t k, int64_t d, int64_t n) {
+// (All arguments are below 2^31 with k <= d, so every sum here fits in 32
+// unsigned bits and converts in one instruction.)
+__device__ __forceinline__ float lit_h_join32(uint32_t k, uint32_t d, uint32_t n) {
     if (d < 2 || k < 1) return 0.f;
-    const float D = (float)(n + d - k), kf = (float)k, df = (float)d;
+    const float D = __uint2float_rn(n + (d - k)), kf = __uint2float_rn(k), df = __uint2float_rn(d);
     const float bk = 0.5f * (kf * (kf - 1.f));
     const float bd = 0.5f * (df * (df - 1.f));
     return (df * (kf * D + bk)) / (bd * (D * (D - 1.f)));
 }
 
-__device__ __forceinline__ float lit_h_leave32(int64_t k, int64_t d, int64_t n) {
+__device__ __forceinline__ float lit_h_leave32(uint32_t k, uint32_t d, uint32_t n) {
     if (d < 2 || k < 2 || n < 3) return 0.f;
-    const float D = (float)(n - 2 + d - k), kf = (float)k, df = (float)d;
+    const float D = __uint2float_rn(n - 2 + (d - k)), kf = __uint2float_rn(k), df = __uint2float_rn(d);
     const float bk1 = 0.5f * ((kf - 1.f) * (kf - 2.f));
     const float bd = 0.5f * (df * (df - 1.f));
     return -(df * (bk1 + (kf - 1.f) * (D + 1.f))) / (bd * (D * (D + 1.f)));
 }
 
-__device__ __forceinline__ float lit_g32(int64_t k, int64_t d, int64_t nu) {
+// nu: n + 1 or n - 1 (never below 0); zero where nu - 1 + d - k <= 0.
+__device__ __forceinline__ float lit_g32(uint32_t k, uint32_t d, uint32_t nu) {
     if (k < 2 || d < 2) return 0.f;
-    const int64_t den = nu - 1 + d - k;
-    if (den <= 0) return 0.f;
-    const float kf = (float)k, df = (float)d;
-    return (0.5f * (kf * (kf - 1.f)) * df) / (0.5f * (df * (df - 1.f)) * (float)den);
+    const uint32_t den1 = nu + (d - k);
+    if (den1 <= 1) return 0.f;
+    const float kf = __uint2float_rn(k), df = __uint2float_rn(d);
+    return (0.5f * (kf * (kf - 1.f)) * df) / (0.5f * (df * (df - 1.f)) * __uint2float_rn(den1 - 1));
 }
 
 // Bracket of one candidate: FP64 value X of the expression above and a bound
@@ -2069,22 +2072,22 @@ __device__ __forceinline__ void lit_screen(const RunArgs &a, int32_t C, uint32_t
     // per community (k_lit_fsum, rounded to float): F(n-1), F(n+1),
     // WCC-hat(C) = p/cc F(n), 1/((n+1) n cc), 1/((n-1)(n-2) cc)
     const bool own = (v & OWN_FLAG) != 0;
-    const int64_t k = (int64_t)(v & CNT_MASK);
+    const uint32_t k = v & CNT_MASK;
     const int4 r = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C]));
-    const int64_t n = r.x;
+    const uint32_t n = (uint32_t)r.x;
     const float m2 = (float)(uint32_t)r.y;
     const float *fp = a.litF + 8 * (int64_t)C;
     const float4 f = __ldcg(reinterpret_cast<const float4 *>(fp));
     float A, S1, Sm, Eh;
     if (!own) {
         A = (m2 + 2.f * (float)k) * f.w;
-        const float gx = lit_g32(k, d, n + 1);
+        const float gx = lit_g32(k, (uint32_t)d, n + 1u);
         S1 = (f.y + Hs) + gx;
         Sm = S1;
         Eh = Hs + gx;
     } else {
         A = (m2 - 2.f * (float)k) * __ldcg(&fp[4]);
-        const float gx = A != 0.f ? lit_g32(k, d, n - 1) : 0.f;
+        const float gx = A != 0.f ? lit_g32(k, (uint32_t)d, n - 1u) : 0.f;
         S1 = (f.x - gx) + Hs;
         Sm = (f.x + gx) - Hs;
         Eh = gx - Hs;
@@ -2114,22 +2117,34 @@ __device__ __forceinline__ void lit_screen(const RunArgs &a, int32_t C, uint32_t
 // not depend on how the entries spread over its neighbours.  fn(C, ky, dy,
 // n): the community, deg(y,C), deg(y) and C's size before the queue.
 // Every lane of the warp must call this with the same range.
-template <typename Fn>
+//
+// Bound by the latency of three dependent gathers (counts, rows, sizes) at few
+// warps per SM, so the gathers are kept in flight: the ids of the 32 neighbours
+// after next and the counts of the next ones load while these are handled, and
+// R rounds of rows, then of sizes, are issued before the first is used.
+// Mean of k_lit_eval over the queues, with the lists of lit_eval_shared: 3.07M nodes,
+// q 65,536: 530 -> 379 us; 767k nodes, q 16,384: 140 -> 106 us; 335k nodes, q 1,024:
+// 27.6 -> 21.7 us (cold caches).
+template <int R, typename Fn>
 __device__ __forceinline__ void lit_warp_entries(const RunArgs &a, int64_t qb, int64_t qe, unsigned long long &pb,
                                                  bool count_bytes, Fn &&fn) {
     const int lane = threadIdx.x & 31;
-    for (int64_t q0 = qb; q0 < qe; q0 += 32) {
-        const int64_t q = q0 + lane;
-        int32_t y = 0, cy = 0, dy = 0;
-        if (q < qe) {
-            y = a.adj[q];
-            if (dbg_ok(a, y >= 0 && y < a.nnodes)) {
-                cy = __ldcg(&a.nmem[y]);
-                if (!dbg_ok(a, cy >= 0 && cy <= a.K)) cy = 0;
-                dy = a.deg[y];
-                if (count_bytes) pb += 12ull + 8ull * (unsigned long long)cy;
-            }
+    auto id_at = [&](int64_t q) { return q < qe ? a.adj[q] : -1; };
+    auto counts = [&](int32_t y, int32_t &cy, int32_t &dy) {
+        cy = dy = 0;
+        if (y >= 0 && dbg_ok(a, y < a.nnodes)) {
+            cy = __ldcg(&a.nmem[y]);
+            dy = a.deg[y];
         }
+    };
+    int32_t y = id_at(qb + lane), ynext = id_at(qb + 32 + lane), cy, dy;
+    counts(y, cy, dy);
+    for (int64_t q0 = qb; q0 < qe; q0 += 32) {
+        const int32_t yafter = id_at(q0 + 64 + lane);
+        int32_t cnext, dnext;
+        counts(ynext, cnext, dnext);
+        if (!dbg_ok(a, cy >= 0 && cy <= a.K)) cy = 0;
+        if (count_bytes && y >= 0) pb += 12ull + 8ull * (unsigned long long)cy;
         int inc = cy;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -2137,22 +2152,40 @@ __device__ __forceinline__ void lit_warp_entries(const RunArgs &a, int64_t qb, i
             if (lane >= o) inc += t;
         }
         const int total = __shfl_sync(FULL, inc, 31);
-        for (int e0 = 0; e0 < total; e0 += 32) {
-            const int e = e0 + lane;
-            int j = 0;   // first lane whose inclusive prefix exceeds e
+        for (int e0 = 0; e0 < total; e0 += 32 * R) {
+            int32_t C[R], ky[R], dj[R], n[R];
 #pragma unroll
-            for (int b = 16; b > 0; b >>= 1)
-                if (__shfl_sync(FULL, inc, j + b - 1) <= e) j += b;
-            const int32_t yj = __shfl_sync(FULL, y, j);
-            const int32_t first = __shfl_sync(FULL, inc - cy, j);
-            const int32_t dj = __shfl_sync(FULL, dy, j);
-            if (e < total) {
-                const int64_t rb = (int64_t)yj * a.K + (e - first);
-                const int32_t C = __ldcg(&a.mem[rb]);
-                const int32_t ky = __ldcg(&a.kmem[rb]);
-                if (dbg_ok(a, C >= 0 && C < a.nnodes)) fn(C, (int64_t)ky, (int64_t)dj, (int64_t)__ldcg(&a.comm[C].n));
+            for (int u = 0; u < R; ++u) {
+                C[u] = -1;
+                if (e0 + 32 * u >= total) continue;   // the whole warp
+                const int e = e0 + 32 * u + lane;
+                int j = 0;   // first lane whose inclusive prefix exceeds e
+#pragma unroll
+                for (int b = 16; b > 0; b >>= 1)
+                    if (__shfl_sync(FULL, inc, j + b - 1) <= e) j += b;
+                const int32_t yj = __shfl_sync(FULL, y, j);
+                const int32_t first = __shfl_sync(FULL, inc - cy, j);
+                dj[u] = __shfl_sync(FULL, dy, j);
+                if (e < total) {
+                    const int64_t rb = (int64_t)yj * a.K + (e - first);
+                    C[u] = __ldcg(&a.mem[rb]);
+                    ky[u] = __ldcg(&a.kmem[rb]);
+                }
             }
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                if (e0 + 32 * u + lane < total && !dbg_ok(a, C[u] >= 0 && C[u] < a.nnodes && ky[u] >= 0 && ky[u] <= dj[u]))
+                    C[u] = -1;
+                n[u] = C[u] >= 0 ? __ldcg(&a.comm[C[u]].n) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < R; ++u)
+                if (C[u] >= 0) fn(C[u], (uint32_t)ky[u], (uint32_t)dj[u], (uint32_t)n[u]);
         }
+        y = ynext;
+        cy = cnext;
+        dy = dnext;
+        ynext = yafter;
     }
 }
 
@@ -2160,10 +2193,22 @@ __device__ __forceinline__ void lit_warp_entries(const RunArgs &a, int64_t qb, i
 // and its joiners since, in C's region and, past its capacity, in C's list --
 // handed to f, entry t to thread `tid` of `nthreads` when t % nthreads == tid.
 // Entries of nodes that left C since are included (f checks the row).
+struct MemberRange {
+    int64_t b0, cap, used;
+};
+
+__device__ __forceinline__ MemberRange lit_member_range(const RunArgs &a, int32_t C) {
+    MemberRange r;
+    r.b0 = (int64_t)a.cm_off[C];
+    r.cap = (int64_t)a.cm_off[C + 1] - r.b0;
+    r.used = (int64_t)__ldcg(&a.cm_cnt[C]);
+    return r;
+}
+
 template <typename F>
-__device__ __forceinline__ void lit_members(const RunArgs &a, int32_t C, int tid, int nthreads, F &&f) {
-    const int64_t b0 = (int64_t)a.cm_off[C], cap = (int64_t)a.cm_off[C + 1] - b0;
-    const int64_t used = (int64_t)__ldcg(&a.cm_cnt[C]);
+__device__ __forceinline__ void lit_members(const RunArgs &a, int32_t C, const MemberRange &r, int tid, int nthreads,
+                                            F &&f) {
+    const int64_t b0 = r.b0, cap = r.cap, used = r.used;
     const int64_t b1 = b0 + (used < cap ? used : cap);
     for (int64_t p = b0 + tid; p < b1; p += nthreads) f(__ldcg(&a.cm_node[p]));
     if (used > cap) {
@@ -2204,6 +2249,7 @@ __device__ double lit_exact_gain(const RunArgs &a, int32_t x, int32_t d, int32_t
     const int tid = block ? (int)threadIdx.x : lane, nthreads = block ? (int)blockDim.x : 32;
     unsigned long long *wacc = block ? acc + (threadIdx.x >> 5) * SACC_CHUNKS : acc;
     const int4 r = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C]));
+    const MemberRange mr = lit_member_range(a, C);
     const int64_t n0 = r.x;
     const uint32_t m20 = (uint32_t)r.y;
     const double cc = a.gcc ? a.gcc[r.w] : a.cc;
@@ -2231,8 +2277,7 @@ __device__ double lit_exact_gain(const RunArgs &a, int32_t x, int32_t d, int32_t
         before = wcchat_term(ky, dy, n0, p0, cc);
     };
     {
-        const int64_t b0 = (int64_t)a.cm_off[C], cap = (int64_t)a.cm_off[C + 1] - b0;
-        const int64_t used = (int64_t)__ldcg(&a.cm_cnt[C]);
+        const int64_t b0 = mr.b0, cap = mr.cap, used = mr.used;
         const int64_t b1 = b0 + (used < cap ? used : cap);
         for (int64_t q0 = b0 + (tid - lane); q0 < b1; q0 += nthreads) {   // a warp's lanes stay together
             double after = 0.0, before = 0.0;
@@ -2277,6 +2322,8 @@ __device__ double lit_exact_gain(const RunArgs &a, int32_t x, int32_t d, int32_t
 
 __device__ __forceinline__ void lit_write_action(const RunArgs &a, int i, int32_t d, const Best &bj, const Best &bl);
 
+constexpr int SURV_LIST = 32;
+
 // Per-warp values a literal team exchanges.
 struct LitScratch {
     float lbj[EV_WARPS], lbl[EV_WARPS];
@@ -2287,6 +2334,10 @@ struct LitScratch {
     int32_t bcj[EV_WARPS], bcl[EV_WARPS], bkj[EV_WARPS], bkl[EV_WARPS];
     int flag[EV_WARPS];
     long long part[EV_WARPS];
+    // per team: candidates listed, survivors of the bracket (all, joins, leaves),
+    // and the slots of the first SURV_LIST of them
+    int ncand[EV_WARPS], ns[EV_WARPS], nsj[EV_WARPS], nsl[EV_WARPS];
+    uint16_t surv[EV_WARPS][SURV_LIST];
 };
 
 struct LitNode {
@@ -2342,9 +2393,9 @@ __device__ __forceinline__ void lit_screen_table(const RunArgs &a, int32_t d, in
 // dv <- X, aux <- E (as a float rounded up).  Per lane: the largest lower
 // ends of the two kinds.  Returns false (team-wide) if the table overflowed.
 template <int T>
-__device__ bool lit_pass(const RunArgs &a, const LitNode &ln, int P, int p, int32_t *keys, uint32_t *vals,
-                         int32_t *aux, float *dv, uint32_t H, LitScratch &ls, int tm, int w_in, float &lbj,
-                         float &lbl, unsigned long long &pb, bool count_bytes) {
+__device__ __forceinline__ bool lit_fill(const RunArgs &a, const LitNode &ln, int P, int p, int32_t *keys, uint32_t *vals,
+                                         int32_t *aux, uint32_t H, LitScratch &ls, int tm, int w_in,
+                                         unsigned long long &pb, bool count_bytes) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int tl = w_in * 32 + lane;
     constexpr int NT = T * 32;
@@ -2366,9 +2417,8 @@ __device__ bool lit_pass(const RunArgs &a, const LitNode &ln, int P, int p, int3
     {   // each warp of the team takes a contiguous share of the neighbours
         const int64_t deg = ln.end - ln.beg, per = (deg + T - 1) / T;
         const int64_t qb = ln.beg + min(deg, (int64_t)w_in * per), qe = ln.beg + min(deg, (int64_t)(w_in + 1) * per);
-        lit_warp_entries(a, qb, qe, pb, count_bytes, [&](int32_t C, int64_t ky, int64_t dy, int64_t n) {
+        lit_warp_entries<T == EV_WARPS ? 2 : 4>(a, qb, qe, pb, count_bytes, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
             if (P > 1 && (int)part_of(C, P) != p) return;
-            if (!dbg_ok(a, ky >= 0 && ky <= dy)) return;
             const int slot = lit_insert(keys, vals, hm, C);
             if (slot < 0) {
                 ok = false;
@@ -2388,7 +2438,14 @@ __device__ bool lit_pass(const RunArgs &a, const LitNode &ln, int P, int p, int3
     } else {
         ok = __all_sync(FULL, ok);
     }
-    if (!ok) return false;
+    return ok;
+}
+
+template <int T>
+__device__ bool lit_pass(const RunArgs &a, const LitNode &ln, int P, int p, int32_t *keys, uint32_t *vals,
+                         int32_t *aux, float *dv, uint32_t H, LitScratch &ls, int tm, int w_in, float &lbj,
+                         float &lbl, unsigned long long &pb, bool count_bytes) {
+    if (!lit_fill<T>(a, ln, P, p, keys, vals, aux, H, ls, tm, w_in, pb, count_bytes)) return false;
     lit_screen_table<T>(a, ln.d, keys, vals, aux, dv, H, tm, w_in, lbj, lbl, pb, count_bytes);
     return true;
 }
@@ -2578,30 +2635,148 @@ __device__ __forceinline__ void lit_finish(const RunArgs &a, int i, const LitNod
     team_sync<T>(tm);
 }
 
-// The decision from one bracketed table (all candidates in it): survivors,
-// their exact gains where the bracket cannot tell, the action written.
-template <int T>
-__device__ __forceinline__ void lit_decide(const RunArgs &a, int i, const LitNode &ln, int32_t *keys, uint32_t *vals,
-                                           const int32_t *aux, const float *dv, uint32_t H, float lbj, float lbl,
-                                           LitScratch &ls, unsigned long long *acc, int tm, int w_in,
-                                           unsigned long long pb) {
+// One shared table that holds all candidates, screened and decided over the
+// list of its used slots: tables are at most half full and mostly far emptier, and
+// a scan of the slots left most lanes idle and, worse, gave a warp one dependent
+// gather of the communities' records per 32 slots; over the list it is one per 32
+// candidates.
+struct LitTable {
+    int32_t *keys, *aux;
+    uint32_t *vals;
+    float *dv;
+    uint16_t *list;
+};
+
+// The used slots listed by one warp of the NW that share the table (ls.ncand[tm]
+// zero before).
+template <int NW>
+__device__ __forceinline__ void lit_collect(const LitTable &t, uint32_t H, LitScratch &ls, int tm, int w_in) {
     const int lane = threadIdx.x & 31;
-    int cj = 0, cl = 0;
-    int32_t Cj = -1, Cl = -1, kj = 0, kl = 0;
-    float Lj = 0.f, Ll = 0.f;
-    lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, cj, cl, Cj, Cl, kj, kl, Lj, Ll);
+    int n = 0;
+    for (uint32_t b0 = (uint32_t)w_in * 32; b0 < H; b0 += NW * 32) {
+        const bool used = t.keys[b0 + lane] != EMPTY_KEY;   // H is a multiple of 32
+        const unsigned m = __ballot_sync(FULL, used);
+        if constexpr (NW > 1) {
+            if (lane == 0) n = m ? atomicAdd(&ls.ncand[tm], __popc(m)) : 0;
+            n = __shfl_sync(FULL, n, 0);
+        }
+        if (used) t.list[n + __popc(m & lanemask_lt())] = (uint16_t)(b0 + lane);
+        if constexpr (NW == 1) n += __popc(m);
+    }
+    if constexpr (NW == 1)
+        if (lane == 0) ls.ncand[tm] = n;
+}
+
+// Brackets of the listed candidates (threads tl of NT), and this lane's largest lower ends.
+template <int NT>
+__device__ __forceinline__ void lit_screen_list(const RunArgs &a, int32_t d, const LitTable &t, int ncand, int tl,
+                                                float &lbj, float &lbl, unsigned long long &pb) {
+    const float *hs = reinterpret_cast<const float *>(t.aux);
+    for (int c = tl; c < ncand; c += NT) {
+        const int s = t.list[c];
+        const uint32_t v = t.vals[s];
+        float X, E;
+        lit_screen(a, t.keys[s], v, d, hs[s], X, E);
+        t.dv[s] = X;
+        t.aux[s] = __float_as_int(E);
+        if (v & OWN_FLAG) lbl = fmaxf(lbl, X - E);
+        else lbj = fmaxf(lbj, X - E);
+        if (a.profile) {
+            pb += 40ull;
+            atomicAdd(&a.ds->prof_cands, 1ull);
+        }
+    }
+}
+
+// Survivors of the bracket test marked, counted and listed (counters zero before).
+template <int NT>
+__device__ __forceinline__ void lit_mark_list(const RunArgs &a, const LitTable &t, int ncand, int tl, float lbj, float lbl,
+                                              LitScratch &ls, int tm) {
+    for (int c = tl; c < ncand; c += NT) {
+        const int s = t.list[c];
+        const uint32_t v = t.vals[s];
+        const float U = t.dv[s] + __int_as_float(t.aux[s]);
+        const bool own = (v & OWN_FLAG) != 0;
+        if (!a.screen || (U > 0.f && U >= (own ? lbl : lbj))) {
+            t.vals[s] = v | SURV_FLAG;
+            const int e = atomicAdd(&ls.ns[tm], 1);
+            if (e < SURV_LIST) ls.surv[tm][e] = (uint16_t)s;
+            atomicAdd(own ? &ls.nsl[tm] : &ls.nsj[tm], 1);
+        }
+    }
+}
+
+// The decision from the survivors, all T warps of the team: none, a lone one
+// whose lower end is positive, or the best of their exact gains, a survivor
+// per warp at a time.
+template <int T>
+__device__ __forceinline__ void lit_resolve(const RunArgs &a, int i, const LitNode &ln, const LitTable &t, LitScratch &ls,
+                                            unsigned long long *acc, int tm, int w_in, unsigned long long pb) {
+    const int lane = threadIdx.x & 31;
+    const int ns = ls.ns[tm], nj = ls.nsj[tm], nl = ls.nsl[tm];
     Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
-    const bool do_j = lit_settle(a, cj, Cj, kj, Lj, bj), do_l = lit_settle(a, cl, Cl, kl, Ll, bl);
+    bool do_j = nj > 0, do_l = nl > 0;
+    if (a.screen && ns <= SURV_LIST && (nj == 1 || nl == 1)) {
+        const int s = lane < ns ? ls.surv[tm][lane] : 0;
+        const uint32_t v = lane < ns ? t.vals[s] : 0u;
+        const float L = lane < ns ? t.dv[s] - __int_as_float(t.aux[s]) : 0.f;
+        const int32_t C = lane < ns ? t.keys[s] : 0;
+        const unsigned ml = __ballot_sync(FULL, lane < ns && (v & OWN_FLAG)), mj = __ballot_sync(FULL, lane < ns && !(v & OWN_FLAG));
+        if (nj == 1) do_j = lit_settle(a, 1, __shfl_sync(FULL, C, __ffs(mj) - 1),
+                                       (int32_t)(__shfl_sync(FULL, v, __ffs(mj) - 1) & CNT_MASK),
+                                       __shfl_sync(FULL, L, __ffs(mj) - 1), bj);
+        if (nl == 1) do_l = lit_settle(a, 1, __shfl_sync(FULL, C, __ffs(ml) - 1),
+                                       (int32_t)(__shfl_sync(FULL, v, __ffs(ml) - 1) & CNT_MASK),
+                                       __shfl_sync(FULL, L, __ffs(ml) - 1), bl);
+    }
     if (do_j || do_l) {
-        lit_exact_survivors<T>(a, ln, keys, vals, H, do_j, do_l, acc, w_in, bj, bl);
-        team_sync<T>(tm);
+        const int count = ns <= SURV_LIST ? ns : ls.ncand[tm];
+        for (int e = w_in; e < count; e += T) {
+            const int s = ns <= SURV_LIST ? ls.surv[tm][e] : t.list[e];
+            const uint32_t v = t.vals[s];
+            const bool own = (v & OWN_FLAG) != 0;
+            if (!(v & SURV_FLAG) || !(own ? do_l : do_j)) continue;
+            const int32_t C = t.keys[s];
+            const int64_t k = (int64_t)(v & CNT_MASK);
+            const double g = lit_exact_gain(a, ln.x, ln.d, C, own, k, acc);
+            if (a.profile && lane == 0) atomicAdd(&a.ds->prof_exact, 1ull);
+            if (g > 0.0) {
+                Best &b = own ? bl : bj;
+                if (better(g, C, b.g, b.c)) b = Best{g, C, (int32_t)k};
+            }
+        }
         lit_team_best<T>(ls, tm, w_in, bj, bl);
     }
     lit_finish<T>(a, i, ln, bj, bl, tm, w_in, pb);
 }
 
-// A node's decision with the paper's gain, by a team of T warps over a table
-// of H slots (P parts of the candidates, one pass each).  False if a part
+__device__ __forceinline__ void lit_zero_counts(LitScratch &ls, int tm) {
+    ls.ncand[tm] = ls.ns[tm] = ls.nsj[tm] = ls.nsl[tm] = 0;
+}
+
+// A node's decision over one shared table (H >= 2 x its entries) by a team of T
+// warps.
+template <int T>
+__device__ __forceinline__ bool lit_eval_shared(const RunArgs &a, int i, const LitNode &ln, const LitTable &t, uint32_t H,
+                                                LitScratch &ls, unsigned long long *acc, int tm, int w_in) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long pb = 0;
+    float lbj = -INFINITY, lbl = -INFINITY;
+    if (w_in == 0 && lane == 0) lit_zero_counts(ls, tm);
+    if (!lit_fill<T>(a, ln, 1, 0, t.keys, t.vals, t.aux, H, ls, tm, w_in, pb, a.profile != 0)) return false;
+    lit_collect<T>(t, H, ls, tm, w_in);
+    team_sync<T>(tm);
+    const int ncand = ls.ncand[tm];
+    lit_screen_list<T * 32>(a, ln.d, t, ncand, w_in * 32 + lane, lbj, lbl, pb);
+    team_max2<T>(ls, tm, lbj, lbl);
+    lit_mark_list<T * 32>(a, t, ncand, w_in * 32 + lane, lbj, lbl, ls, tm);
+    team_sync<T>(tm);
+    lit_resolve<T>(a, i, ln, t, ls, acc, tm, w_in, pb);
+    return true;
+}
+
+// A node's decision with the paper's gain, by a team of T warps over a table in
+// global memory, or over a shared one in P parts of the candidates, a pass each.  False if a part
 // overflowed the table (the caller retries with more parts).
 template <int T>
 __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P, int32_t *keys, uint32_t *vals,
@@ -2613,27 +2788,26 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
         if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, a.profile != 0))
             return false;
     team_max2<T>(ls, tm, lbj, lbl);
-    if (P == 1) {
-        lit_decide<T>(a, i, ln, keys, vals, aux, dv, H, lbj, lbl, ls, acc, tm, w_in, pb);
-        return true;
-    }
     int cj = 0, cl = 0;
     int32_t Cj = -1, Cl = -1, kj = 0, kl = 0;
     float Lj = 0.f, Ll = 0.f;
     for (int p = 0; p < P; ++p) {
-        if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, false)) return false;
+        if (P > 1 && !lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, lbj, lbl, pb, false))
+            return false;
         lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, cj, cl, Cj, Cl, kj, kl, Lj, Ll);
     }
     Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
     const bool do_j = lit_settle(a, cj, Cj, kj, Lj, bj), do_l = lit_settle(a, cl, Cl, kl, Ll, bl);
     if (do_j || do_l) {
         for (int p = 0; p < P; ++p) {
-            float d1 = -INFINITY, d2 = -INFINITY;
-            if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, d1, d2, pb, false)) return false;
-            int c1 = 0, c2 = 0;
-            int32_t e1 = -1, e2 = -1, e3 = 0, e4 = 0;
-            float e5 = 0.f, e6 = 0.f;
-            lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, c1, c2, e1, e2, e3, e4, e5, e6);
+            if (P > 1) {
+                float d1 = -INFINITY, d2 = -INFINITY;
+                if (!lit_pass<T>(a, ln, P, p, keys, vals, aux, dv, H, ls, tm, w_in, d1, d2, pb, false)) return false;
+                int c1 = 0, c2 = 0;
+                int32_t e1 = -1, e2 = -1, e3 = 0, e4 = 0;
+                float e5 = 0.f, e6 = 0.f;
+                lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, c1, c2, e1, e2, e3, e4, e5, e6);
+            }
             lit_exact_survivors<T>(a, ln, keys, vals, H, do_j, do_l, acc, w_in, bj, bl);
             team_sync<T>(tm);
         }
@@ -2643,7 +2817,8 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
     return true;
 }
 
-// A node of at most 32 neighbours, by one warp over a table of up to hcap slots:
+// A node of at most 32 neighbours up to its marked survivors, by one warp over
+// a table of up to hcap slots:
 // a neighbour per lane, whose count, degree, ids and deg(y,C) load together, so
 // the chain of dependent loads is neighbour -> rows -> community sizes ->
 // bracket values, half of the general path's (which counts the entries first
@@ -2651,9 +2826,9 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
 // the entries could fill more than half of the table.
 constexpr int LIT_SMALL_DEG = 32;
 
-__device__ bool lit_eval_small(const RunArgs &a, int i, LitNode &ln, int32_t y0, int32_t *keys, uint32_t *vals,
-                               int32_t *aux, float *dv, uint32_t hcap, LitScratch &ls, unsigned long long *acc) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+__device__ __forceinline__ bool lit_small(const RunArgs &a, LitNode &ln, int32_t y0, const LitTable &t, uint32_t hcap,
+                                          LitScratch &ls, int tm, unsigned long long &pb) {
+    const int lane = threadIdx.x & 31;
     const bool on = lane < ln.d && dbg_ok(a, y0 >= 0 && y0 < a.nnodes);
     const int32_t y = on ? y0 : ln.x;
     const RowHead ids = row_head8(a.mem, y, a.K), ks = row_head8(a.kmem, y, a.K), own = row_head8(a.mem, ln.x, a.K);
@@ -2668,64 +2843,61 @@ __device__ bool lit_eval_small(const RunArgs &a, int i, LitNode &ln, int32_t y0,
     while (H < 2u * (uint32_t)entries) H <<= 1;
     if (H > hcap) return false;
     const uint32_t hm = H - 1;
-    float *hs = reinterpret_cast<float *>(aux);
+    float *hs = reinterpret_cast<float *>(t.aux);
     for (uint32_t s = lane; s < H; s += 32) {
-        keys[s] = EMPTY_KEY;
-        vals[s] = 0u;
+        t.keys[s] = EMPTY_KEY;
+        t.vals[s] = 0u;
         hs[s] = 0.f;
     }
+    if (lane == 0) lit_zero_counts(ls, tm);
     __syncwarp();
     const int32_t *rowx = a.mem + (int64_t)ln.x * a.K;
-    for (int j = lane; j < ln.cx; j += 32) ht_insert(keys, vals, hm, head_entry(own, rowx, j), 0u, true);
+    for (int j = lane; j < ln.cx; j += 32) ht_insert(t.keys, t.vals, hm, head_entry(own, rowx, j), 0u, true);
     __syncwarp();
     const int32_t *rowy = a.mem + (int64_t)y * a.K, *krowy = a.kmem + (int64_t)y * a.K;
     for (int s0 = 0; s0 < cmax; s0 += 4) {
         int32_t C[4], k[4], n[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {   // four communities' sizes in flight
-            C[t] = -1;
-            n[t] = 0;
-            k[t] = 0;
-            if (s0 + t < cy) {
-                C[t] = head_entry(ids, rowy, s0 + t);
-                k[t] = head_entry(ks, krowy, s0 + t);
-                if (!dbg_ok(a, C[t] >= 0 && C[t] < a.nnodes && k[t] >= 0 && k[t] <= dy)) C[t] = -1;
-                if (C[t] >= 0) n[t] = __ldcg(&a.comm[C[t]].n);
+        for (int u = 0; u < 4; ++u) {   // four communities' sizes in flight
+            C[u] = -1;
+            n[u] = 0;
+            k[u] = 0;
+            if (s0 + u < cy) {
+                C[u] = head_entry(ids, rowy, s0 + u);
+                k[u] = head_entry(ks, krowy, s0 + u);
+                if (!dbg_ok(a, C[u] >= 0 && C[u] < a.nnodes && k[u] >= 0 && k[u] <= dy)) C[u] = -1;
+                if (C[u] >= 0) n[u] = __ldcg(&a.comm[C[u]].n);
             }
         }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            if (C[t] < 0) continue;
-            const int slot = lit_insert(keys, vals, hm, C[t]);   // has room: H >= 2 x entries
+        for (int u = 0; u < 4; ++u) {
+            if (C[u] < 0) continue;
+            const int slot = lit_insert(t.keys, t.vals, hm, C[u]);   // has room: H >= 2 x entries
             if (slot < 0) continue;
-            const float h = (vals[slot] & OWN_FLAG) ? lit_h_leave32(k[t], dy, n[t]) : lit_h_join32(k[t], dy, n[t]);
+            const float h = (t.vals[slot] & OWN_FLAG) ? lit_h_leave32((uint32_t)k[u], (uint32_t)dy, (uint32_t)n[u])
+                                                      : lit_h_join32((uint32_t)k[u], (uint32_t)dy, (uint32_t)n[u]);
             if (h != 0.f) atomicAdd(&hs[slot], h);
         }
     }
     __syncwarp();
-    unsigned long long pb = a.profile && on ? 12ull + 8ull * (unsigned long long)cy : 0ull;
+    pb = a.profile && on ? 12ull + 8ull * (unsigned long long)cy : 0ull;
+    lit_collect<1>(t, H, ls, tm, 0);
+    __syncwarp();
+    const int ncand = ls.ncand[tm];
     float lbj = -INFINITY, lbl = -INFINITY;
-    lit_screen_table<1>(a, ln.d, keys, vals, aux, dv, H, w, 0, lbj, lbl, pb, a.profile != 0);
-    lbj = warp_max_f(lbj);
-    lbl = warp_max_f(lbl);
-    lit_decide<1>(a, i, ln, keys, vals, aux, dv, H, lbj, lbl, ls, acc, w, 0, pb);
+    lit_screen_list<32>(a, ln.d, t, ncand, lane, lbj, lbl, pb);
+    __syncwarp();
+    lit_mark_list<32>(a, t, ncand, lane, warp_max_f(lbj), warp_max_f(lbl), ls, tm);
+    __syncwarp();
     return true;
 }
 
-__device__ __forceinline__ void lit_smem(double *base, float *&dv, int32_t *&keys, uint32_t *&vals, int32_t *&aux,
-                                         unsigned long long *&acc) {
-    dv = reinterpret_cast<float *>(base);
-    keys = reinterpret_cast<int32_t *>(dv + LB_SLOTS);
-    vals = reinterpret_cast<uint32_t *>(keys + LB_SLOTS);
-    aux = reinterpret_cast<int32_t *>(vals + LB_SLOTS);
-    acc = reinterpret_cast<unsigned long long *>(aux + LB_SLOTS);
-}
-
-struct LitTables {   // a block's shared tables and per-warp accumulators
-    int32_t *keys, *aux;
-    uint32_t *vals;
-    float *dv;
+struct LitTables {   // a block's shared tables, candidate lists and per-warp accumulators
+    LitTable tab;
     unsigned long long *acc;
+    __device__ __forceinline__ LitTable at(int slot) const {   // the part that starts at a slot
+        return LitTable{tab.keys + slot, tab.aux + slot, tab.vals + slot, tab.dv + slot, tab.list + slot / 2};
+    }
 };
 
 // One queued node by a team of T warps (index i in the queue; its static data and
@@ -2741,15 +2913,18 @@ __device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const Nod
     ln.beg = pf.beg;
     ln.end = pf.end;
     ln.d = pf.d;
-    const int base = tm * T * LW;
+    const LitTable tab = t.at(tm * T * LW);
+    unsigned long long *acc = t.acc + w * SACC_CHUNKS;
     if (ln.d <= LIT_SMALL_DEG) {
+        unsigned long long pb = 0;
         if constexpr (T == 1) {
-            return lit_eval_small(a, i, ln, pf.y0, t.keys + base, t.vals + base, t.aux + base, t.dv + base, LW, ls,
-                                  t.acc + w * SACC_CHUNKS);
+            if (!lit_small(a, ln, pf.y0, tab, LW, ls, tm, pb)) return false;
+            lit_resolve<1>(a, i, ln, tab, ls, acc, tm, 0, pb);
+            return true;
         } else if (2 * (ln.d + 1) * a.K <= T * LW) {   // the table holds it whatever its rows
-            if (w_in == 0)
-                lit_eval_small(a, i, ln, pf.y0, t.keys + base, t.vals + base, t.aux + base, t.dv + base, T * LW, ls,
-                               t.acc + w * SACC_CHUNKS);
+            if (w_in == 0) lit_small(a, ln, pf.y0, tab, T * LW, ls, tm, pb);
+            team_sync<T>(tm);
+            lit_resolve<T>(a, i, ln, tab, ls, acc, tm, w_in, pb);
             return true;
         }
     }
@@ -2768,8 +2943,7 @@ __device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const Nod
     uint32_t H = 32;
     while ((long long)H < 2 * bound) H <<= 1;
     if (H > (uint32_t)(T * LW)) return false;
-    if (!lit_eval_node<T>(a, i, ln, 1, t.keys + base, t.vals + base, t.aux + base, t.dv + base, H, ls,
-                          t.acc + w * SACC_CHUNKS, tm, w_in)) {
+    if (!lit_eval_shared<T>(a, i, ln, tab, H, ls, acc, tm, w_in)) {
         if (w_in == 0 && lane == 0) atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: H >= 2 x entries
     }
     return true;
@@ -2777,7 +2951,12 @@ __device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const Nod
 
 __device__ __forceinline__ LitTables lit_tables(double *dyn) {
     LitTables t;
-    lit_smem(dyn, t.dv, t.keys, t.vals, t.aux, t.acc);
+    t.tab.dv = reinterpret_cast<float *>(dyn);
+    t.tab.keys = reinterpret_cast<int32_t *>(t.tab.dv + LB_SLOTS);
+    t.tab.vals = reinterpret_cast<uint32_t *>(t.tab.keys + LB_SLOTS);
+    t.tab.aux = reinterpret_cast<int32_t *>(t.tab.vals + LB_SLOTS);
+    t.acc = reinterpret_cast<unsigned long long *>(t.tab.aux + LB_SLOTS);
+    t.tab.list = reinterpret_cast<uint16_t *>(t.acc + EV_WARPS * SACC_CHUNKS);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int c = lane; c < SACC_CHUNKS; c += 32) t.acc[w * SACC_CHUNKS + c] = 0ull;
     __syncwarp();
@@ -2843,15 +3022,16 @@ __device__ void lit_big_node(const RunArgs &a, int64_t bstart, int i, const LitT
             return;
         }
     }
-    int P = (int)((bound + LIT_PART_ENTRIES - 1) / LIT_PART_ENTRIES);
-    uint32_t Hs = (uint32_t)LB_SLOTS;
-    if (P < 1 || 2 * bound <= LB_SLOTS) {   // one pass over a table of pow2 >= 2 x entries
-        P = 1;
-        Hs = 32;
-        while ((long long)Hs < 2 * bound) Hs <<= 1;
+    if (2 * bound <= LB_SLOTS) {   // one pass over a table of pow2 >= 2 x entries
+        uint32_t H = 32;
+        while ((long long)H < 2 * bound) H <<= 1;
+        if (!lit_eval_shared<EV_WARPS>(a, i, ln, t.tab, H, ls, t.acc + w * SACC_CHUNKS, 0, w) && threadIdx.x == 0)
+            atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: H >= 2 x entries
+        return;
     }
-    while (!lit_eval_node<EV_WARPS>(a, i, ln, P, t.keys, t.vals, t.aux, t.dv, Hs, ls, t.acc + w * SACC_CHUNKS, 0, w)) {
-        Hs = (uint32_t)LB_SLOTS;
+    int P = (int)((bound + LIT_PART_ENTRIES - 1) / LIT_PART_ENTRIES);
+    while (!lit_eval_node<EV_WARPS>(a, i, ln, P, t.tab.keys, t.tab.vals, t.tab.aux, t.tab.dv, LB_SLOTS, ls,
+                                    t.acc + w * SACC_CHUNKS, 0, w)) {
         P *= 2;
         if (P > (1 << 22)) {   // cannot happen for < 2^31 entries; leave an error, not a loop
             if (threadIdx.x == 0) atomicOr(&a.ds->err, DERR_CHECK);
@@ -2962,8 +3142,7 @@ __global__ void __launch_bounds__(256) k_lh_fill(RunArgs a, LitHubPlan hp, int64
     {   // each warp takes a contiguous eighth of the chunk
         const int64_t per = (ce - cb + 7) / 8, w = threadIdx.x >> 5;
         const int64_t qb = min(ce, cb + w * per), qe = min(ce, cb + (w + 1) * per);
-        lit_warp_entries(a, qb, qe, pb, a.profile != 0, [&](int32_t C, int64_t ky, int64_t dy, int64_t n) {
-            if (!dbg_ok(a, ky >= 0 && ky <= dy)) return;
+        lit_warp_entries<4>(a, qb, qe, pb, a.profile != 0, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
             const int slot = lit_insert(keys, vals, hm, C);
             if (slot < 0) {   // cannot happen: the table holds 2 (d+1) K slots
                 atomicOr(&a.ds->err, DERR_CHECK);
@@ -3197,12 +3376,13 @@ __device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, 
                                 int64_t xe, uint32_t serial, unsigned long long &nj, unsigned long long &nl) {
     const int lane = threadIdx.x & 31;
     const int32_t j = __ldcg(&a.act[i]), l = __ldcg(&a.act[a.qcap + i]);
-    if (j < 0 && l < 0) return;
-    if (!dbg_ok(a, j < a.nnodes && l < a.nnodes && (j < 0 || j != l))) return;
     const int32_t kjoin = __ldcg(&a.act[2 * a.qcap + i]), kl = __ldcg(&a.act[3 * a.qcap + i]);
     int32_t *row = a.mem + (int64_t)x * a.K;
     int32_t *krow = a.kmem + (int64_t)x * a.K;
     const int32_t c = __ldcg(&a.nmem[x]);
+    const int32_t v0 = lane < a.K ? __ldcg(&row[lane]) : 0;   // ids move only in this warp: loaded with the rest
+    if (j < 0 && l < 0) return;
+    if (!dbg_ok(a, j < a.nnodes && l < a.nnodes && (j < 0 || j != l))) return;
     const int32_t d = (int32_t)(xe - xb);
     if (!dbg_ok(a, c >= 0 && c <= a.K && (j < 0 || (kjoin >= 0 && kjoin <= d)))) return;
     int jj = 0, jl = 0, ll = 0;
@@ -3279,7 +3459,7 @@ __device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, 
     int32_t c_new = c;
     if (c <= 32) {
         // the whole row in one load per array: leave l, insert j, ascending
-        const int32_t v = lane < c ? __ldcg(&row[lane]) : 0;
+        const int32_t v = v0;
         const int32_t kv = lane < c ? __ldcg(&krow[lane]) : 0;
         const bool keep = lane < c && v != l;
         const unsigned km = __ballot_sync(FULL, keep);
@@ -3336,14 +3516,18 @@ __device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, 
     const int32_t C = lane == 0 ? l : lane == 1 ? j : -1;
     if (C >= 0) {
         const bool in = lane == 1;
+        // both answers on their way before either is used
+        const uint32_t seen = atomicExch(&a.tstamp[C], serial);
+        const unsigned long long slot = in ? (unsigned long long)atomicAdd(&a.cm_cnt[C], 1u) : 0ull;
+        const unsigned long long o0 = a.cm_off[C], o1 = a.cm_off[C + 1];
         atomicAdd(&a.comm[C].n, in ? 1 : -1);
         atomicAdd(&a.comm[C].vol, in ? (uint32_t)d : (uint32_t)(-d));
         atomicAdd(&a.comm[C].m2, (uint32_t)(in ? 2 * kjoin + jj - 2 * jl : -2 * kl + ll));
+        if (seen != serial) a.touched[atomicAdd(a.ntouched, 1u)] = C;
         if (in) {
             ++nj;
-            const unsigned long long slot = atomicAdd(&a.cm_cnt[C], 1u);
-            if ((long long)slot < (long long)(a.cm_off[C + 1] - a.cm_off[C])) {
-                a.cm_node[a.cm_off[C] + slot] = x;
+            if (slot < o1 - o0) {
+                a.cm_node[o0 + slot] = x;
             } else {
                 const int32_t e = (int32_t)atomicAdd(a.jl_count, 1u);
                 a.jl_node[e] = x;
@@ -3352,7 +3536,6 @@ __device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, 
         } else {
             ++nl;
         }
-        if (atomicExch(&a.tstamp[C], serial) != serial) a.touched[atomicAdd(a.ntouched, 1u)] = C;
     }
     if (lane == 0) a.nmem[x] = c_new;
 }
@@ -3421,9 +3604,9 @@ __device__ __forceinline__ void lit_fsum_member(const RunArgs &a, int32_t C, int
 // The per-community values of the bracket from the member sums (rounded
 // to float; the bound E allows for it).  Lane t of the first three of a group
 // (all of which hold the sums) forms the t-th factor.
-__device__ __forceinline__ void lit_fsum_store(const RunArgs &a, int32_t C, int t, double f0, double f1, double f2) {
+__device__ __forceinline__ void lit_fsum_store(const RunArgs &a, int32_t C, const int4 &r, int t, double f0, double f1,
+                                               double f2) {
     if (t > 2) return;
-    const int4 r = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C]));
     const int32_t n = r.x;
     const double cc = a.gcc ? a.gcc[r.w] : a.cc;
     const double nd = __int2double_rn(n);
@@ -3467,42 +3650,50 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
     const bool few = step * EV_WARPS >= total;
     const int group = few ? -1 : LIT_FSUM_GROUP, warp = few ? LIT_FSUM_FEW : LIT_FSUM_WARP;
     const int64_t t = t0 + (few ? w : 4 * w + grp) * step;
-    int32_t C = 0, n = -1;
+    int32_t C = 0;
+    int4 rec = make_int4(-1, 0, 0, 0);
+    MemberRange mr{0, 0, 0};
     if (t < total && (!few || grp == 0)) {
         C = list ? __ldcg(&list[t]) : (int32_t)t;
-        n = __ldcg(&a.comm[C].n);
+        rec = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C]));
+        mr = lit_member_range(a, C);
     }
+    const int32_t n = rec.x;
     if (!few) {
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
         const bool mine = n >= 0 && n <= group;
         if (mine && n > 0)
-            lit_members(a, C, sub, 8, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
+            lit_members(a, C, mr, sub, 8, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 8);
-        if (mine) lit_fsum_store(a, C, sub, f0, f1, f2);
+        if (mine) lit_fsum_store(a, C, rec, sub, f0, f1, f2);
     }
     unsigned mid = __ballot_sync(FULL, sub == 0 && n > group);
     while (mid) {
         const int src = __ffs(mid) - 1;
         mid &= mid - 1;
         const int32_t C1 = __shfl_sync(FULL, C, src), n1 = __shfl_sync(FULL, n, src);
+        const int4 rec1 = make_int4(n1, __shfl_sync(FULL, rec.y, src), 0, __shfl_sync(FULL, rec.w, src));
+        const MemberRange mr1{__shfl_sync(FULL, mr.b0, src), __shfl_sync(FULL, mr.cap, src),
+                              __shfl_sync(FULL, mr.used, src)};
         if (n1 > warp) {
             if (lane == 0) fs.big[atomicAdd(&fs.nbig, 1)] = C1;
             continue;
         }
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-        lit_members(a, C1, lane, 32, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
+        lit_members(a, C1, mr1, lane, 32, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 32);
-        lit_fsum_store(a, C1, lane, f0, f1, f2);
+        lit_fsum_store(a, C1, rec1, lane, f0, f1, f2);
     }
     __syncthreads();
     const int nbig = fs.nbig;
     for (int b = 0; b < nbig; ++b) {
         const int32_t C1 = fs.big[b];
-        const int32_t n1 = __ldcg(&a.comm[C1].n);
+        const int4 rec1 = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C1]));
+        const int32_t n1 = rec1.x;
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-        lit_members(a, C1, threadIdx.x, blockDim.x, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
+        lit_members(a, C1, lit_member_range(a, C1), threadIdx.x, blockDim.x, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 32);
         if (lane == 0) {
@@ -3515,7 +3706,7 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
             double sum[3] = {0.0, 0.0, 0.0};
             for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2)
                 for (int t2 = 0; t2 < 3; ++t2) sum[t2] += fs.red[t2][k2];
-            lit_fsum_store(a, C1, lane, sum[0], sum[1], sum[2]);
+            lit_fsum_store(a, C1, rec1, lane, sum[0], sum[1], sum[2]);
         }
         __syncthreads();
     }
