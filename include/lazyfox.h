@@ -73,8 +73,8 @@ typedef struct lf_options {
                                 iteration captured in a CUDA graph; 2: one persistent
                                 cooperative kernel per iteration runs every queue
                                 (evaluate, grid barrier, apply, grid barrier); 0 (default):
-                                persistent for queues of at most 256 nodes (LF_GAIN_LITERAL: 16
-                                nodes, and never for graphs with nodes of degree above 1024 or
+                                persistent for queues of at most 256 nodes (LF_GAIN_LITERAL: 1
+                                node, and never for graphs with nodes of degree above 1024 or
                                 batches), else per queue */
     int32_t barrier_timeout_ms; /* bound on one grid-barrier wait (0: 2000 ms); a wait that
                                 runs out ends the call with LF_ERR_TIMEOUT */

@@ -242,11 +242,11 @@ struct lf_graph {
     uint32_t *lit_misc = nullptr;         // [0]: joiners listed in this iteration
     float *litF = nullptr;                // 8n: F(n-1), F(n+1), WCC-hat(C), 1/((n+1)n cc), 1/((n-1)(n-2) cc)
     uint32_t *tstamp = nullptr;           // n
-    uint32_t *lit_ctr = nullptr;          // 4 per queue
+    uint32_t *lit_ctr = nullptr;          // 8 per queue
     unsigned long long *lit_items = nullptr;   // movers of a queue, in pieces
     int32_t *lit_apacc = nullptr;         // 4 qcap, zero between queues
     int64_t lit_ctr_cap = 0;
-    int32_t *lit_over = nullptr;          // qcap
+    int32_t *lit_over = nullptr;          // 4 qcap: two lists of (position, entries)
     int32_t *touched = nullptr;           // 2 qcap
     int64_t lit_qcap = 0;
     unsigned long long *lit_used = nullptr;   // per queue: global table slots handed out

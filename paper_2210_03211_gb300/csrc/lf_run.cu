@@ -1827,7 +1827,10 @@ constexpr int LW = 512;                            // table slots of one warp
 constexpr int LB_SLOTS = EV_WARPS * LW;            // table slots of a block
 constexpr uint32_t SURV_FLAG = 0x40000000u;        // candidate survives the bracket test
 constexpr uint32_t CNT_MASK = 0x3fffffffu;
-constexpr size_t LIT_SMEM = (size_t)LB_SLOTS * 16 + (size_t)EV_WARPS * SACC_CHUNKS * 8 + (size_t)LB_SLOTS;   // tables, accumulators, candidate lists
+// tables (key, count, correction per slot), accumulators, candidate lists
+constexpr size_t LIT_SMEM = (size_t)LB_SLOTS * 12 + (size_t)EV_WARPS * SACC_CHUNKS * 8 + (size_t)LB_SLOTS * 2;
+constexpr uint32_t POS_FLAG = 0x20000000u;         // shared tables: the lower end is positive
+constexpr uint32_t LIST_CNT_MASK = 0xffffu;        // shared tables: counts are below 2^16
 constexpr int LIT_PART_ENTRIES = 1024;             // entries per pass of a multi-pass node
 
 // Signed exact accumulation: like sacc_add, with negative values added as
@@ -2592,9 +2595,9 @@ __device__ void lit_exact_survivors(const RunArgs &a, const LitNode &ln, const i
 
 // One kind's survivors: none or a lone one with a positive lower end settles
 // it; true if exact sums have to.
-__device__ __forceinline__ bool lit_settle(const RunArgs &a, int count, int32_t C, int32_t k, float L, Best &b) {
+__device__ __forceinline__ bool lit_settle(const RunArgs &a, int count, int32_t C, int32_t k, bool positive, Best &b) {
     if (count == 0) return false;
-    if (a.screen && count == 1 && L > 0.f) {
+    if (a.screen && count == 1 && positive) {
         b = Best{INFINITY, C, k};
         return false;
     }
@@ -2641,11 +2644,20 @@ __device__ __forceinline__ void lit_finish(const RunArgs &a, int i, const LitNod
 // gather of the communities' records per 32 slots; over the list it is one per 32
 // candidates.
 struct LitTable {
-    int32_t *keys, *aux;
+    int32_t *keys, *aux;   // aux: the FP32 corrections, then the bracket's upper end
     uint32_t *vals;
-    float *dv;
     uint16_t *list;
 };
+
+// Slots of a shared table for `entries` entries, at most cap of them; above cap if
+// it does not fit.  Twice the entries; up to three quarters of the largest table
+// are accepted (distinct communities are fewer than entries).
+__device__ __forceinline__ uint32_t lit_table_slots(long long entries, uint32_t cap) {
+    if (4 * entries > 3 * (long long)cap) return 2 * cap;
+    uint32_t H = 32;
+    while (H < cap && H < 2 * entries) H <<= 1;
+    return H;
+}
 
 // The used slots listed by one warp of the NW that share the table (ls.ncand[tm]
 // zero before).
@@ -2677,8 +2689,8 @@ __device__ __forceinline__ void lit_screen_list(const RunArgs &a, int32_t d, con
         const uint32_t v = t.vals[s];
         float X, E;
         lit_screen(a, t.keys[s], v, d, hs[s], X, E);
-        t.dv[s] = X;
-        t.aux[s] = __float_as_int(E);
+        t.aux[s] = __float_as_int(X + E);
+        if (X - E > 0.f) t.vals[s] = v | POS_FLAG;
         if (v & OWN_FLAG) lbl = fmaxf(lbl, X - E);
         else lbj = fmaxf(lbj, X - E);
         if (a.profile) {
@@ -2695,7 +2707,7 @@ __device__ __forceinline__ void lit_mark_list(const RunArgs &a, const LitTable &
     for (int c = tl; c < ncand; c += NT) {
         const int s = t.list[c];
         const uint32_t v = t.vals[s];
-        const float U = t.dv[s] + __int_as_float(t.aux[s]);
+        const float U = __int_as_float(t.aux[s]);
         const bool own = (v & OWN_FLAG) != 0;
         if (!a.screen || (U > 0.f && U >= (own ? lbl : lbj))) {
             t.vals[s] = v | SURV_FLAG;
@@ -2719,15 +2731,16 @@ __device__ __forceinline__ void lit_resolve(const RunArgs &a, int i, const LitNo
     if (a.screen && ns <= SURV_LIST && (nj == 1 || nl == 1)) {
         const int s = lane < ns ? ls.surv[tm][lane] : 0;
         const uint32_t v = lane < ns ? t.vals[s] : 0u;
-        const float L = lane < ns ? t.dv[s] - __int_as_float(t.aux[s]) : 0.f;
         const int32_t C = lane < ns ? t.keys[s] : 0;
         const unsigned ml = __ballot_sync(FULL, lane < ns && (v & OWN_FLAG)), mj = __ballot_sync(FULL, lane < ns && !(v & OWN_FLAG));
-        if (nj == 1) do_j = lit_settle(a, 1, __shfl_sync(FULL, C, __ffs(mj) - 1),
-                                       (int32_t)(__shfl_sync(FULL, v, __ffs(mj) - 1) & CNT_MASK),
-                                       __shfl_sync(FULL, L, __ffs(mj) - 1), bj);
-        if (nl == 1) do_l = lit_settle(a, 1, __shfl_sync(FULL, C, __ffs(ml) - 1),
-                                       (int32_t)(__shfl_sync(FULL, v, __ffs(ml) - 1) & CNT_MASK),
-                                       __shfl_sync(FULL, L, __ffs(ml) - 1), bl);
+        if (nj == 1) {
+            const uint32_t v1 = __shfl_sync(FULL, v, __ffs(mj) - 1);
+            do_j = lit_settle(a, 1, __shfl_sync(FULL, C, __ffs(mj) - 1), (int32_t)(v1 & LIST_CNT_MASK), v1 & POS_FLAG, bj);
+        }
+        if (nl == 1) {
+            const uint32_t v1 = __shfl_sync(FULL, v, __ffs(ml) - 1);
+            do_l = lit_settle(a, 1, __shfl_sync(FULL, C, __ffs(ml) - 1), (int32_t)(v1 & LIST_CNT_MASK), v1 & POS_FLAG, bl);
+        }
     }
     if (do_j || do_l) {
         const int count = ns <= SURV_LIST ? ns : ls.ncand[tm];
@@ -2737,7 +2750,7 @@ __device__ __forceinline__ void lit_resolve(const RunArgs &a, int i, const LitNo
             const bool own = (v & OWN_FLAG) != 0;
             if (!(v & SURV_FLAG) || !(own ? do_l : do_j)) continue;
             const int32_t C = t.keys[s];
-            const int64_t k = (int64_t)(v & CNT_MASK);
+            const int64_t k = (int64_t)(v & LIST_CNT_MASK);
             const double g = lit_exact_gain(a, ln.x, ln.d, C, own, k, acc);
             if (a.profile && lane == 0) atomicAdd(&a.ds->prof_exact, 1ull);
             if (g > 0.0) {
@@ -2754,8 +2767,8 @@ __device__ __forceinline__ void lit_zero_counts(LitScratch &ls, int tm) {
     ls.ncand[tm] = ls.ns[tm] = ls.nsj[tm] = ls.nsl[tm] = 0;
 }
 
-// A node's decision over one shared table (H >= 2 x its entries) by a team of T
-// warps.
+// A node's decision over one shared table with room for its entries by a team
+// of T warps.
 template <int T>
 __device__ __forceinline__ bool lit_eval_shared(const RunArgs &a, int i, const LitNode &ln, const LitTable &t, uint32_t H,
                                                 LitScratch &ls, unsigned long long *acc, int tm, int w_in) {
@@ -2797,7 +2810,7 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
         lit_mark<T>(a, keys, vals, aux, dv, H, lbj, lbl, ls, tm, w_in, cj, cl, Cj, Cl, kj, kl, Lj, Ll);
     }
     Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
-    const bool do_j = lit_settle(a, cj, Cj, kj, Lj, bj), do_l = lit_settle(a, cl, Cl, kl, Ll, bl);
+    const bool do_j = lit_settle(a, cj, Cj, kj, Lj > 0.f, bj), do_l = lit_settle(a, cl, Cl, kl, Ll > 0.f, bl);
     if (do_j || do_l) {
         for (int p = 0; p < P; ++p) {
             if (P > 1) {
@@ -2823,11 +2836,11 @@ __device__ bool lit_eval_node(const RunArgs &a, int i, const LitNode &ln, int P,
 // the chain of dependent loads is neighbour -> rows -> community sizes ->
 // bracket values, half of the general path's (which counts the entries first
 // to size its table, then reads the rows).  y0: this lane's neighbour.  False if
-// the entries could fill more than half of the table.
+// the table has no room for the entries (bound: their number).
 constexpr int LIT_SMALL_DEG = 32;
 
 __device__ __forceinline__ bool lit_small(const RunArgs &a, LitNode &ln, int32_t y0, const LitTable &t, uint32_t hcap,
-                                          LitScratch &ls, int tm, unsigned long long &pb) {
+                                          LitScratch &ls, int tm, unsigned long long &pb, long long &bound) {
     const int lane = threadIdx.x & 31;
     const bool on = lane < ln.d && dbg_ok(a, y0 >= 0 && y0 < a.nnodes);
     const int32_t y = on ? y0 : ln.x;
@@ -2839,8 +2852,8 @@ __device__ __forceinline__ bool lit_small(const RunArgs &a, LitNode &ln, int32_t
     if (!dbg_ok(a, ln.cx >= 0 && ln.cx <= a.K)) ln.cx = 0;
     const int32_t entries = __reduce_add_sync(FULL, cy) + ln.cx;
     const int32_t cmax = __reduce_max_sync(FULL, cy);
-    uint32_t H = 32;
-    while (H < 2u * (uint32_t)entries) H <<= 1;
+    bound = entries;
+    const uint32_t H = lit_table_slots(entries, hcap);
     if (H > hcap) return false;
     const uint32_t hm = H - 1;
     float *hs = reinterpret_cast<float *>(t.aux);
@@ -2872,7 +2885,7 @@ __device__ __forceinline__ bool lit_small(const RunArgs &a, LitNode &ln, int32_t
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (C[u] < 0) continue;
-            const int slot = lit_insert(t.keys, t.vals, hm, C[u]);   // has room: H >= 2 x entries
+            const int slot = lit_insert(t.keys, t.vals, hm, C[u]);   // has room
             if (slot < 0) continue;
             const float h = (t.vals[slot] & OWN_FLAG) ? lit_h_leave32((uint32_t)k[u], (uint32_t)dy, (uint32_t)n[u])
                                                       : lit_h_join32((uint32_t)k[u], (uint32_t)dy, (uint32_t)n[u]);
@@ -2896,17 +2909,16 @@ struct LitTables {   // a block's shared tables, candidate lists and per-warp ac
     LitTable tab;
     unsigned long long *acc;
     __device__ __forceinline__ LitTable at(int slot) const {   // the part that starts at a slot
-        return LitTable{tab.keys + slot, tab.aux + slot, tab.vals + slot, tab.dv + slot, tab.list + slot / 2};
+        return LitTable{tab.keys + slot, tab.aux + slot, tab.vals + slot, tab.list + slot};
     }
 };
 
 // One queued node by a team of T warps (index i in the queue; its static data and
-// this warp's first neighbours prefetched in pf).  False if its entries (own row
-// plus its neighbours' rows) could fill more than half of the team's table: a
-// whole block has to take it.
+// this warp's first neighbours prefetched in pf).  False if the team's table has no
+// room for its entries (own row plus its neighbours' rows; bound: their number).
 template <int T>
 __device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const NodePrefetch &pf, const LitTables &t,
-                                              LitScratch &ls, int tm, int w_in) {
+                                              LitScratch &ls, int tm, int w_in, long long &bound) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     LitNode ln;
     ln.x = pf.x;
@@ -2918,18 +2930,18 @@ __device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const Nod
     if (ln.d <= LIT_SMALL_DEG) {
         unsigned long long pb = 0;
         if constexpr (T == 1) {
-            if (!lit_small(a, ln, pf.y0, tab, LW, ls, tm, pb)) return false;
+            if (!lit_small(a, ln, pf.y0, tab, LW, ls, tm, pb, bound)) return false;
             lit_resolve<1>(a, i, ln, tab, ls, acc, tm, 0, pb);
             return true;
-        } else if (2 * (ln.d + 1) * a.K <= T * LW) {   // the table holds it whatever its rows
-            if (w_in == 0) lit_small(a, ln, pf.y0, tab, T * LW, ls, tm, pb);
+        } else if (4 * (ln.d + 1) * a.K <= 3 * T * LW) {   // the table holds it whatever its rows
+            if (w_in == 0) lit_small(a, ln, pf.y0, tab, T * LW, ls, tm, pb, bound);
             team_sync<T>(tm);
             lit_resolve<T>(a, i, ln, tab, ls, acc, tm, w_in, pb);
             return true;
         }
     }
     ln.cx = __ldcg(&a.nmem[ln.x]);
-    long long bound = w_in == 0 && lane == 0 ? ln.cx : 0;
+    bound = w_in == 0 && lane == 0 ? ln.cx : 0;
     for (int64_t q = ln.beg + w_in * 32 + lane; q < ln.end; q += T * 32) bound += __ldcg(&a.nmem[a.adj[q]]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) bound += __shfl_xor_sync(FULL, bound, o);
@@ -2940,19 +2952,17 @@ __device__ __forceinline__ bool lit_eval_team(const RunArgs &a, int i, const Nod
         for (int k2 = 0; k2 < T; ++k2) bound += ls.part[tm * T + k2];
         team_sync<T>(tm);
     }
-    uint32_t H = 32;
-    while ((long long)H < 2 * bound) H <<= 1;
+    const uint32_t H = lit_table_slots(bound, T * LW);
     if (H > (uint32_t)(T * LW)) return false;
     if (!lit_eval_shared<T>(a, i, ln, tab, H, ls, acc, tm, w_in)) {
-        if (w_in == 0 && lane == 0) atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: H >= 2 x entries
+        if (w_in == 0 && lane == 0) atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: the table has room
     }
     return true;
 }
 
 __device__ __forceinline__ LitTables lit_tables(double *dyn) {
     LitTables t;
-    t.tab.dv = reinterpret_cast<float *>(dyn);
-    t.tab.keys = reinterpret_cast<int32_t *>(t.tab.dv + LB_SLOTS);
+    t.tab.keys = reinterpret_cast<int32_t *>(dyn);
     t.tab.vals = reinterpret_cast<uint32_t *>(t.tab.keys + LB_SLOTS);
     t.tab.aux = reinterpret_cast<int32_t *>(t.tab.vals + LB_SLOTS);
     t.acc = reinterpret_cast<unsigned long long *>(t.tab.aux + LB_SLOTS);
@@ -2963,75 +2973,52 @@ __device__ __forceinline__ LitTables lit_tables(double *dyn) {
     return t;
 }
 
-// Teams of T warps, one queued node each.  A node too large for its team is listed
-// for k_lit_big.  Counters: over[0] = listed nodes, over[1] = next.  The
-// order, offsets and neighbour ids never change in a run, so they are read
-// before the wait for the previous kernel.
-template <int T>
-__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t bstart, int32_t blen, uint32_t *over,
-                                                           int32_t *over_list) {
-    extern __shared__ double lit_dyn[];
-    __shared__ LitScratch ls;
-    const LitTables t = lit_tables(lit_dyn);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tm = w / T, w_in = w % T;
-    const int i = (int)blockIdx.x * (EV_WARPS / T) + tm;
-    NodePrefetch pf;
-    prefetch_node(a, bstart, blen, i, w_in, pf);
-    pdl_trigger();
-    pdl_wait();
-    if (i >= blen) return;   // the whole team leaves together
-    if (pf.d > a.lit_hub_deg) return;   // the hub kernels decide it
-    if (!lit_eval_team<T>(a, i, pf, t, ls, tm, w_in) && w_in == 0 && lane == 0) over_list[atomicAdd(&over[0], 1u)] = i;
-}
+// Nodes a team's table has no room for, with their number of entries.
+struct LitOver {
+    int2 *mid, *big;           // for teams of LIT_MID warps, for blocks
+    uint32_t *ctr;             // [0] big listed, [1] big taken, [4] mid listed, [5] mid taken
+    unsigned long long *used;  // slots of the global area handed out
+};
 
-// One node by the whole block: over the block's table in as many parts as needed
-// (a part that overflows doubles the parts), or over a table of its own in
-// global memory if the queue's area has room.
-__device__ void lit_big_node(const RunArgs &a, int64_t bstart, int i, const LitTables &t, LitScratch &ls,
-                             long long &s_base, unsigned long long *used) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// One node by the whole block: over the block's table if it has room for the
+// node's entries (bound), else over a table of its own in global memory if the
+// queue's area has room, else over the block's table in as many parts as
+// needed (a part that overflows doubles the parts).
+__device__ void lit_big_node(const RunArgs &a, int64_t bstart, int i, long long bound, const LitTables &t,
+                             LitScratch &ls, long long &s_base, unsigned long long *used) {
+    const int w = threadIdx.x >> 5;
     LitNode ln;
     ln.x = a.order[bstart + i];
     ln.beg = a.off[ln.x];
     ln.end = a.off[ln.x + 1];
     ln.d = (int32_t)(ln.end - ln.beg);
     ln.cx = __ldcg(&a.nmem[ln.x]);
-    long long bound = threadIdx.x == 0 ? ln.cx : 0;
-    for (int64_t q = ln.beg + threadIdx.x; q < ln.end; q += EV_THREADS) bound += __ldcg(&a.nmem[a.adj[q]]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bound += __shfl_xor_sync(FULL, bound, o);
-    if (lane == 0) ls.part[w] = bound;
-    __syncthreads();
-    bound = 0;
-    for (int k2 = 0; k2 < EV_WARPS; ++k2) bound += ls.part[k2];
-    __syncthreads();
-    if (2 * bound > LB_SLOTS) {   // a table of its own in global memory, if the queue's area has room
-        unsigned long long H = 32;
-        while ((long long)H < 2 * bound) H <<= 1;
-        if (threadIdx.x == 0) {
-            const unsigned long long base = atomicAdd(used, H);
-            s_base = base + H <= a.lg_cap ? (long long)base : -1ll;
-        }
-        __syncthreads();
-        const long long base = s_base;
-        __syncthreads();
-        if (base >= 0) {
-            lit_eval_node<EV_WARPS>(a, i, ln, 1, a.lg_keys + base, a.lg_vals + base, a.lg_aux + base, a.lg_dv + base,
-                                    (uint32_t)H, ls, t.acc + w * SACC_CHUNKS, 0, w);
-            return;
-        }
-    }
-    if (2 * bound <= LB_SLOTS) {   // one pass over a table of pow2 >= 2 x entries
-        uint32_t H = 32;
-        while ((long long)H < 2 * bound) H <<= 1;
-        if (!lit_eval_shared<EV_WARPS>(a, i, ln, t.tab, H, ls, t.acc + w * SACC_CHUNKS, 0, w) && threadIdx.x == 0)
-            atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: H >= 2 x entries
+    unsigned long long *acc = t.acc + w * SACC_CHUNKS;
+    const uint32_t Hs = lit_table_slots(bound, LB_SLOTS);
+    if (Hs <= (uint32_t)LB_SLOTS) {
+        if (!lit_eval_shared<EV_WARPS>(a, i, ln, t.tab, Hs, ls, acc, 0, w) && threadIdx.x == 0)
+            atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: the table has room
         return;
     }
+    unsigned long long H = 32;
+    while ((long long)H < 2 * bound) H <<= 1;
+    if (threadIdx.x == 0) {
+        const unsigned long long base = atomicAdd(used, H);
+        s_base = base + H <= a.lg_cap ? (long long)base : -1ll;
+    }
+    __syncthreads();
+    const long long base = s_base;
+    __syncthreads();
+    if (base >= 0) {
+        lit_eval_node<EV_WARPS>(a, i, ln, 1, a.lg_keys + base, a.lg_vals + base, a.lg_aux + base, a.lg_dv + base,
+                                (uint32_t)H, ls, acc, 0, w);
+        return;
+    }
+    // parts: a table of half the slots, the brackets in the other half of the keys
+    constexpr uint32_t HP = LB_SLOTS / 2;
     int P = (int)((bound + LIT_PART_ENTRIES - 1) / LIT_PART_ENTRIES);
-    while (!lit_eval_node<EV_WARPS>(a, i, ln, P, t.tab.keys, t.tab.vals, t.tab.aux, t.tab.dv, LB_SLOTS, ls,
-                                    t.acc + w * SACC_CHUNKS, 0, w)) {
+    while (!lit_eval_node<EV_WARPS>(a, i, ln, P, t.tab.keys, t.tab.vals, t.tab.aux,
+                                    reinterpret_cast<float *>(t.tab.keys + HP), HP, ls, acc, 0, w)) {
         P *= 2;
         if (P > (1 << 22)) {   // cannot happen for < 2^31 entries; leave an error, not a loop
             if (threadIdx.x == 0) atomicOr(&a.ds->err, DERR_CHECK);
@@ -3040,27 +3027,113 @@ __device__ void lit_big_node(const RunArgs &a, int64_t bstart, int i, const LitT
     }
 }
 
-// Listed nodes, one block each, taken from a counter.
-__global__ void __launch_bounds__(EV_THREADS, 3) k_lit_big(RunArgs a, int64_t bstart, uint32_t *over,
-                                                          const int32_t *over_list, unsigned long long *used) {
+// Teams of T warps, one queued node each; the hub kernels take nodes above
+// lit_hub_deg.  A node too large for its team is listed for k_lit_mid or k_lit_big,
+// or, with INBLOCK, evaluated by its own block right after (queues of at most one
+// wave of blocks: two kernels' launches saved, 3 us a queue even when nothing is
+// listed; longer queues list many and balance better from a counter).  The order,
+// offsets and neighbour ids never change in a run, so they are read before the
+// wait for the previous kernel.
+//
+// Tiers by a node's entries: one warp up to 384 (three quarters of 512 slots), two
+// warps up to 768, a block up to 3,072, global tables or parts beyond.  Mean over the
+// queues of all tiers: 767k nodes, q 16,384: 106 + 247 (warps up to 256 entries, then
+// blocks, which a few hundred entries left idle between barriers) -> 141 + 60 + 98 us;
+// 3.07M nodes, q 65,536: 379 + 375 -> 453 + 80 + 92 us.
+constexpr int LIT_MID = 2;   // warps of the teams between one warp and a block
+
+template <int T, bool INBLOCK>
+__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t bstart, int32_t blen, LitOver ov) {
     extern __shared__ double lit_dyn[];
     __shared__ LitScratch ls;
-    __shared__ int s_i;
+    const LitTables t = lit_tables(lit_dyn);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int tm = w / T, w_in = w % T;
+    const int i = (int)blockIdx.x * (EV_WARPS / T) + tm;
+    NodePrefetch pf;
+    prefetch_node(a, bstart, blen, i, w_in, pf);
+    if constexpr (INBLOCK) {
+        __shared__ int2 s_over[EV_WARPS];
+        __shared__ int s_nover;
+        __shared__ long long s_base;
+        if (threadIdx.x == 0) s_nover = 0;
+        __syncthreads();
+        pdl_trigger();
+        pdl_wait();
+        if (i < blen && pf.d <= a.lit_hub_deg) {
+            long long bound = 0;
+            if (!lit_eval_team<T>(a, i, pf, t, ls, tm, w_in, bound) && w_in == 0 && lane == 0)
+                s_over[atomicAdd(&s_nover, 1)] = make_int2(i, (int)min(bound, 0x7fffffffll));
+        }
+        __syncthreads();
+        const int nover = s_nover;
+        for (int h = 0; h < nover; ++h) lit_big_node(a, bstart, s_over[h].x, s_over[h].y, t, ls, s_base, ov.used);
+    } else {
+        pdl_trigger();
+        pdl_wait();
+        if (i >= blen || pf.d > a.lit_hub_deg) return;   // the whole team leaves together
+        long long bound = 0;
+        if (!lit_eval_team<T>(a, i, pf, t, ls, tm, w_in, bound) && w_in == 0 && lane == 0) {
+            const int2 e = make_int2(i, (int)min(bound, 0x7fffffffll));
+            if (T < LIT_MID && lit_table_slots(bound, LIT_MID * LW) <= LIT_MID * LW) ov.mid[atomicAdd(&ov.ctr[4], 1u)] = e;
+            else ov.big[atomicAdd(&ov.ctr[0], 1u)] = e;
+        }
+    }
+}
+
+// Listed nodes by teams of LIT_MID warps, taken from a counter.
+__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_mid(RunArgs a, int64_t bstart, LitOver ov) {
+    extern __shared__ double lit_dyn[];
+    __shared__ LitScratch ls;
+    __shared__ uint32_t s_at[EV_WARPS / LIT_MID];
+    const LitTables t = lit_tables(lit_dyn);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int tm = w / LIT_MID, w_in = w % LIT_MID;
+    const LitTable tab = t.at(tm * LIT_MID * LW);
+    pdl_trigger();
+    pdl_wait();
+    const uint32_t count = __ldcg(&ov.ctr[4]);
+    for (;;) {
+        if (w_in == 0 && lane == 0) s_at[tm] = atomicAdd(&ov.ctr[5], 1u);
+        team_sync<LIT_MID>(tm);
+        const uint32_t n = s_at[tm];
+        if (n >= count) break;
+        const int2 e = __ldcg(&ov.mid[n]);
+        LitNode ln;
+        ln.x = a.order[bstart + e.x];
+        ln.beg = a.off[ln.x];
+        ln.end = a.off[ln.x + 1];
+        ln.d = (int32_t)(ln.end - ln.beg);
+        ln.cx = __ldcg(&a.nmem[ln.x]);
+        if (!lit_eval_shared<LIT_MID>(a, e.x, ln, tab, lit_table_slots(e.y, LIT_MID * LW), ls, t.acc + w * SACC_CHUNKS,
+                                      tm, w_in) &&
+            w_in == 0 && lane == 0)
+            atomicOr(&a.ds->err, DERR_CHECK);   // cannot happen: the table has room
+        team_sync<LIT_MID>(tm);
+    }
+}
+
+// Listed nodes, one block each, taken from a counter.
+__global__ void __launch_bounds__(EV_THREADS, 3) k_lit_big(RunArgs a, int64_t bstart, LitOver ov) {
+    extern __shared__ double lit_dyn[];
+    __shared__ LitScratch ls;
+    __shared__ int2 s_e;
     __shared__ long long s_base;
     const LitTables t = lit_tables(lit_dyn);
     pdl_trigger();
     pdl_wait();
-    const uint32_t count = __ldcg(&over[0]);
+    const uint32_t count = __ldcg(&ov.ctr[0]);
     for (;;) {
         if (threadIdx.x == 0) {
-            const uint32_t n = atomicAdd(&over[1], 1u);
-            s_i = n < count ? over_list[n] : -1;
+            const uint32_t n = atomicAdd(&ov.ctr[1], 1u);
+            s_e = n < count ? __ldcg(&ov.big[n]) : make_int2(-1, 0);
         }
         __syncthreads();
-        const int i = s_i;
+        const int2 e = s_e;
         __syncthreads();
-        if (i < 0) break;
-        lit_big_node(a, bstart, i, t, ls, s_base, used);
+        if (e.x < 0) break;
+        lit_big_node(a, bstart, e.x, e.y, t, ls, s_base, ov.used);
+        __syncthreads();
     }
 }
 
@@ -4101,7 +4174,7 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_iterate(RunArgs a, int64_t q,
 struct LitIterShared {
     LitScratch ls;
     FsumShared fs;
-    int32_t over[EV_WARPS];
+    int2 over[EV_WARPS];
     int nover, ok;
     long long base;
 };
@@ -4140,7 +4213,7 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, const 
     if (a.qtimes && blockIdx.x == 0 && threadIdx.x == 0) a.qtimes[0] = global_ns();
     for (int64_t b = first; b < first + count; ++b) {
         const uint32_t serial = (uint32_t)queue_serial(a, b);
-        a.ntouched = ctr + 4 * b + 2;
+        a.ntouched = ctr + 8 * b + 2;
         // evaluate
         NodePrefetch cur = pf;
         for (int64_t base = base0; base < blen; base += round) {
@@ -4148,11 +4221,13 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, const 
             if (base != base0) prefetch_node(a, bstart, blen, i, w_in, cur);
             if (threadIdx.x == 0) sh.nover = 0;
             __syncthreads();
-            if (i < blen && !lit_eval_team<T>(a, i, cur, t, sh.ls, tm, w_in) && w_in == 0 && lane == 0)
-                sh.over[atomicAdd(&sh.nover, 1)] = i;
+            long long bound = 0;
+            if (i < blen && !lit_eval_team<T>(a, i, cur, t, sh.ls, tm, w_in, bound) && w_in == 0 && lane == 0)
+                sh.over[atomicAdd(&sh.nover, 1)] = make_int2(i, (int)min(bound, 0x7fffffffll));
             __syncthreads();
             const int nover = sh.nover;
-            for (int h = 0; h < nover; ++h) lit_big_node(a, bstart, sh.over[h], t, sh.ls, sh.base, used + b);
+            for (int h = 0; h < nover; ++h)
+                lit_big_node(a, bstart, sh.over[h].x, sh.over[h].y, t, sh.ls, sh.base, used + b);
         }
         if (!meet()) return;
         // apply: each team's first warp, its own nodes
@@ -4733,10 +4808,15 @@ void set_eval_attrs() {
     LF_CUDA(cudaFuncSetAttribute(k_eval_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EV_DYN_SMEM));
     LF_CUDA(cudaFuncSetAttribute(k_eval_tdyn<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EV_DYN_SMEM));
     LF_CUDA(cudaFuncSetAttribute(k_huge_chunks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(HUGE_SH * 8)));
-    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
-    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
-    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
-    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_eval<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
     LF_CUDA(cudaFuncSetAttribute(k_lit_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
 }
 
@@ -4891,11 +4971,11 @@ void free_lit_hub_plan(lf_graph *g) {
     g->lh_plan_K = 0;
 }
 
-// Queues up to this size run in the persistent loop under the paper's gain: one
-// block and no grid barrier at queue size 1. Measured, us a queue, loop / launches:
-// 1,000 nodes (planted) q 1 13.0 / 18.1, q 4 19.8 / 21.3, q 16 22.9 / 24.3; 84k nodes
-// q 16 18.3 / 18.8, q 64 25.2 / 24.1, q 256 36.1 / 30.1.
-constexpr int64_t LIT_LOOP_MAX_Q = 16;
+// Queues up to this size run in the persistent loop under the paper's gain: at
+// queue size 1 one block holds it, with no grid barrier.  Measured, us a queue, loop /
+// launches: 1,000 nodes (planted) q 1 13.3 / 16.9, q 2 19.2 / 17.8, q 8 21.0 / 21.1, q 16
+// 23.2 / 22.4; 84k nodes q 64 25.0 / 21.9, q 256 36.4 / 27.6.
+constexpr int64_t LIT_LOOP_MAX_Q = 1;
 
 // The hubs of every queue (degree > LIT_HUB_DEG): worst-case tables of
 // pow2 >= 2 (d+1) K slots (K bounds every row), fill items of LH_CHUNK
@@ -5028,7 +5108,9 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
     const int T0 = choose_team(g, q);
     static const int per_sm_big = blocks_per_sm(k_lit_big, EV_THREADS, LIT_SMEM);
     const unsigned big_grid = (unsigned)(num_sms() * std::max(1, per_sm_big));
-    LF_CUDA(cudaMemsetAsync(g->lit_ctr + 4 * first, 0, (size_t)(4 * count) * sizeof(uint32_t), g->stream));
+    static const int per_sm_mid = blocks_per_sm(k_lit_mid, EV_THREADS, LIT_SMEM);
+    const unsigned mid_grid = (unsigned)(num_sms() * std::max(1, per_sm_mid));
+    LF_CUDA(cudaMemsetAsync(g->lit_ctr + 8 * first, 0, (size_t)(8 * count) * sizeof(uint32_t), g->stream));
     LF_CUDA(cudaMemsetAsync(g->lit_used + first, 0, (size_t)count * sizeof(unsigned long long), g->stream));
     const bool prof = g->profile && (int64_t)g->prof_ev.size() >= 2 * (first + count);
     for (int64_t b = first; b < first + count; ++b) {
@@ -5037,20 +5119,29 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         queue_bounds(g, q, b, bstart, blen);
         const int T = sched ? choose_team(g, blen) : T0;
         const int teams = EV_WARPS / T;
-        uint32_t *ctr = g->lit_ctr + 4 * b;
+        uint32_t *ctr = g->lit_ctr + 8 * b;
         RunArgs ab = a;
         ab.ntouched = ctr + 2;
         ab.nitems = ctr + 3;
         if (prof) record_event(g, g->prof_ev[2 * b], capturing);
         const unsigned grid = (unsigned)((blen + teams - 1) / teams);
+        const LitOver ov{reinterpret_cast<int2 *>(g->lit_over), reinterpret_cast<int2 *>(g->lit_over) + g->lit_qcap, ctr,
+                         g->lit_used + b};
+        const bool inblock = grid <= 2 * (unsigned)num_sms();
         switch (T) {
-        case 1: launch_pdl(k_lit_eval<1>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ctr, g->lit_over); break;
-        case 2: launch_pdl(k_lit_eval<2>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ctr, g->lit_over); break;
-        case 4: launch_pdl(k_lit_eval<4>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ctr, g->lit_over); break;
-        default: launch_pdl(k_lit_eval<8>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ctr, g->lit_over); break;
+        case 1: launch_pdl(inblock ? k_lit_eval<1, true> : k_lit_eval<1, false>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ov); break;
+        case 2: launch_pdl(inblock ? k_lit_eval<2, true> : k_lit_eval<2, false>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ov); break;
+        case 4: launch_pdl(inblock ? k_lit_eval<4, true> : k_lit_eval<4, false>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ov); break;
+        default: launch_pdl(inblock ? k_lit_eval<8, true> : k_lit_eval<8, false>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ov); break;
         }
-        launch_pdl(k_lit_big, std::min<unsigned>(big_grid, (unsigned)blen), EV_THREADS, LIT_SMEM, g->stream, ab,
-                   bstart, ctr, (const int32_t *)g->lit_over, g->lit_used + b);
+        if (!inblock) {
+            if (T < LIT_MID) {
+                launch_pdl(k_lit_mid, std::min<unsigned>(mid_grid, (unsigned)blen), EV_THREADS, LIT_SMEM, g->stream, ab, bstart, ov);
+                ++g->launches;
+            }
+            launch_pdl(k_lit_big, std::min<unsigned>(big_grid, (unsigned)blen), EV_THREADS, LIT_SMEM, g->stream, ab, bstart, ov);
+            ++g->launches;
+        }
         const int64_t f0 = g->lh_fq.empty() ? 0 : g->lh_fq[(size_t)b];
         const int64_t nf = g->lh_fq.empty() ? 0 : g->lh_fq[(size_t)b + 1] - f0;
         if (nf > 0) {
@@ -5070,7 +5161,7 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         launch_pdl(k_lit_apply, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
         k_lit_fsum<<<(unsigned)std::min<int64_t>(2 * (int64_t)blen, 4 * (int64_t)num_sms()), EV_THREADS, 0,
                      g->stream>>>(ab, g->touched, ctr + 2, 0);
-        g->launches += 4;
+        g->launches += 3;
     }
     LF_LAUNCHED();
 }
@@ -5107,15 +5198,15 @@ void ensure_lit(lf_graph *g, int64_t q, int64_t nb) {
         g->lit_apacc = dalloc_n<int32_t>(g, 4 * q);
         LF_CUDA(cudaMemsetAsync(g->lit_apacc, 0, (size_t)(4 * q) * 4, g->stream));
         g->lit_qcap = q;
-        g->lit_over = dalloc_n<int32_t>(g, q);
+        g->lit_over = dalloc_n<int32_t>(g, 4 * q);   // two lists of (position, entries)
         g->touched = dalloc_n<int32_t>(g, 2 * q);
         drop_graph(g);
     }
-    if (g->lit_ctr_cap < 4 * nb) {
+    if (g->lit_ctr_cap < 8 * nb) {
         if (g->lit_ctr) dfree(g, g->lit_ctr);
         if (g->lit_used) dfree(g, g->lit_used);
-        g->lit_ctr_cap = 4 * nb;
-        g->lit_ctr = dalloc_n<uint32_t>(g, 4 * nb);
+        g->lit_ctr_cap = 8 * nb;
+        g->lit_ctr = dalloc_n<uint32_t>(g, 8 * nb);
         g->lit_used = dalloc_n<unsigned long long>(g, nb);
         drop_graph(g);
     }
@@ -5394,7 +5485,7 @@ void launch_lit_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int
     unsigned long long *used = g->lit_used;
     const int64_t *qstart = nullptr;
     a.items = nullptr;
-    LF_CUDA(cudaMemsetAsync(ctr + 4 * first, 0, (size_t)(4 * count) * sizeof(uint32_t), g->stream));
+    LF_CUDA(cudaMemsetAsync(ctr + 8 * first, 0, (size_t)(8 * count) * sizeof(uint32_t), g->stream));
     LF_CUDA(cudaMemsetAsync(used + first, 0, (size_t)count * sizeof(unsigned long long), g->stream));
     void *args[] = {&a, &qstart, &q, &first, &count, &ctr, &used, &spin, &inject, &flags, &epoch, &bar_mode};
     if (e0) LF_CUDA(cudaEventRecord(e0, g->stream));
