@@ -252,25 +252,19 @@ struct lf_graph {
     unsigned long long *lit_used = nullptr;   // per queue: global table slots handed out
     void *lg_area = nullptr;              // global tables: lg_cap slots of 16 bytes
     unsigned long long lg_cap = 0;
-    int64_t lg_plan_q = -1, lg_plan_sched = -1;
-    int32_t lg_plan_K = 0;
-    // hubs under the paper's gain: per hub its queue position, table offset
-    // and size, survivor-list offset, slot items, best lower ends, counters;
-    // fill items and slot items of all queues (offsets per queue on the host);
-    // the tables and survivor lists shared by the queues
+    // hubs under the paper's gain (see LitHubPlan): per hub its queue position,
+    // areas, first chunk item, entries, best lower ends, listed candidates; chunk
+    // and part items of all queues (offsets per queue on the host); the entries,
+    // their groups' offsets and the candidate lists, shared by the queues
     int64_t lh_plan_q = -1, lh_plan_sched = -1;
     int32_t lh_plan_K = 0;
     int64_t lh_n = 0;
-    std::vector<int64_t> lh_fq, lh_sq, lh_hq;
-    uint32_t *lh_heff = nullptr;
-    int32_t *lh_pos = nullptr, *lh_nsr = nullptr, *lh_fh = nullptr, *lh_fc = nullptr, *lh_sh = nullptr,
-            *lh_sr = nullptr, *lh_svc = nullptr;
-    int64_t *lh_toff = nullptr, *lh_soff = nullptr;
-    uint32_t *lh_tcap = nullptr, *lh_ns = nullptr, *lh_svv = nullptr;
-    int32_t *lh_lb = nullptr;
-    float *lh_svl = nullptr;
-    void *lh_tab = nullptr;               // tables: 16 bytes per slot
-    int64_t lh_tab_cap = 0;
+    std::vector<int64_t> lh_fq, lh_pq, lh_hq;
+    int32_t *lh_pos = nullptr, *lh_fh = nullptr, *lh_fc = nullptr, *lh_ph = nullptr, *lh_pp = nullptr,
+            *lh_lb = nullptr, *lh_ent = nullptr, *lh_cand = nullptr;
+    int64_t *lh_eoff = nullptr, *lh_fbase = nullptr;
+    uint32_t *lh_total = nullptr, *lh_ns = nullptr, *lh_seg = nullptr;
+    int64_t lh_area = 0;                  // entries of the areas
     // second stream: hub chunks run beside the other evaluation kernels of a queue
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;

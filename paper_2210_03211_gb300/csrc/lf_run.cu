@@ -2128,7 +2128,8 @@ __device__ __forceinline__ void lit_screen(const RunArgs &a, int32_t C, uint32_t
 // Mean of k_lit_eval over the queues, with the lists of lit_eval_shared: 3.07M nodes,
 // q 65,536: 530 -> 379 us; 767k nodes, q 16,384: 140 -> 106 us; 335k nodes, q 1,024:
 // 27.6 -> 21.7 us (cold caches).
-template <int R, typename Fn>
+// (SIZES = false: n is not loaded.)
+template <int R, bool SIZES, typename Fn>
 __device__ __forceinline__ void lit_warp_entries(const RunArgs &a, int64_t qb, int64_t qe, unsigned long long &pb,
                                                  bool count_bytes, Fn &&fn) {
     const int lane = threadIdx.x & 31;
@@ -2179,7 +2180,7 @@ __device__ __forceinline__ void lit_warp_entries(const RunArgs &a, int64_t qb, i
             for (int u = 0; u < R; ++u) {
                 if (e0 + 32 * u + lane < total && !dbg_ok(a, C[u] >= 0 && C[u] < a.nnodes && ky[u] >= 0 && ky[u] <= dj[u]))
                     C[u] = -1;
-                n[u] = C[u] >= 0 ? __ldcg(&a.comm[C[u]].n) : 0;
+                n[u] = SIZES && C[u] >= 0 ? __ldcg(&a.comm[C[u]].n) : 0;
             }
 #pragma unroll
             for (int u = 0; u < R; ++u)
@@ -2420,7 +2421,7 @@ __device__ __forceinline__ bool lit_fill(const RunArgs &a, const LitNode &ln, in
     {   // each warp of the team takes a contiguous share of the neighbours
         const int64_t deg = ln.end - ln.beg, per = (deg + T - 1) / T;
         const int64_t qb = ln.beg + min(deg, (int64_t)w_in * per), qe = ln.beg + min(deg, (int64_t)(w_in + 1) * per);
-        lit_warp_entries<T == EV_WARPS ? 2 : 4>(a, qb, qe, pb, count_bytes, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
+        lit_warp_entries<T == EV_WARPS ? 2 : 4, true>(a, qb, qe, pb, count_bytes, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
             if (P > 1 && (int)part_of(C, P) != p) return;
             const int slot = lit_insert(keys, vals, hm, C);
             if (slot < 0) {
@@ -3138,220 +3139,355 @@ __global__ void __launch_bounds__(EV_THREADS, 3) k_lit_big(RunArgs a, int64_t bs
 }
 
 // ---------------------------------------------------------------------------
-// Hubs under the paper's gain: a queued node of degree > LIT_HUB_DEG is
-// evaluated by many blocks over one table in global memory (planned per
-// queue for the worst case, pow2 >= 2 (d+1) K slots): k_lh_fill (one block per
-// 1024 neighbours: counts, own flags, FP32 corrections), k_lh_bound (one
-// block per 4096 slots: brackets, the hub's best lower ends by an
-// order-preserving integer max), k_lh_mark (one block per 4096 slots:
-// survivors listed, slots cleared) and k_lh_decide (one block per hub: a lone
-// survivor with a positive lower end, or the survivors' exact sums; those of
-// large communities by the whole block, with the hub's adjacency searched
-// through a fence in shared memory).  Team and block kernels skip these nodes.
+// Hubs under the paper's gain: a queued node of degree > LIT_HUB_DEG has more
+// entries than a block's table holds.  Its entries are partitioned by community
+// instead of meeting in one table in global memory (three global atomics per
+// entry on three sectors, then two scans of a table sized for the worst case):
+//   k_lh_count    a block per LH_CHUNK neighbours: the hub's number of entries,
+//                 which sets its number of parts (LH_PART entries each);
+//   k_lh_scatter  a block per LH_CHUNK neighbours: the entries (C, deg(y,C), deg(y))
+//                 written grouped by the part of C, with the groups' offsets;
+//   k_lh_part     a block per part: the groups of all chunks into a table in shared
+//                 memory, brackets, the hub's best lower ends raised (order-
+//                 preserving integer max), and of its candidates those listed that
+//                 the best so far does not rule out -- a handful, so the table
+//                 never leaves the block;
+//   k_lh_decide   a block per hub: the listed ones that the final best lower ends
+//                 leave, a lone survivor with a positive lower end, or the
+//                 survivors' exact sums; those of large communities by the whole
+//                 block, with the hub's adjacency searched through a fence in
+//                 shared memory.
+// Team and block kernels skip these nodes.
+// Mean over the queues that have hubs, all kernels but the decision: 767k nodes, q 16,384:
+// 1,060 -> 475 us; 3.07M nodes, q 65,536: 1,900 -> 1,130 us (cold caches).
 // ---------------------------------------------------------------------------
 constexpr int LIT_HUB_DEG = 1024;
-constexpr int LH_CHUNK = 1024;       // neighbours per fill block
-constexpr int LH_SLOTS = 4096;       // table slots per bracket / mark block
+constexpr int LH_CHUNK = 1024;       // neighbours per counting / scattering block
+constexpr int LH_PART = 1536;        // entries per part (more beyond LH_PARTS parts)
+constexpr int LH_PARTS = 128;
+constexpr uint32_t LH_SLOTS = 4096;  // table slots of a part's block
 
 struct LitHubPlan {
     const int32_t *pos;       // per hub: its position in the queue
-    const int64_t *toff;      // per hub: first slot of its table
-    const uint32_t *tcap;     // per hub: table slots
-    const int64_t *soff;      // per hub: first entry of its survivor list (tcap/2 entries)
-    const int32_t *fh, *fc;   // fill items of every queue: hub, chunk
-    const int32_t *sh, *sr;   // slot items of every queue: hub, range
-    const int32_t *nsr;       // per hub: its slot items (worst case)
-    uint32_t *heff;           // per hub: table slots used in this queue
+    const int64_t *eoff;      // per hub: first entry of its areas ((d+1) K entries)
+    const int64_t *fbase;     // per hub: its first chunk item
+    const int32_t *fh, *fc;   // chunk items of every queue: hub, chunk
+    const int32_t *ph, *pp;   // part items of every queue: hub, part (worst case)
+    uint32_t *total;          // per hub: entries in this queue (zero between queues)
     int32_t *lb;              // per hub: best lower ends (join, leave), order-preserving
-    uint32_t *ns;             // per hub: survivors listed
-    int32_t *sv_c;            // survivor lists: community, count word, lower end
-    uint32_t *sv_v;
-    float *sv_l;
-    int32_t *keys;            // tables: keys, counts, FP32 corrections (then E), X
-    uint32_t *vals;
-    float *hs;
-    float *dv;
+    uint32_t *ns;             // per hub: candidates listed
+    uint32_t *seg;            // per chunk item: offsets of its LH_PARTS groups
+    int32_t *ec, *ek, *ed;    // entries: community, deg(y,C), deg(y)
+    int32_t *sv_c;            // candidate lists: community, count word (SURV_FLAG: the lower
+    uint32_t *sv_v;           // end is positive), upper end
+    float *sv_u;
 };
 
-// Each hub's table size for this queue: pow2 >= 2 (own row + neighbours'
-// rows), at least LH_SLOTS, at most the planned worst case (one block per hub).
-__global__ void __launch_bounds__(256) k_lh_size(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t h0, int64_t nh) {
-    __shared__ long long part[8];
-    const int64_t h = h0 + blockIdx.x;
-    if (blockIdx.x >= nh) return;
-    const int32_t x = a.order[bstart + hp.pos[h]];
-    long long b = threadIdx.x == 0 ? __ldcg(&a.nmem[x]) : 0;
-    for (int64_t q = a.off[x] + threadIdx.x; q < a.off[x + 1]; q += blockDim.x) b += __ldcg(&a.nmem[a.adj[q]]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(FULL, b, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = b;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long t = 0;
-        for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2) t += part[k2];
-        unsigned long long H = LH_SLOTS;
-        while ((long long)H < 2 * t && H < hp.tcap[h]) H <<= 1;
-        hp.heff[h] = (uint32_t)H;
-    }
+__device__ __forceinline__ int lh_parts(uint32_t total) {
+    return (int)min((uint32_t)LH_PARTS, max(1u, (total + LH_PART - 1) / LH_PART));
 }
 
-__global__ void __launch_bounds__(256) k_lh_fill(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t first) {
+__device__ __forceinline__ int lh_part_of(int32_t C, int P) {
+    return (int)__umulhi(hash32((uint32_t)C ^ 0x9e3779b9u), (uint32_t)P);
+}
+
+__global__ void __launch_bounds__(256) k_lh_count(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t first) {
+    const int64_t it = first + blockIdx.x;
+    const int h = hp.fh[it], c = hp.fc[it];
+    const int32_t x = a.order[bstart + hp.pos[h]];
+    const int64_t cb = a.off[x] + (int64_t)c * LH_CHUNK, ce = min(a.off[x + 1], cb + LH_CHUNK);
+    int b = 0;
+#pragma unroll
+    for (int u = 0; u < LH_CHUNK / 256; ++u) {
+        const int64_t q = cb + u * 256 + threadIdx.x;
+        if (q < ce) b += __ldcg(&a.nmem[a.adj[q]]);
+    }
+    b = __reduce_add_sync(FULL, b);
+    if ((threadIdx.x & 31) == 0 && b) atomicAdd(&hp.total[h], (uint32_t)b);
+}
+
+__global__ void __launch_bounds__(256) k_lh_scatter(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t first) {
+    __shared__ int s_cur[LH_PARTS];
     const int64_t it = first + blockIdx.x;
     const int h = hp.fh[it], c = hp.fc[it];
     const int32_t x = a.order[bstart + hp.pos[h]];
     const int64_t beg = a.off[x], end = a.off[x + 1];
-    const int64_t t0 = hp.toff[h];
-    const uint32_t hm = __ldcg(&hp.heff[h]) - 1;
-    int32_t *keys = hp.keys + t0;
-    uint32_t *vals = hp.vals + t0;
-    float *hs = hp.hs + t0;
-    const int32_t cx = __ldcg(&a.nmem[x]);
-    const int32_t *rowx = a.mem + (int64_t)x * a.K;
-    if (c == 0)
-        for (int j = threadIdx.x; j < cx; j += blockDim.x)
-            if (!ht_insert(keys, vals, hm, __ldcg(&rowx[j]), 0u, true)) atomicOr(&a.ds->err, DERR_CHECK);
+    const int P = lh_parts(__ldcg(&hp.total[h]));
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x < LH_PARTS) s_cur[threadIdx.x] = 0;
+    __syncthreads();
     unsigned long long pb = 0;
     const int64_t cb = beg + (int64_t)c * LH_CHUNK, ce = min(end, cb + LH_CHUNK);
-    {   // each warp takes a contiguous eighth of the chunk
-        const int64_t per = (ce - cb + 7) / 8, w = threadIdx.x >> 5;
-        const int64_t qb = min(ce, cb + w * per), qe = min(ce, cb + (w + 1) * per);
-        lit_warp_entries<4>(a, qb, qe, pb, a.profile != 0, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
-            const int slot = lit_insert(keys, vals, hm, C);
-            if (slot < 0) {   // cannot happen: the table holds 2 (d+1) K slots
-                atomicOr(&a.ds->err, DERR_CHECK);
-                return;
-            }
-            const float hv = row_find(rowx, cx, C) >= 0 ? lit_h_leave32(ky, dy, n) : lit_h_join32(ky, dy, n);
-            if (hv != 0.f) atomicAdd(&hs[slot], hv);
-        });
+    // each warp takes a contiguous eighth of the chunk
+    const int64_t per = (ce - cb + 7) / 8;
+    const int64_t qb = min(ce, cb + w * per), qe = min(ce, cb + (w + 1) * per);
+    lit_warp_entries<4, false>(a, qb, qe, pb, a.profile != 0, [&](int32_t C, uint32_t, uint32_t, uint32_t) {
+        atomicAdd(&s_cur[lh_part_of(C, P)], 1);
+    });
+    __syncthreads();
+    if (w == 0) {   // offsets of the groups: LH_PARTS / 32 counters a lane
+        constexpr int PER = LH_PARTS / 32;
+        int v[PER], sum = 0;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            v[u] = s_cur[lane * PER + u];
+            sum += v[u];
+        }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += t;
+        }
+        int run = inc - sum;
+        uint32_t *seg = hp.seg + it * (LH_PARTS + 1);
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            s_cur[lane * PER + u] = run;
+            seg[lane * PER + u] = (uint32_t)run;
+            run += v[u];
+        }
+        if (lane == 31) seg[LH_PARTS] = (uint32_t)run;
     }
+    __syncthreads();
+    const int64_t area = hp.eoff[h] + (int64_t)c * LH_CHUNK * a.K;
+    lit_warp_entries<4, false>(a, qb, qe, pb, false, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t) {
+        const int64_t e = area + atomicAdd(&s_cur[lh_part_of(C, P)], 1);
+        hp.ec[e] = C;
+        hp.ek[e] = (int32_t)ky;
+        hp.ed[e] = (int32_t)dy;
+    });
     if (a.profile) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) pb += __shfl_down_sync(FULL, pb, o);
-        if ((threadIdx.x & 31) == 0 && pb) atomicAdd(&a.ds->prof_bytes, pb);
+        if (lane == 0 && pb) atomicAdd(&a.ds->prof_bytes, pb);
     }
 }
 
-__global__ void __launch_bounds__(256) k_lh_bound(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t first) {
-    __shared__ float red[2][8];
+// Second hash of a community, 16 bits: a part whose distinct communities overflow
+// the table is done in ranges of it.
+__device__ __forceinline__ uint32_t lh_range_of(int32_t C) { return hash32((uint32_t)C * 0x9e3779b1u + 0x7f4a7c15u) >> 16; }
+
+constexpr size_t LH_SMEM = (size_t)LH_SLOTS * 12 + (size_t)LH_SLOTS * 2;
+
+__global__ void __launch_bounds__(256, 3) k_lh_part(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t first) {
+    extern __shared__ double lh_dyn[];
+    __shared__ float s_red[2][8];
+    __shared__ float s_lb[2];
+    __shared__ uint32_t s_cnt;
+    __shared__ int s_n, s_over;
+    LitTable t;
+    t.keys = reinterpret_cast<int32_t *>(lh_dyn);
+    t.vals = reinterpret_cast<uint32_t *>(t.keys + LH_SLOTS);
+    t.aux = reinterpret_cast<int32_t *>(t.vals + LH_SLOTS);
+    t.list = reinterpret_cast<uint16_t *>(t.aux + LH_SLOTS);
+    float *hs = reinterpret_cast<float *>(t.aux);
     const int64_t it = first + blockIdx.x;
-    const int h = hp.sh[it], r = hp.sr[it];
+    const int h = hp.ph[it], p = hp.pp[it];
+    const int P = lh_parts(__ldcg(&hp.total[h]));
+    if (p >= P) return;
     const int32_t x = a.order[bstart + hp.pos[h]];
     const int32_t d = (int32_t)(a.off[x + 1] - a.off[x]);
-    const int64_t t0 = hp.toff[h];
-    const uint32_t lo = (uint32_t)r * LH_SLOTS, hi = min(__ldcg(&hp.heff[h]), lo + LH_SLOTS);
-    if (lo >= hi) return;   // beyond this queue's table
-    float lbj = -INFINITY, lbl = -INFINITY;
-    unsigned long long nc = 0;
-    for (uint32_t s = lo + threadIdx.x; s < hi; s += blockDim.x) {
-        const int32_t C = hp.keys[t0 + s];
-        if (C == EMPTY_KEY) continue;
-        const uint32_t v = hp.vals[t0 + s];
-        float X, E;
-        lit_screen(a, C, v, d, hp.hs[t0 + s], X, E);
-        hp.dv[t0 + s] = X;
-        hp.hs[t0 + s] = E;
-        const float L = X - E;
-        if (v & OWN_FLAG) lbl = fmaxf(lbl, L);
-        else lbj = fmaxf(lbj, L);
-        ++nc;
-    }
-    lbj = warp_max_f(lbj);
-    lbl = warp_max_f(lbl);
+    const int nf = (d + LH_CHUNK - 1) / LH_CHUNK;
+    const uint32_t *seg0 = hp.seg + hp.fbase[h] * (LH_PARTS + 1) + p;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[0][w] = lbj;
-        red[1][w] = lbl;
-    }
-    if (a.profile) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) nc += __shfl_down_sync(FULL, nc, o);
-        if (lane == 0 && nc) {
-            atomicAdd(&a.ds->prof_cands, nc);
-            atomicAdd(&a.ds->prof_bytes, 40ull * nc);
-        }
-    }
+    const int32_t cx = __ldcg(&a.nmem[x]);
+    const int32_t *rowx = a.mem + (int64_t)x * a.K;
+    if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
-    if (threadIdx.x < 2) {
-        float m = -INFINITY;
-        for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2) m = fmaxf(m, red[threadIdx.x][k2]);
-        if (m > -INFINITY) atomicMax(&hp.lb[2 * h + threadIdx.x], f2ord(m));
+    uint32_t cnt = 0;
+    for (int c = threadIdx.x; c < nf; c += 256) {
+        const uint32_t *sg = seg0 + (int64_t)c * (LH_PARTS + 1);
+        cnt += __ldcg(sg + 1) - __ldcg(sg);
+    }
+    cnt = __reduce_add_sync(FULL, cnt);
+    if (lane == 0 && cnt) atomicAdd(&s_cnt, cnt);
+    __syncthreads();
+    cnt = s_cnt + (uint32_t)cx;
+    uint32_t H = 32;
+    while (H < LH_SLOTS && H < 2 * cnt) H <<= 1;
+    const uint32_t hm = H - 1;
+    const int split = nf >= 8 ? 1 : nf >= 4 ? 2 : nf >= 2 ? 4 : 8;   // strips of a chunk's group, for eight warps
+    for (uint32_t lo = 0, width = 65536; lo < 65536;) {   // ranges of the second hash: one unless the table overflows
+        for (uint32_t s = threadIdx.x; s < H; s += 256) {
+            t.keys[s] = EMPTY_KEY;
+            t.vals[s] = 0u;
+            hs[s] = 0.f;
+        }
+        if (threadIdx.x == 0) s_n = s_over = 0;
+        __syncthreads();
+        bool ok = true;
+        for (int j = threadIdx.x; j < cx; j += 256) {
+            const int32_t C = __ldcg(&rowx[j]);
+            if (lh_part_of(C, P) == p && lh_range_of(C) - lo < width) ok &= ht_insert(t.keys, t.vals, hm, C, 0u, true);
+        }
+        __syncthreads();
+        for (int u = w; u < nf * split; u += 8) {
+            const int c = u / split, strip = u % split;
+            const uint32_t *sg = seg0 + (int64_t)c * (LH_PARTS + 1);
+            const int64_t base = hp.eoff[h] + (int64_t)c * LH_CHUNK * a.K;
+            const int64_t e1 = base + __ldcg(sg + 1);
+            for (int64_t e0 = base + __ldcg(sg) + strip * 128; e0 < e1; e0 += 128 * split) {
+                int32_t C[4], k[4], dy[4], n[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int64_t e = e0 + r * 32 + lane;
+                    C[r] = e < e1 ? __ldcg(&hp.ec[e]) : -1;
+                    k[r] = e < e1 ? __ldcg(&hp.ek[e]) : 0;
+                    dy[r] = e < e1 ? __ldcg(&hp.ed[e]) : 0;
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (width < 65536 && C[r] >= 0 && lh_range_of(C[r]) - lo >= width) C[r] = -1;
+                    n[r] = C[r] >= 0 ? __ldcg(&a.comm[C[r]].n) : 0;
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (C[r] < 0) continue;
+                    const int slot = lit_insert(t.keys, t.vals, hm, C[r]);
+                    if (slot < 0) {
+                        ok = false;
+                        continue;
+                    }
+                    const float hv = (t.vals[slot] & OWN_FLAG)
+                                         ? lit_h_leave32((uint32_t)k[r], (uint32_t)dy[r], (uint32_t)n[r])
+                                         : lit_h_join32((uint32_t)k[r], (uint32_t)dy[r], (uint32_t)n[r]);
+                    if (hv != 0.f) atomicAdd(&hs[slot], hv);
+                }
+                if (!ok) break;
+            }
+        }
+        if (!ok) s_over = 1;
+        __syncthreads();
+        if (s_over) {   // more distinct communities than slots: half the range (one hash value always fits in practice)
+            __syncthreads();
+            if (width == 1) {
+                if (threadIdx.x == 0) atomicOr(&a.ds->err, DERR_CHECK);
+                return;
+            }
+            width >>= 1;
+            continue;
+        }
+        // the used slots listed, bracketed, the hub's best lower ends raised
+        for (uint32_t b0 = (uint32_t)w * 32; b0 < H; b0 += 256) {
+            const bool used = t.keys[b0 + lane] != EMPTY_KEY;
+            const unsigned m = __ballot_sync(FULL, used);
+            int n0 = 0;
+            if (lane == 0 && m) n0 = atomicAdd(&s_n, __popc(m));
+            n0 = __shfl_sync(FULL, n0, 0);
+            if (used) t.list[n0 + __popc(m & lanemask_lt())] = (uint16_t)(b0 + lane);
+        }
+        __syncthreads();
+        const int ncand = s_n;
+        float lbj = -INFINITY, lbl = -INFINITY;
+        for (int c = threadIdx.x; c < ncand; c += 256) {
+            const int s = t.list[c];
+            const uint32_t v = t.vals[s];
+            float X, E;
+            lit_screen(a, t.keys[s], v, d, hs[s], X, E);
+            hs[s] = X + E;
+            if (X - E > 0.f) t.vals[s] = v | SURV_FLAG;   // here: the lower end is positive
+            if (v & OWN_FLAG) lbl = fmaxf(lbl, X - E);
+            else lbj = fmaxf(lbj, X - E);
+        }
+        lbj = warp_max_f(lbj);
+        lbl = warp_max_f(lbl);
+        if (lane == 0) {
+            s_red[0][w] = lbj;
+            s_red[1][w] = lbl;
+        }
+        if (a.profile && threadIdx.x == 0 && ncand) {
+            atomicAdd(&a.ds->prof_cands, (unsigned long long)ncand);
+            atomicAdd(&a.ds->prof_bytes, 40ull * (unsigned long long)ncand);
+        }
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            float m = -INFINITY;
+            for (int k2 = 0; k2 < 8; ++k2) m = fmaxf(m, s_red[threadIdx.x][k2]);
+            int32_t *g = &hp.lb[2 * h + threadIdx.x];
+            const int32_t old = m > -INFINITY ? atomicMax(g, f2ord(m)) : __ldcg(g);
+            s_lb[threadIdx.x] = fmaxf(m, ord2f(old));
+        }
+        __syncthreads();
+        lbj = s_lb[0];
+        lbl = s_lb[1];
+        for (int c = threadIdx.x; c < ncand; c += 256) {
+            const int s = t.list[c];
+            const uint32_t v = t.vals[s];
+            const float U = hs[s];
+            if (!a.screen || (U > 0.f && U >= ((v & OWN_FLAG) ? lbl : lbj))) {
+                const int64_t e = hp.eoff[h] + atomicAdd(&hp.ns[h], 1u);   // at most one per distinct community
+                hp.sv_c[e] = t.keys[s];
+                hp.sv_v[e] = v;
+                hp.sv_u[e] = U;
+            }
+        }
+        __syncthreads();
+        lo += width;
     }
 }
 
 constexpr int LH_FENCE = 2048;        // fence entries of a hub's adjacency (exact sums)
 constexpr int64_t LH_BLOCK_MEMBERS = 256;   // survivors of larger communities are summed by the whole block
 
-// Survivors of a hub's bracket test listed (one block per 4096 slots), the
-// table left clean for the hub's next queue.
-__global__ void __launch_bounds__(256, 4) k_lh_mark(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t first) {
-    const int64_t it = first + blockIdx.x;
-    const int h = hp.sh[it], r = hp.sr[it];
-    const int64_t t0 = hp.toff[h], so = hp.soff[h];
-    const float lbj = ord2f(__ldcg(&hp.lb[2 * h])), lbl = ord2f(__ldcg(&hp.lb[2 * h + 1]));
-    const uint32_t heff = __ldcg(&hp.heff[h]);
-    const uint32_t lo = (uint32_t)r * LH_SLOTS, hi = min(heff, lo + LH_SLOTS);
-    if (lo >= hi) return;   // beyond this queue's table
-    for (uint32_t s = lo + threadIdx.x; s < hi; s += blockDim.x) {
-        const int32_t C = hp.keys[t0 + s];
-        if (C == EMPTY_KEY) continue;
-        const uint32_t v = hp.vals[t0 + s];
-        const float X = hp.dv[t0 + s], E = hp.hs[t0 + s];
-        const float U = X + E;
-        const bool own = (v & OWN_FLAG) != 0;
-        if (!a.screen || (U > 0.f && U >= (own ? lbl : lbj))) {
-            const uint32_t e = atomicAdd(&hp.ns[h], 1u);
-            hp.sv_c[so + e] = C;
-            hp.sv_v[so + e] = v;
-            hp.sv_l[so + e] = X - E;
-        }
-        hp.keys[t0 + s] = EMPTY_KEY;   // the table is left clean for the hub's next queue
-        hp.vals[t0 + s] = 0u;
-        hp.hs[t0 + s] = 0.f;
-    }
-}
+// A hub's decision from its listed candidates (one block per hub of the
+// queue), of which the hub's best lower ends, now final, leave the survivors: a
+// lone one with a positive lower end wins; otherwise the survivors' gains are
+// summed exactly and compared.
+constexpr int LH_KEEP = 256;   // survivors kept in shared memory (more are tested again as they are met)
 
-// A hub's decision from its listed survivors (one block per hub of the
-// queue): a lone survivor with a positive lower end wins; otherwise the
-// survivors' gains are summed exactly and compared.
 __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int64_t bstart, int64_t h0, int64_t nh) {
     __shared__ unsigned long long acc_s[8 * SACC_CHUNKS];
     __shared__ int32_t fence[LH_FENCE];
     __shared__ double s_g;
     __shared__ double bg[2][8];
     __shared__ int32_t bc[2][8], bk[2][8];
+    __shared__ uint32_t s_keep[LH_KEEP];
+    __shared__ int s_cnt[2];         // survivors: joins, leaves
+    __shared__ uint32_t s_one[2];    // one of each kind
     if (blockIdx.x >= nh) return;
     const int64_t h = h0 + blockIdx.x;
     const int32_t i = hp.pos[h];
     const int32_t x = a.order[bstart + i];
     const int32_t d = (int32_t)(a.off[x + 1] - a.off[x]);
-    const int64_t so = hp.soff[h];
+    const int64_t so = hp.eoff[h];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t ns = __ldcg(&hp.ns[h]);
-    int cj = 0, cl = 0;
-    int32_t Cj = -1, Cl = -1, kj = 0, kl = 0;
-    float Lj = 0.f, Ll = 0.f;
-    for (uint32_t e = 0; e < ns; ++e) {   // every thread reads the (short) list
-        const uint32_t v = __ldcg(&hp.sv_v[so + e]);
-        const int32_t C = __ldcg(&hp.sv_c[so + e]);
-        const float L = __ldcg(&hp.sv_l[so + e]);
-        if (v & OWN_FLAG) {
-            if (cl++ == 0) { Cl = C; kl = (int32_t)(v & CNT_MASK); Ll = L; }
-        } else {
-            if (cj++ == 0) { Cj = C; kj = (int32_t)(v & CNT_MASK); Lj = L; }
+    const uint32_t nlist = __ldcg(&hp.ns[h]);
+    const float lbj = ord2f(__ldcg(&hp.lb[2 * h])), lbl = ord2f(__ldcg(&hp.lb[2 * h + 1]));
+    auto survives = [&](uint32_t e) {
+        const float U = __ldcg(&hp.sv_u[so + e]);
+        return !a.screen || U >= ((__ldcg(&hp.sv_v[so + e]) & OWN_FLAG) ? lbl : lbj);   // listed: U > 0
+    };
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    for (uint32_t e = threadIdx.x; e < nlist; e += blockDim.x)
+        if (survives(e)) {
+            const int own = (__ldcg(&hp.sv_v[so + e]) & OWN_FLAG) ? 1 : 0;
+            atomicAdd(&s_cnt[own], 1);
+            s_one[own] = e;
         }
-    }
+    __syncthreads();
+    const int cj = s_cnt[0], cl = s_cnt[1];
     Best bj{0.0, -1, 0}, bl{0.0, -1, 0};
     bool do_j = cj > 0, do_l = cl > 0;
-    if (a.screen && cj == 1 && Lj > 0.f) {
-        bj = Best{INFINITY, Cj, kj};
-        do_j = false;
+    if (cj == 1) {
+        const uint32_t v = __ldcg(&hp.sv_v[so + s_one[0]]);
+        do_j = lit_settle(a, 1, __ldcg(&hp.sv_c[so + s_one[0]]), (int32_t)(v & CNT_MASK), v & SURV_FLAG, bj);
     }
-    if (a.screen && cl == 1 && Ll > 0.f) {
-        bl = Best{INFINITY, Cl, kl};
-        do_l = false;
+    if (cl == 1) {
+        const uint32_t v = __ldcg(&hp.sv_v[so + s_one[1]]);
+        do_l = lit_settle(a, 1, __ldcg(&hp.sv_c[so + s_one[1]]), (int32_t)(v & CNT_MASK), v & SURV_FLAG, bl);
     }
+    const bool kept = cj + cl <= LH_KEEP;
+    const uint32_t ns = kept ? (uint32_t)(cj + cl) : nlist;
     if (do_j || do_l) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_cnt[0] = 0;
+        __syncthreads();
+        if (kept)
+            for (uint32_t e = threadIdx.x; e < nlist; e += blockDim.x)
+                if (survives(e)) s_keep[atomicAdd(&s_cnt[0], 1)] = e;
+        __syncthreads();
         unsigned long long *acc = acc_s + w * SACC_CHUNKS;
         for (int c2 = lane; c2 < SACC_CHUNKS; c2 += 32) acc[c2] = 0ull;
         // every step-th entry of x's adjacency, for the neighbour tests of the member passes
@@ -3361,7 +3497,9 @@ __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int
         for (int j = threadIdx.x; j < nf; j += blockDim.x) fence[j] = a.adj[xb + (int64_t)j * step];
         __syncthreads();
         // survivors of large communities: one at a time, the whole block over the members
-        for (uint32_t e = 0; e < ns; ++e) {
+        for (uint32_t q = 0; q < ns; ++q) {
+            const uint32_t e = kept ? s_keep[q] : q;
+            if (!kept && !survives(e)) continue;
             const uint32_t v = __ldcg(&hp.sv_v[so + e]);
             const bool own = (v & OWN_FLAG) != 0;
             if (own ? !do_l : !do_j) continue;
@@ -3376,7 +3514,9 @@ __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int
             }
         }
         // the others: a warp each
-        for (uint32_t e = w; e < ns; e += blockDim.x >> 5) {
+        for (uint32_t q = w; q < ns; q += blockDim.x >> 5) {
+            const uint32_t e = kept ? s_keep[q] : q;
+            if (!kept && !survives(e)) continue;
             const uint32_t v = __ldcg(&hp.sv_v[so + e]);
             const bool own = (v & OWN_FLAG) != 0;
             if (own ? !do_l : !do_j) continue;
@@ -3405,6 +3545,7 @@ __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int
         lit_write_action(a, i, d, bj, bl);
         if (a.profile) atomicAdd(&a.ds->prof_bytes, 44ull + 8ull * (unsigned long long)__ldcg(&a.nmem[x]));
         hp.ns[h] = 0u;   // ready for the hub's next queue
+        hp.total[h] = 0u;
         hp.lb[2 * h] = f2ord(-INFINITY);
         hp.lb[2 * h + 1] = f2ord(-INFINITY);
     }
@@ -4817,6 +4958,7 @@ void set_eval_attrs() {
     LF_CUDA(cudaFuncSetAttribute(k_lit_eval<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
     LF_CUDA(cudaFuncSetAttribute(k_lit_eval<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
     LF_CUDA(cudaFuncSetAttribute(k_lit_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lh_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LH_SMEM));
     LF_CUDA(cudaFuncSetAttribute(k_lit_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
 }
 
@@ -4941,31 +5083,18 @@ void launch_batches(lf_graph *g, const RunArgs &a, int64_t q, int64_t first, int
 }
 
 void free_lit_hub_plan(lf_graph *g) {
-    for (int32_t **pp : {&g->lh_pos, &g->lh_nsr, &g->lh_fh, &g->lh_fc, &g->lh_sh, &g->lh_sr, &g->lh_svc})
-        if (*pp) {
-            dfree(g, *pp);
-            *pp = nullptr;
-        }
-    for (int64_t **pp : {&g->lh_toff, &g->lh_soff})
-        if (*pp) {
-            dfree(g, *pp);
-            *pp = nullptr;
-        }
-    for (uint32_t **pp : {&g->lh_tcap, &g->lh_ns, &g->lh_svv, &g->lh_heff})
-        if (*pp) {
-            dfree(g, *pp);
-            *pp = nullptr;
-        }
-    if (g->lh_lb) dfree(g, g->lh_lb);
-    if (g->lh_svl) dfree(g, g->lh_svl);
-    if (g->lh_tab) dfree(g, g->lh_tab);
-    g->lh_lb = nullptr;
-    g->lh_svl = nullptr;
-    g->lh_tab = nullptr;
-    g->lh_tab_cap = 0;
+    auto drop = [&](auto *&p) {
+        if (p) dfree(g, p);
+        p = nullptr;
+    };
+    for (int32_t **pp : {&g->lh_pos, &g->lh_fh, &g->lh_fc, &g->lh_ph, &g->lh_pp, &g->lh_lb, &g->lh_ent, &g->lh_cand})
+        drop(*pp);
+    for (int64_t **pp : {&g->lh_eoff, &g->lh_fbase}) drop(*pp);
+    for (uint32_t **pp : {&g->lh_ns, &g->lh_total, &g->lh_seg}) drop(*pp);
+    g->lh_area = 0;
     g->lh_n = 0;
     g->lh_fq.clear();
-    g->lh_sq.clear();
+    g->lh_pq.clear();
     g->lh_hq.clear();
     g->lh_plan_q = g->lh_plan_sched = -1;
     g->lh_plan_K = 0;
@@ -4977,124 +5106,174 @@ void free_lit_hub_plan(lf_graph *g) {
 // 23.2 / 22.4; 84k nodes q 64 25.0 / 21.9, q 256 36.4 / 27.6.
 constexpr int64_t LIT_LOOP_MAX_Q = 1;
 
-// The hubs of every queue (degree > LIT_HUB_DEG): worst-case tables of
-// pow2 >= 2 (d+1) K slots (K bounds every row), fill items of LH_CHUNK
-// neighbours, slot items of LH_SLOTS slots.  Queues run one after the other,
-// so their tables and survivor lists share one area.
+// The nodes of degree > LIT_HUB_DEG by position in the order the queues take,
+// and per queue the slots of global tables its other nodes could want at most
+// (K bounds every row, so (d+1) K bounds a node's entries).  qstart: queue
+// boundaries of a batch (nb + 1), null for queues of q.  One pass on the device:
+// copied to the host node by node, these plans took 36 ms of a run on 3.07M nodes.
+__global__ void k_lit_plan(const int32_t *order, const int32_t *deg, int64_t len, const int64_t *qstart, int64_t nb,
+                           int64_t q, int32_t K, uint32_t *nhub, int2 *hubs, unsigned long long *want) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < len; p += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t d = deg[order[p]];
+        if (d > LIT_HUB_DEG) {
+            hubs[atomicAdd(nhub, 1u)] = make_int2((int32_t)p, d);
+            continue;
+        }
+        const unsigned long long e = (unsigned long long)(d + 1) * (unsigned)K;
+        if (4 * e <= 3ull * LB_SLOTS) continue;
+        unsigned long long H = 32;
+        while (H < 2 * e) H <<= 1;
+        int64_t b = p / q;
+        if (qstart) {   // the last queue that starts at or before p
+            int64_t lo = 0, hi = nb - 1;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi + 1) >> 1;
+                if (qstart[mid] <= p) lo = mid;
+                else hi = mid - 1;
+            }
+            b = lo;
+        }
+        atomicAdd(&want[b], H);
+    }
+}
+
+// The hubs of every queue: areas of (d+1) K entries (K bounds every row), chunk
+// items of LH_CHUNK neighbours, part items for the worst case.  Queues run one
+// after the other, so they share the areas.  Also the global tables of the other
+// nodes (lg_area), sized for the largest queue.
 void build_lit_hub_plan(lf_graph *g, int64_t q, int64_t nb) {
     if (g->lh_plan_q == q && g->lh_plan_K == g->K && g->lh_plan_sched == g->sched_version) return;
     free_lit_hub_plan(g);
     drop_graph(g);
-    g->lh_plan_q = q;
-    g->lh_plan_K = g->K;
-    g->lh_plan_sched = g->sched_version;
     g->lh_fq.assign((size_t)nb + 1, 0);
-    g->lh_sq.assign((size_t)nb + 1, 0);
+    g->lh_pq.assign((size_t)nb + 1, 0);
     g->lh_hq.assign((size_t)nb + 1, 0);
-    if (g->n == 0 || g->max_deg <= LIT_HUB_DEG) return;
     const int64_t len = g->sched.empty() ? g->n : g->sched.back();
-    std::vector<int32_t> order((size_t)std::max<int64_t>(len, 1)), deg((size_t)g->n);
-    if (len > 0)
-        LF_CUDA(cudaMemcpyAsync(order.data(), g->sched.empty() ? g->order : g->qorder, (size_t)len * 4,
-                                cudaMemcpyDeviceToHost, g->stream));
-    LF_CUDA(cudaMemcpyAsync(deg.data(), g->deg, (size_t)g->n * 4, cudaMemcpyDeviceToHost, g->stream));
-    LF_CUDA(cudaStreamSynchronize(g->stream));
-    std::vector<int32_t> pos, nsr, fh, fc, sh, sr;
-    std::vector<int64_t> toff, soff;
-    std::vector<uint32_t> tcap;
+    std::vector<int2> hubs;
+    unsigned long long cap = 0;
+    if (len > 0 && (g->max_deg > LIT_HUB_DEG || 4 * (int64_t)(g->max_deg + 1) * g->K > 3 * LB_SLOTS)) {
+        // hubs number at most 2m / LIT_HUB_DEG
+        const int64_t most = std::min<int64_t>(len, 2 * g->m / LIT_HUB_DEG + 1);
+        const int64_t words = nb + 1 + (g->sched.empty() ? 0 : nb + 1) + most;
+        unsigned long long *buf = dalloc_n<unsigned long long>(g, words);
+        unsigned long long *want = buf;
+        uint32_t *nhub = reinterpret_cast<uint32_t *>(buf + nb);
+        int2 *dh = reinterpret_cast<int2 *>(buf + nb + 1);
+        int64_t *qs = g->sched.empty() ? nullptr : reinterpret_cast<int64_t *>(buf + nb + 1 + most);
+        LF_CUDA(cudaMemsetAsync(buf, 0, (size_t)(nb + 1) * 8, g->stream));
+        if (qs)
+            LF_CUDA(cudaMemcpyAsync(qs, g->sched.data(), (size_t)(nb + 1) * 8, cudaMemcpyHostToDevice, g->stream));
+        k_lit_plan<<<grid_for(len, 256, 1 << 12), 256, 0, g->stream>>>(g->sched.empty() ? g->order : g->qorder, g->deg,
+                                                                     len, qs, nb, q, g->K, nhub, dh, want);
+        ++g->launches;
+        LF_LAUNCHED();
+        std::vector<unsigned long long> host((size_t)nb + 1);
+        LF_CUDA(cudaMemcpyAsync(host.data(), buf, (size_t)(nb + 1) * 8, cudaMemcpyDeviceToHost, g->stream));
+        LF_CUDA(cudaStreamSynchronize(g->stream));
+        for (int64_t b = 0; b < nb; ++b) cap = std::max(cap, host[(size_t)b]);
+        hubs.resize((size_t)(uint32_t)host[(size_t)nb]);
+        if (!hubs.empty())
+            LF_CUDA(cudaMemcpyAsync(hubs.data(), dh, hubs.size() * sizeof(int2), cudaMemcpyDeviceToHost, g->stream));
+        LF_CUDA(cudaStreamSynchronize(g->stream));
+        dfree(g, buf);
+        std::sort(hubs.begin(), hubs.end(), [](const int2 &u, const int2 &v) { return u.x < v.x; });
+    }
+    // the area is a reservation for the worst case; past 32 MiB + 64 bytes per edge
+    // a node that finds no room takes the multi-pass shared path
+    cap = std::min<unsigned long long>(cap, ((32ull << 20) + 64ull * (unsigned long long)g->m) / 16);
+    if (cap != g->lg_cap) {
+        if (g->lg_area) dfree(g, g->lg_area);
+        g->lg_area = nullptr;
+        g->lg_cap = 0;
+        if (cap) g->lg_area = dalloc(g, (size_t)cap * 16);
+        g->lg_cap = cap;
+    }
+    std::vector<int32_t> pos, fh, fc, ph, pp;
+    std::vector<int64_t> eoff, fbase;
     int64_t area = 0;
+    size_t at = 0;
     for (int64_t b = 0; b < nb; ++b) {
         int64_t qs;
         int32_t ql;
         queue_bounds(g, q, b, qs, ql);
         int64_t used = 0;
-        for (int64_t p = qs; p < qs + ql; ++p) {
-            const int32_t d = deg[(size_t)order[(size_t)p]];
-            if (d <= LIT_HUB_DEG) continue;
-            uint64_t cap = LH_SLOTS;
-            while (cap < 2ull * (uint64_t)(d + 1) * (uint64_t)g->K) cap <<= 1;
+        for (; at < hubs.size() && hubs[at].x < qs + ql; ++at) {
+            const int64_t d = hubs[at].y, most = (d + 1) * g->K;
             const int32_t h = (int32_t)pos.size();
-            pos.push_back((int32_t)(p - qs));
-            toff.push_back(used);
-            soff.push_back(used / 2);
-            tcap.push_back((uint32_t)cap);
-            const int32_t nf = (d + LH_CHUNK - 1) / LH_CHUNK, ns = (int32_t)(cap / LH_SLOTS);
-            nsr.push_back(ns);
-            for (int32_t c = 0; c < nf; ++c) {
+            pos.push_back((int32_t)(hubs[at].x - qs));
+            eoff.push_back(used);
+            fbase.push_back((int64_t)fh.size());
+            for (int32_t c = 0; c < (int32_t)((d + LH_CHUNK - 1) / LH_CHUNK); ++c) {
                 fh.push_back(h);
                 fc.push_back(c);
             }
-            for (int32_t r = 0; r < ns; ++r) {
-                sh.push_back(h);
-                sr.push_back(r);
+            const int32_t parts = (int32_t)std::min<int64_t>(LH_PARTS, (most + LH_PART - 1) / LH_PART);
+            for (int32_t r = 0; r < parts; ++r) {
+                ph.push_back(h);
+                pp.push_back(r);
             }
-            used += (int64_t)cap;
+            used += (most + 31) / 32 * 32;
         }
         g->lh_fq[(size_t)b + 1] = (int64_t)fh.size();
-        g->lh_sq[(size_t)b + 1] = (int64_t)sh.size();
+        g->lh_pq[(size_t)b + 1] = (int64_t)ph.size();
         g->lh_hq[(size_t)b + 1] = (int64_t)pos.size();
         area = std::max(area, used);
     }
     const int64_t H = (int64_t)pos.size();
     g->lh_n = H;
-    if (H == 0) return;
-    auto up = [&](auto *&dst, const auto &v) {
-        using E = typename std::decay<decltype(v[0])>::type;
-        dst = dalloc_n<E>(g, (int64_t)v.size());
-        LF_CUDA(cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, g->stream));
-    };
-    up(g->lh_pos, pos);
-    up(g->lh_nsr, nsr);
-    up(g->lh_fh, fh);
-    up(g->lh_fc, fc);
-    up(g->lh_sh, sh);
-    up(g->lh_sr, sr);
-    up(g->lh_toff, toff);
-    up(g->lh_soff, soff);
-    up(g->lh_tcap, tcap);
-    g->lh_heff = dalloc_n<uint32_t>(g, H);
-    g->lh_ns = dalloc_n<uint32_t>(g, H);
-    LF_CUDA(cudaMemsetAsync(g->lh_ns, 0, (size_t)H * 4, g->stream));
-    {
-        // best lower ends start at -inf (order-preserving: -inf's bits ^ 0x7fffffff)
-        const int32_t ninf = (int32_t)(0xff800000u ^ 0x7fffffffu);
-        std::vector<int32_t> lb((size_t)(2 * H), ninf);
-        up(g->lh_lb, lb);
+    if (H > 0) {
+        auto up = [&](auto *&dst, const auto &v) {
+            using E = typename std::decay<decltype(v[0])>::type;
+            dst = dalloc_n<E>(g, (int64_t)v.size());
+            LF_CUDA(cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, g->stream));
+        };
+        up(g->lh_pos, pos);
+        up(g->lh_fh, fh);
+        up(g->lh_fc, fc);
+        up(g->lh_ph, ph);
+        up(g->lh_pp, pp);
+        up(g->lh_eoff, eoff);
+        up(g->lh_fbase, fbase);
+        g->lh_total = dalloc_n<uint32_t>(g, H);
+        g->lh_ns = dalloc_n<uint32_t>(g, H);
+        LF_CUDA(cudaMemsetAsync(g->lh_total, 0, (size_t)H * 4, g->stream));
+        LF_CUDA(cudaMemsetAsync(g->lh_ns, 0, (size_t)H * 4, g->stream));
+        {
+            // best lower ends start at -inf (order-preserving: -inf's bits ^ 0x7fffffff)
+            const int32_t ninf = (int32_t)(0xff800000u ^ 0x7fffffffu);
+            std::vector<int32_t> lb((size_t)(2 * H), ninf);
+            up(g->lh_lb, lb);
+        }
+        g->lh_seg = dalloc_n<uint32_t>(g, (int64_t)fh.size() * (LH_PARTS + 1));
+        g->lh_area = area;
+        g->lh_ent = dalloc_n<int32_t>(g, 3 * area);
+        g->lh_cand = dalloc_n<int32_t>(g, 3 * area);
+        LF_CUDA(cudaStreamSynchronize(g->stream));
     }
-    g->lh_tab_cap = area;
-    g->lh_tab = dalloc(g, (size_t)area * 16);
-    // keys empty, counts and corrections zero (the X area needs no start value)
-    char *t = static_cast<char *>(g->lh_tab);
-    LF_CUDA(cudaMemsetAsync(t + (size_t)area * 4, 0xff, (size_t)area * 4, g->stream));
-    LF_CUDA(cudaMemsetAsync(t + (size_t)area * 8, 0, (size_t)area * 8, g->stream));
-    g->lh_svc = dalloc_n<int32_t>(g, area / 2);
-    g->lh_svv = dalloc_n<uint32_t>(g, area / 2);
-    g->lh_svl = dalloc_n<float>(g, area / 2);
-    LF_CUDA(cudaStreamSynchronize(g->stream));
+    g->lh_plan_q = q;
+    g->lh_plan_K = g->K;
+    g->lh_plan_sched = g->sched_version;
 }
 
 LitHubPlan lit_hub_plan(lf_graph *g) {
     LitHubPlan hp;
     hp.pos = g->lh_pos;
-    hp.toff = g->lh_toff;
-    hp.tcap = g->lh_tcap;
-    hp.soff = g->lh_soff;
+    hp.eoff = g->lh_eoff;
+    hp.fbase = g->lh_fbase;
     hp.fh = g->lh_fh;
     hp.fc = g->lh_fc;
-    hp.sh = g->lh_sh;
-    hp.sr = g->lh_sr;
-    hp.nsr = g->lh_nsr;
-    hp.heff = g->lh_heff;
+    hp.ph = g->lh_ph;
+    hp.pp = g->lh_pp;
+    hp.total = g->lh_total;
     hp.lb = g->lh_lb;
     hp.ns = g->lh_ns;
-    hp.sv_c = g->lh_svc;
-    hp.sv_v = g->lh_svv;
-    hp.sv_l = g->lh_svl;
-    const int64_t cap = g->lh_tab_cap;
-    hp.dv = static_cast<float *>(g->lh_tab);
-    hp.keys = reinterpret_cast<int32_t *>(hp.dv + cap);
-    hp.vals = reinterpret_cast<uint32_t *>(hp.keys + cap);
-    hp.hs = reinterpret_cast<float *>(hp.vals + cap);
+    hp.seg = g->lh_seg;
+    hp.ec = g->lh_ent;
+    hp.ek = hp.ec + g->lh_area;
+    hp.ed = hp.ek + g->lh_area;
+    hp.sv_c = g->lh_cand;
+    hp.sv_v = reinterpret_cast<uint32_t *>(hp.sv_c + g->lh_area);
+    hp.sv_u = reinterpret_cast<float *>(hp.sv_v + g->lh_area);
     return hp;
 }
 
@@ -5146,14 +5325,13 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         const int64_t nf = g->lh_fq.empty() ? 0 : g->lh_fq[(size_t)b + 1] - f0;
         if (nf > 0) {
             const LitHubPlan hp = lit_hub_plan(g);
-            const int64_t s0 = g->lh_sq[(size_t)b], nsl = g->lh_sq[(size_t)b + 1] - s0;
+            const int64_t p0 = g->lh_pq[(size_t)b], np = g->lh_pq[(size_t)b + 1] - p0;
             const int64_t h0 = g->lh_hq[(size_t)b], nh = g->lh_hq[(size_t)b + 1] - h0;
-            k_lh_size<<<(unsigned)nh, 256, 0, g->stream>>>(ab, hp, bstart, h0, nh);
-            k_lh_fill<<<(unsigned)nf, 256, 0, g->stream>>>(ab, hp, bstart, f0);
-            k_lh_bound<<<(unsigned)nsl, 256, 0, g->stream>>>(ab, hp, bstart, s0);
-            k_lh_mark<<<(unsigned)nsl, 256, 0, g->stream>>>(ab, hp, bstart, s0);
+            k_lh_count<<<(unsigned)nf, 256, 0, g->stream>>>(ab, hp, bstart, f0);
+            k_lh_scatter<<<(unsigned)nf, 256, 0, g->stream>>>(ab, hp, bstart, f0);
+            k_lh_part<<<(unsigned)np, 256, LH_SMEM, g->stream>>>(ab, hp, bstart, p0);
             k_lh_decide<<<(unsigned)nh, 256, 0, g->stream>>>(ab, hp, bstart, h0, nh);
-            g->launches += 5;
+            g->launches += 4;
         }
         if (prof) record_event(g, g->prof_ev[2 * b + 1], capturing);
         const int64_t longest = g->max_deg / AP_CHUNK + 1;   // pieces of one node at most
@@ -5211,48 +5389,6 @@ void ensure_lit(lf_graph *g, int64_t q, int64_t nb) {
         drop_graph(g);
     }
     build_lit_hub_plan(g, q, nb);
-    // global tables: per queue, every node whose entries can exceed half a
-    // block's table gets pow2 >= 2 (d+1) K slots (K bounds every row, so
-    // (d+1) K bounds its entries); queues run one after the other and share
-    // the area, sized for the largest queue
-    if (g->lg_plan_q != q || g->lg_plan_K != g->K || g->lg_plan_sched != g->sched_version) {
-        g->lg_plan_q = q;
-        g->lg_plan_K = g->K;
-        g->lg_plan_sched = g->sched_version;
-        unsigned long long cap = 0;
-        if (g->n > 0 && (long long)(g->max_deg + 1) * g->K * 2 > LB_SLOTS) {
-            const int64_t len = g->sched.empty() ? g->n : g->sched.back();
-            std::vector<int32_t> order((size_t)std::max<int64_t>(len, 1)), deg((size_t)g->n);
-            if (len > 0)
-                LF_CUDA(cudaMemcpyAsync(order.data(), g->sched.empty() ? g->order : g->qorder, (size_t)len * 4,
-                                        cudaMemcpyDeviceToHost, g->stream));
-            LF_CUDA(cudaMemcpyAsync(deg.data(), g->deg, (size_t)g->n * 4, cudaMemcpyDeviceToHost, g->stream));
-            LF_CUDA(cudaStreamSynchronize(g->stream));
-            for (int64_t b = 0; b < nb; ++b) {
-                int64_t qs;
-                int32_t ql;
-                queue_bounds(g, q, b, qs, ql);
-                unsigned long long used = 0;
-                for (int64_t p2 = qs; p2 < qs + ql; ++p2) {
-                    const unsigned long long e = (unsigned long long)(deg[(size_t)order[(size_t)p2]] + 1) * g->K;
-                    if (2 * e <= (unsigned long long)LB_SLOTS) continue;
-                    unsigned long long H = 32;
-                    while (H < 2 * e) H <<= 1;
-                    used += H;
-                }
-                cap = std::max(cap, used);
-            }
-        }
-        // the area is a reservation for the worst case; past 32 MiB + 64 bytes
-        // per edge a node that finds no room takes the multi-pass shared path
-        cap = std::min<unsigned long long>(cap, ((32ull << 20) + 64ull * (unsigned long long)g->m) / 16);
-        if (cap != g->lg_cap) {
-            if (g->lg_area) dfree(g, g->lg_area);
-            g->lg_area = cap ? dalloc(g, (size_t)cap * 16) : nullptr;
-            g->lg_cap = cap;
-            drop_graph(g);
-        }
-    }
 }
 
 // Start of an iteration under the paper's gain: the member index (members
@@ -5748,8 +5884,6 @@ void free_run_state(lf_graph *g) {
     if (g->lg_area) dfree(g, g->lg_area);
     g->lg_area = nullptr;
     g->lg_cap = 0;
-    g->lg_plan_q = g->lg_plan_sched = -1;
-    g->lg_plan_K = 0;
     for (uint32_t **pp : {&g->lit_misc, &g->tstamp, &g->lit_ctr, &g->cm_cnt})
         if (*pp) {
             dfree(g, *pp);
