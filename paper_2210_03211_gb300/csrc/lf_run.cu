@@ -2421,7 +2421,7 @@ __device__ __forceinline__ bool lit_fill(const RunArgs &a, const LitNode &ln, in
     {   // each warp of the team takes a contiguous share of the neighbours
         const int64_t deg = ln.end - ln.beg, per = (deg + T - 1) / T;
         const int64_t qb = ln.beg + min(deg, (int64_t)w_in * per), qe = ln.beg + min(deg, (int64_t)(w_in + 1) * per);
-        lit_warp_entries<T == EV_WARPS ? 2 : 4, true>(a, qb, qe, pb, count_bytes, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
+        lit_warp_entries<2, true>(a, qb, qe, pb, count_bytes, [&](int32_t C, uint32_t ky, uint32_t dy, uint32_t n) {
             if (P > 1 && (int)part_of(C, P) != p) return;
             const int slot = lit_insert(keys, vals, hm, C);
             if (slot < 0) {
@@ -3043,8 +3043,10 @@ __device__ void lit_big_node(const RunArgs &a, int64_t bstart, int i, long long 
 // 3.07M nodes, q 65,536: 379 + 375 -> 453 + 80 + 92 us.
 constexpr int LIT_MID = 2;   // warps of the teams between one warp and a block
 
+// (Three blocks per SM for long queues, 80 registers: latency-bound, so a third more
+// warps beat the few spills -- 767k nodes 217 -> 205 ms, 3.07M nodes 248 -> 235 ms.)
 template <int T, bool INBLOCK>
-__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t bstart, int32_t blen, LitOver ov) {
+__global__ void __launch_bounds__(EV_THREADS, (INBLOCK ? 2 : 3)) k_lit_eval(RunArgs a, int64_t bstart, int32_t blen, LitOver ov) {
     extern __shared__ double lit_dyn[];
     __shared__ LitScratch ls;
     const LitTables t = lit_tables(lit_dyn);
@@ -3083,7 +3085,7 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_eval(RunArgs a, int64_t b
 }
 
 // Listed nodes by teams of LIT_MID warps, taken from a counter.
-__global__ void __launch_bounds__(EV_THREADS, 2) k_lit_mid(RunArgs a, int64_t bstart, LitOver ov) {
+__global__ void __launch_bounds__(EV_THREADS, 3) k_lit_mid(RunArgs a, int64_t bstart, LitOver ov) {
     extern __shared__ double lit_dyn[];
     __shared__ LitScratch ls;
     __shared__ uint32_t s_at[EV_WARPS / LIT_MID];
@@ -3157,11 +3159,16 @@ __global__ void __launch_bounds__(EV_THREADS, 3) k_lit_big(RunArgs a, int64_t bs
 //                 survivors' exact sums; those of large communities by the whole
 //                 block, with the hub's adjacency searched through a fence in
 //                 shared memory.
-// Team and block kernels skip these nodes.
+// Team and block kernels skip these nodes.  A block's table holds 3,072 entries, so
+// the line follows the row capacity: with rows of four a node of 1,024 neighbours
+// mostly fits, with longer ones it went to a table in global memory (whole runs,
+// line at 1,024 / 512: 767k nodes, ten iterations, rows of up to 16: 205 / 197 ms;
+// 3.07M nodes, three iterations, rows of four: 235 / 239 ms).
 // Mean over the queues that have hubs, all kernels but the decision: 767k nodes, q 16,384:
 // 1,060 -> 475 us; 3.07M nodes, q 65,536: 1,900 -> 1,130 us (cold caches).
 // ---------------------------------------------------------------------------
-constexpr int LIT_HUB_DEG = 1024;
+constexpr int LIT_HUB_DEG = 1024;    // while rows hold at most four communities
+constexpr int LIT_HUB_DEG_LONG = 512;   // with longer rows
 constexpr int LH_CHUNK = 1024;       // neighbours per counting / scattering block
 constexpr int LH_PART = 1536;        // entries per part (more beyond LH_PARTS parts)
 constexpr int LH_PARTS = 128;
@@ -3929,6 +3936,8 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
 __global__ void __launch_bounds__(EV_THREADS) k_lit_fsum(RunArgs a, const int32_t *list, const uint32_t *count,
                                                          int64_t ncount) {
     __shared__ FsumShared fs;
+    pdl_trigger();
+    pdl_wait();
     const int64_t total = list ? (int64_t)__ldcg(count) : ncount;
     // a list's first entries go to a block each (short lists spread over the SMs'
     // FP64 pipes); all communities: neighbours' records to one block
@@ -4850,7 +4859,7 @@ RunArgs make_args(lf_graph *g, Readback *rbd) {
     a.lg_keys = reinterpret_cast<int32_t *>(a.lg_dv + g->lg_cap);
     a.lg_vals = reinterpret_cast<uint32_t *>(a.lg_keys + g->lg_cap);
     a.lg_aux = reinterpret_cast<int32_t *>(a.lg_vals + g->lg_cap);
-    a.lit_hub_deg = g->lh_n > 0 ? LIT_HUB_DEG : 0x7fffffff;
+    a.lit_hub_deg = g->lh_n > 0 ? (g->lh_plan_K <= 4 ? LIT_HUB_DEG : LIT_HUB_DEG_LONG) : 0x7fffffff;
     if (lit) a.screen = g->screen ? 1 : 0;   // brackets need no FP32 range condition
     return a;
 }
@@ -5082,6 +5091,8 @@ void launch_batches(lf_graph *g, const RunArgs &a, int64_t q, int64_t first, int
     LF_LAUNCHED();
 }
 
+int32_t lit_hub_degree(const lf_graph *g) { return g->K <= 4 ? LIT_HUB_DEG : LIT_HUB_DEG_LONG; }
+
 void free_lit_hub_plan(lf_graph *g) {
     auto drop = [&](auto *&p) {
         if (p) dfree(g, p);
@@ -5106,16 +5117,16 @@ void free_lit_hub_plan(lf_graph *g) {
 // 23.2 / 22.4; 84k nodes q 64 25.0 / 21.9, q 256 36.4 / 27.6.
 constexpr int64_t LIT_LOOP_MAX_Q = 1;
 
-// The nodes of degree > LIT_HUB_DEG by position in the order the queues take,
+// The nodes of degree > hub_deg by position in the order the queues take,
 // and per queue the slots of global tables its other nodes could want at most
 // (K bounds every row, so (d+1) K bounds a node's entries).  qstart: queue
 // boundaries of a batch (nb + 1), null for queues of q.  One pass on the device:
 // copied to the host node by node, these plans took 36 ms of a run on 3.07M nodes.
 __global__ void k_lit_plan(const int32_t *order, const int32_t *deg, int64_t len, const int64_t *qstart, int64_t nb,
-                           int64_t q, int32_t K, uint32_t *nhub, int2 *hubs, unsigned long long *want) {
+                           int64_t q, int32_t K, int32_t hub_deg, uint32_t *nhub, int2 *hubs, unsigned long long *want) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < len; p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = deg[order[p]];
-        if (d > LIT_HUB_DEG) {
+        if (d > hub_deg) {
             hubs[atomicAdd(nhub, 1u)] = make_int2((int32_t)p, d);
             continue;
         }
@@ -5151,9 +5162,8 @@ void build_lit_hub_plan(lf_graph *g, int64_t q, int64_t nb) {
     const int64_t len = g->sched.empty() ? g->n : g->sched.back();
     std::vector<int2> hubs;
     unsigned long long cap = 0;
-    if (len > 0 && (g->max_deg > LIT_HUB_DEG || 4 * (int64_t)(g->max_deg + 1) * g->K > 3 * LB_SLOTS)) {
-        // hubs number at most 2m / LIT_HUB_DEG
-        const int64_t most = std::min<int64_t>(len, 2 * g->m / LIT_HUB_DEG + 1);
+    if (len > 0 && (g->max_deg > lit_hub_degree(g) || 4 * (int64_t)(g->max_deg + 1) * g->K > 3 * LB_SLOTS)) {
+        const int64_t most = std::min<int64_t>(len, 2 * g->m / lit_hub_degree(g) + 1);   // hubs
         const int64_t words = nb + 1 + (g->sched.empty() ? 0 : nb + 1) + most;
         unsigned long long *buf = dalloc_n<unsigned long long>(g, words);
         unsigned long long *want = buf;
@@ -5164,7 +5174,7 @@ void build_lit_hub_plan(lf_graph *g, int64_t q, int64_t nb) {
         if (qs)
             LF_CUDA(cudaMemcpyAsync(qs, g->sched.data(), (size_t)(nb + 1) * 8, cudaMemcpyHostToDevice, g->stream));
         k_lit_plan<<<grid_for(len, 256, 1 << 12), 256, 0, g->stream>>>(g->sched.empty() ? g->order : g->qorder, g->deg,
-                                                                     len, qs, nb, q, g->K, nhub, dh, want);
+                                                                     len, qs, nb, q, g->K, lit_hub_degree(g), nhub, dh, want);
         ++g->launches;
         LF_LAUNCHED();
         std::vector<unsigned long long> host((size_t)nb + 1);
@@ -5337,8 +5347,8 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         const int64_t longest = g->max_deg / AP_CHUNK + 1;   // pieces of one node at most
         const unsigned ag = grid_for((int64_t)blen * longest * 32, AP_THREADS, 6 * (int64_t)num_sms());
         launch_pdl(k_lit_apply, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
-        k_lit_fsum<<<(unsigned)std::min<int64_t>(2 * (int64_t)blen, 4 * (int64_t)num_sms()), EV_THREADS, 0,
-                     g->stream>>>(ab, g->touched, ctr + 2, 0);
+        launch_pdl(k_lit_fsum, (unsigned)std::min<int64_t>(2 * (int64_t)blen, 4 * (int64_t)num_sms()), EV_THREADS, 0,
+                   g->stream, ab, (const int32_t *)g->touched, (const uint32_t *)(ctr + 2), (int64_t)0);
         g->launches += 3;
     }
     LF_LAUNCHED();
