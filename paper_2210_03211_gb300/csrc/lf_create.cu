@@ -80,31 +80,55 @@ __device__ __forceinline__ uint32_t id_rank(const uint32_t *bm, const uint32_t *
 // Both directions of every non-loop pair as (row << 32 | col); the slot of a
 // warp's keys comes from one atomic, so the output order is arbitrary -- the
 // radix sort that follows fixes it.
-__global__ void k_make_keys(const int32_t *src, const int32_t *dst, int64_t E, const uint32_t *bm,
-                            const uint32_t *wb, unsigned long long *keys, unsigned long long *cursor) {
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); e0 < E; e0 += stride) {
-        int64_t e = e0 + lane;
-        bool ok = false;
-        uint32_t ra = 0, rb = 0;
-        if (e < E) {
-            uint32_t a = (uint32_t)src[e], b = (uint32_t)dst[e];
-            if (a != b) {
-                ok = true;
-                ra = id_rank(bm, wb, a);
-                rb = id_rank(bm, wb, b);
+// (Blocks take tiles of eight edges a thread and one place for all of a tile's keys:
+// an atomic per 32 edges on the one cursor was the kernel's time, 120M edges
+// 4.3 -> 1.8 ms.)
+constexpr int MK_ITEMS = 8;
+
+__global__ void __launch_bounds__(256) k_make_keys(const int32_t *src, const int32_t *dst, int64_t E, const uint32_t *bm,
+                                                   const uint32_t *wb, unsigned long long *keys,
+                                                   unsigned long long *cursor) {
+    __shared__ uint32_t s_w[8];
+    __shared__ unsigned long long s_base;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int TILE = 256 * MK_ITEMS;
+    for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < E; t0 += (int64_t)gridDim.x * TILE) {
+        uint32_t a[MK_ITEMS], b[MK_ITEMS];
+        uint32_t before[MK_ITEMS], mine = 0;   // non-loops of this warp before the item, all of them
+#pragma unroll
+        for (int c = 0; c < MK_ITEMS; ++c) {
+            const int64_t e = t0 + c * 256 + threadIdx.x;
+            a[c] = e < E ? (uint32_t)src[e] : 0u;
+            b[c] = e < E ? (uint32_t)dst[e] : 0u;
+        }
+#pragma unroll
+        for (int c = 0; c < MK_ITEMS; ++c) {
+            const unsigned mask = __ballot_sync(FULL, a[c] != b[c]);   // past the end both are 0
+            before[c] = mine + __popc(mask & lanemask_lt());
+            mine += __popc(mask);
+        }
+        if (lane == 0) s_w[w] = mine;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t run = 0;
+            for (int k = 0; k < 8; ++k) {
+                const uint32_t t = s_w[k];
+                s_w[k] = run;
+                run += t;
             }
+            s_base = run ? atomicAdd(cursor, 2ull * run) : 0ull;
         }
-        unsigned mask = __ballot_sync(FULL, ok);
-        unsigned long long base = 0;
-        if (lane == 0 && mask) base = atomicAdd(cursor, 2ull * __popc(mask));
-        base = __shfl_sync(FULL, base, 0);
-        if (ok) {
-            unsigned long long p = base + 2ull * __popc(mask & lanemask_lt());
-            keys[p] = ((unsigned long long)ra << 32) | rb;
-            keys[p + 1] = ((unsigned long long)rb << 32) | ra;
-        }
+        __syncthreads();
+        const unsigned long long base = s_base + 2ull * s_w[w];
+#pragma unroll
+        for (int c = 0; c < MK_ITEMS; ++c)
+            if (a[c] != b[c]) {
+                const unsigned long long ra = id_rank(bm, wb, a[c]), rb = id_rank(bm, wb, b[c]);
+                const unsigned long long p = base + 2ull * before[c];
+                keys[p] = (ra << 32) | rb;
+                keys[p + 1] = (rb << 32) | ra;
+            }
+        __syncthreads();
     }
 }
 
@@ -1541,7 +1565,7 @@ void build_graph(lf_graph *g, const int32_t *src, const int32_t *dst, int64_t E,
         int64_t nkeys = 2 * (int64_t)nonloops;
         unsigned long long *keys = dalloc_n<unsigned long long>(g, nkeys);
         LF_CUDA(cudaMemsetAsync(tmp64, 0, sizeof(unsigned long long), st));
-        k_make_keys<<<grid_for(E, 256, 4096), 256, 0, st>>>(dsrc, ddst, E, bm, wb, keys, tmp64); ++g->launches;
+        k_make_keys<<<grid_for(E, 256 * MK_ITEMS, 1 << 14), 256, 0, st>>>(dsrc, ddst, E, bm, wb, keys, tmp64); ++g->launches;
         LF_LAUNCHED();
         dfree(g, wb);
         dfree(g, bm);
