@@ -105,6 +105,7 @@ struct RunArgs {
     int2 *items;
     uint32_t *nitems;
     int32_t *apacc;
+    int32_t list_above;   // only movers of higher degree are listed
     // tables in global memory for nodes with more entries than a block's
     // shared table holds (bump-allocated per queue, lg_cap slots)
     int32_t *lg_keys;
@@ -1654,9 +1655,9 @@ __global__ void __launch_bounds__(EV_THREADS, 3) k_eval(RunArgs a, int64_t bstar
 // of the same queue targets C.  Integer atomics: order-independent.
 // ---------------------------------------------------------------------------
 // Static data of a node to apply (never changes in a run): node, neighbours, the
-// lane's first neighbour's position in the order.
+// lane's first neighbour and its position in the order.
 struct ApplyPrefetch {
-    int32_t x;
+    int32_t x, y0;
     int64_t beg, end, py0;
 };
 
@@ -1666,7 +1667,8 @@ __device__ __forceinline__ ApplyPrefetch apply_prefetch(const RunArgs &a, int64_
     ap.beg = a.off[ap.x];
     ap.end = a.off[ap.x + 1];
     const int64_t p = ap.beg + (threadIdx.x & 31);
-    ap.py0 = p < ap.end ? (int64_t)a.pos[a.adj[p]] : -1;
+    ap.y0 = p < ap.end ? a.adj[p] : 0;
+    ap.py0 = p < ap.end ? (int64_t)a.pos[ap.y0] : -1;
     return ap;
 }
 
@@ -3599,7 +3601,9 @@ __global__ void __launch_bounds__(256) k_lh_decide(RunArgs a, LitHubPlan hp, int
 // AP_CHUNK neighbours per item: idle nodes cost nothing, and a hub's
 // neighbours are spread over many warps (one warp walking 30,000 neighbours
 // alone held its queue for 2 ms); the warp that finishes a node's last piece
-// rewrites its row.
+// rewrites its row.  A short queue's time is its chain of dependent loads, so there
+// every position has a warp, which reads its node's static data before the wait
+// for the evaluation, and only nodes of several pieces are listed (335k nodes, q 1,024: 33.2 -> 30.5 us a queue).
 // Mean over the queues, both steps together: 767k nodes, q 16,384: 142 -> 57 us;
 // 84k nodes, q 64: 15.3 -> 10.8 us and one launch less (cold caches).
 // ---------------------------------------------------------------------------
@@ -3608,16 +3612,19 @@ constexpr int AP_CHUNK = 512;
 // The decision of queue position i, and its pieces of work if it moves.  One thread.
 __device__ __forceinline__ void lit_write_action(const RunArgs &a, int i, int32_t d, const Best &bj, const Best &bl) {
     write_action(a, i, bj, bl, 0ull);
-    if ((bj.c < 0 && bl.c < 0) || !a.items) return;   // the persistent loop's blocks apply their own nodes
+    if ((bj.c < 0 && bl.c < 0) || d <= a.list_above) return;
     const uint32_t pieces = d > AP_CHUNK ? (uint32_t)(d + AP_CHUNK - 1) / AP_CHUNK : 1u;
     const uint32_t at = atomicAdd(a.nitems, pieces);
     for (uint32_t c = 0; c < pieces; ++c) a.items[at + c] = make_int2(i, (int)c);
 }
 
-// One piece of queue position i (node x, neighbours adj[xb, xe)), by one warp.
-__device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, int i, int piece, int32_t x, int64_t xb,
-                                int64_t xe, uint32_t serial, unsigned long long &nj, unsigned long long &nl) {
+// One piece of queue position i, by one warp.
+// (ap: its static data.)
+__device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, int i, int piece, const ApplyPrefetch &ap,
+                                uint32_t serial, unsigned long long &nj, unsigned long long &nl) {
     const int lane = threadIdx.x & 31;
+    const int32_t x = ap.x;
+    const int64_t xb = ap.beg, xe = ap.end;
     const int32_t j = __ldcg(&a.act[i]), l = __ldcg(&a.act[a.qcap + i]);
     const int32_t kjoin = __ldcg(&a.act[2 * a.qcap + i]), kl = __ldcg(&a.act[3 * a.qcap + i]);
     int32_t *row = a.mem + (int64_t)x * a.K;
@@ -3631,10 +3638,11 @@ __device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, 
     int jj = 0, jl = 0, ll = 0;
     const int64_t pe = min(xe, xb + (int64_t)(piece + 1) * AP_CHUNK);
     for (int64_t p = xb + (int64_t)piece * AP_CHUNK + lane; p < pe; p += 32) {
-        const int32_t y = a.adj[p];
+        const bool first = p < xb + 32;
+        const int32_t y = first ? ap.y0 : a.adj[p];
         const RowHead ids = row_head8(a.mem, y, a.K);
         const int32_t cy = __ldcg(&a.nmem[y]);
-        const int64_t iy = (int64_t)a.pos[y] - bstart;
+        const int64_t iy = (first ? ap.py0 : (int64_t)a.pos[y]) - bstart;
         int32_t aj = -1, al = -1;
         if (iy >= 0 && iy < blen) {
             aj = __ldcg(&a.act[iy]);
@@ -3783,17 +3791,23 @@ __device__ void lit_apply_piece(const RunArgs &a, int64_t bstart, int32_t blen, 
     if (lane == 0) a.nmem[x] = c_new;
 }
 
-// A resident grid at most; warps stride over the queue's items.
+// Warps stride over the queue's items (a resident grid at most); DIRECT: a warp
+// per position of the queue first.
+template <bool DIRECT>
 __global__ void __launch_bounds__(AP_THREADS) k_lit_apply(RunArgs a, int64_t bstart, int32_t blen, int64_t bidx) {
+    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = (gridDim.x * blockDim.x) >> 5;
+    const bool mine = DIRECT && gw < (uint32_t)blen;
+    ApplyPrefetch ap{};
+    if (mine) ap = apply_prefetch(a, bstart, gw);
     pdl_trigger();
     pdl_wait();
     const uint32_t serial = (uint32_t)queue_serial(a, bidx);
     const uint32_t count = __ldcg(a.nitems);
     unsigned long long nj = 0, nl = 0;
-    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < count; t += (gridDim.x * blockDim.x) >> 5) {
+    if (mine && ap.end - ap.beg <= a.list_above) lit_apply_piece(a, bstart, blen, (int)gw, 0, ap, serial, nj, nl);
+    for (uint32_t t = gw; t < count; t += warps) {
         const int2 item = __ldcg(&a.items[t]);
-        const int32_t x = a.order[bstart + item.x];
-        lit_apply_piece(a, bstart, blen, item.x, item.y, x, a.off[x], a.off[x + 1], serial, nj, nl);
+        lit_apply_piece(a, bstart, blen, item.x, item.y, apply_prefetch(a, bstart, item.x), serial, nj, nl);
     }
     flush_counts(a, nj, nl);
 }
@@ -4409,8 +4423,10 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, const 
             if (base != base0) prefetch_node(a, bstart, blen, i, w_in, cur);
             else cur = pf;
             if (i >= blen || w_in != 0) continue;
+            ApplyPrefetch ap{cur.x, cur.y0, cur.beg, cur.end, -1};
+            if (cur.beg + lane < cur.end) ap.py0 = a.pos[cur.y0];
             for (int piece = 0; piece == 0 || piece * AP_CHUNK < cur.d; ++piece)
-                lit_apply_piece(a, bstart, blen, i, piece, cur.x, cur.beg, cur.end, serial, nj, nl);
+                lit_apply_piece(a, bstart, blen, i, piece, ap, serial, nj, nl);
         }
         // the next queue's static data load while the barrier completes
         const bool more = b + 1 < first + count;
@@ -4877,6 +4893,7 @@ RunArgs make_args(lf_graph *g, Readback *rbd) {
     a.items = reinterpret_cast<int2 *>(g->lit_items);
     a.nitems = g->lit_ctr;
     a.apacc = g->lit_apacc;
+    a.list_above = -1;
     a.lg_cap = g->lg_cap;
     a.lg_dv = static_cast<float *>(g->lg_area);
     a.lg_keys = reinterpret_cast<int32_t *>(a.lg_dv + g->lg_cap);
@@ -5339,7 +5356,8 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         const unsigned grid = (unsigned)((blen + teams - 1) / teams);
         const LitOver ov{reinterpret_cast<int2 *>(g->lit_over), reinterpret_cast<int2 *>(g->lit_over) + g->lit_qcap, ctr,
                          g->lit_used + b};
-        const bool inblock = grid <= 2 * (unsigned)num_sms();
+        const bool inblock = grid <= 2 * (unsigned)num_sms();   // a short queue: one wave of blocks
+        ab.list_above = inblock ? AP_CHUNK : -1;
         switch (T) {
         case 1: launch_pdl(inblock ? k_lit_eval<1, true> : k_lit_eval<1, false>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ov); break;
         case 2: launch_pdl(inblock ? k_lit_eval<2, true> : k_lit_eval<2, false>, grid, EV_THREADS, LIT_SMEM, g->stream, ab, bstart, blen, ov); break;
@@ -5369,7 +5387,10 @@ void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first,
         if (prof) record_event(g, g->prof_ev[2 * b + 1], capturing);
         const int64_t longest = g->max_deg / AP_CHUNK + 1;   // pieces of one node at most
         const unsigned ag = grid_for((int64_t)blen * longest * 32, AP_THREADS, 6 * (int64_t)num_sms());
-        launch_pdl(k_lit_apply, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
+        if (inblock)
+            launch_pdl(k_lit_apply<true>, grid_for((int64_t)blen * 32, AP_THREADS), AP_THREADS, 0, g->stream, ab, bstart, blen, b);
+        else
+            launch_pdl(k_lit_apply<false>, ag, AP_THREADS, 0, g->stream, ab, bstart, blen, b);
         launch_pdl(k_lit_fsum, (unsigned)std::min<int64_t>(2 * (int64_t)blen, 4 * (int64_t)num_sms()), EV_THREADS, 0,
                    g->stream, ab, (const int32_t *)g->touched, (const uint32_t *)(ctr + 2), (int64_t)0);
         g->launches += 3;
@@ -5653,7 +5674,7 @@ void launch_lit_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int
     uint32_t *ctr = g->lit_ctr;
     unsigned long long *used = g->lit_used;
     const int64_t *qstart = nullptr;
-    a.items = nullptr;
+    a.list_above = 0x7fffffff;   // the blocks apply the nodes they evaluated
     LF_CUDA(cudaMemsetAsync(ctr + 8 * first, 0, (size_t)(8 * count) * sizeof(uint32_t), g->stream));
     LF_CUDA(cudaMemsetAsync(used + first, 0, (size_t)count * sizeof(unsigned long long), g->stream));
     void *args[] = {&a, &qstart, &q, &first, &count, &ctr, &used, &spin, &inject, &flags, &epoch, &bar_mode};
