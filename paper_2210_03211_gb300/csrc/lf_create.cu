@@ -1436,17 +1436,19 @@ __global__ void k_cc_sum(const unsigned long long *tri, const int32_t *deg, int6
     __shared__ unsigned long long acc[SACC_CHUNKS];
     for (int i = threadIdx.x; i < SACC_CHUNKS; i += blockDim.x) acc[i] = 0ull;
     __syncthreads();
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-        sacc_add(acc, local_cc((long long)tri[x], deg[x]));
+    for (int64_t x0 = (int64_t)blockIdx.x * blockDim.x; x0 < n; x0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t x = x0 + threadIdx.x;
+        sacc_add_warp(acc, x < n ? local_cc((long long)tri[x], deg[x]) : 0.0);
+    }
     __syncthreads();
     for (int i = threadIdx.x; i < SACC_CHUNKS; i += blockDim.x)
         if (acc[i]) atomicAdd(&ds->sacc[i], acc[i]);
 }
 
 __global__ void k_cc_final(DevScalars *ds, int64_t n) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = sacc_round_and_clear(ds->sacc);
-    ds->cc = n > 0 ? __ddiv_rn(s, (double)n) : 0.0;
+    __shared__ unsigned long long acc[SACC_CHUNKS];
+    const double s = sacc_take_warp(ds->sacc, acc);   // one warp
+    if (threadIdx.x == 0) ds->cc = n > 0 ? __ddiv_rn(s, (double)n) : 0.0;
 }
 
 // ---- batches of graphs -----------------------------------------------------
@@ -1470,18 +1472,29 @@ __global__ void k_gid_keys(const uint32_t *vals, const int32_t *gid, int64_t n, 
 // cc of every graph of a batch: RN(exact sum of RN(CC_i) over its nodes) / n_i.
 __global__ void k_cc_sum_batch(const unsigned long long *tri, const int32_t *deg, const int32_t *gid, int64_t n,
                                unsigned long long *gsacc) {
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-        sacc_add(gsacc + (int64_t)gid[x] * SACC_CHUNKS, local_cc((long long)tri[x], deg[x]));
+    for (int64_t x0 = (int64_t)blockIdx.x * blockDim.x; x0 < n; x0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t x = x0 + threadIdx.x;
+        const double v = x < n ? local_cc((long long)tri[x], deg[x]) : 0.0;
+        const int32_t g = x < n ? gid[x] : -1, g0 = __shfl_sync(FULL, g, 0);
+        if (__all_sync(FULL, g == g0 || g < 0)) {   // nearly always: a graph's nodes are consecutive
+            if (g0 >= 0) sacc_add_warp(gsacc + (int64_t)g0 * SACC_CHUNKS, v);
+        } else if (g >= 0) {
+            sacc_add(gsacc + (int64_t)g * SACC_CHUNKS, v);
+        }
+    }
 }
 
-__global__ void k_cc_final_batch(unsigned long long *gsacc, const int64_t *gnoff, int64_t G, double *gcc,
-                                 float *gcc32) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < G; i += (int64_t)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(256) k_cc_final_batch(unsigned long long *gsacc, const int64_t *gnoff, int64_t G,
+                                                        double *gcc, float *gcc32) {
+    __shared__ unsigned long long acc[8][SACC_CHUNKS];
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < G; i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int64_t ni = gnoff[i + 1] - gnoff[i];
-        const double s = sacc_round_and_clear(gsacc + i * SACC_CHUNKS);
+        const double s = sacc_take_warp(gsacc + i * SACC_CHUNKS, acc[threadIdx.x >> 5]);
         const double c = ni > 0 ? __ddiv_rn(s, (double)ni) : 0.0;
-        gcc[i] = c;
-        gcc32[i] = c >= 1e-30 ? (float)c : 0.f;   // 0 turns the FP32 screen off for the graph
+        if ((threadIdx.x & 31) == 0) {
+            gcc[i] = c;
+            gcc32[i] = c >= 1e-30 ? (float)c : 0.f;   // 0 turns the FP32 screen off for the graph
+        }
     }
 }
 
@@ -1724,7 +1737,7 @@ void build_graph(lf_graph *g, const int32_t *src, const int32_t *dst, int64_t E,
         LF_LAUNCHED();
     }
     if (g->ngraphs > 0) {
-        k_cc_final_batch<<<grid_for(g->ngraphs, 256, 1024), 256, 0, st>>>(g->gsacc, gnoff_d, g->ngraphs, g->gcc,
+        k_cc_final_batch<<<grid_for(g->ngraphs * 32, 256, 1024), 256, 0, st>>>(g->gsacc, gnoff_d, g->ngraphs, g->gcc,
                                                                           g->gcc32); ++g->launches;
         LF_LAUNCHED();
         g->gcc_host.assign((size_t)g->ngraphs, 0.0);

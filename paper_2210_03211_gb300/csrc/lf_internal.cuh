@@ -377,46 +377,102 @@ __device__ __forceinline__ void sacc_add(unsigned long long *acc, double v) {
     if (hi) atomicAdd(&acc[c + 2], hi);
 }
 
-// Round the accumulated exact value to the nearest double (ties to even) and
-// clear the accumulator.  One thread.
-__device__ inline double sacc_round_and_clear(unsigned long long *acc) {
-    uint32_t dg[SACC_CHUNKS];
-    unsigned long long carry = 0;
-    for (int i = 0; i < SACC_CHUNKS; ++i) {
-        unsigned long long v = acc[i] + carry;
+// A warp's values v >= 0 (zero for lanes without one) into an accumulator shared
+// with other warps (shared or global memory): the digits are summed over the lanes
+// by integer reductions of their 16-bit halves, so a warp queues a few atomics on
+// the few words in question instead of two or three a lane.
+__device__ __forceinline__ void sacc_add_warp(unsigned long long *acc, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    const unsigned long long mant = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    const int p = e ? (int)e - 1 : 0;
+    const int c = p >> 5, sh = p & 31;
+    const unsigned long long lo = mant << sh;
+    const uint32_t d0 = (uint32_t)lo, d1 = (uint32_t)(lo >> 32), d2 = sh ? (uint32_t)(mant >> (64 - sh)) : 0u;
+    const int c0 = __reduce_min_sync(FULL, b ? c : SACC_CHUNKS);
+    const int c1 = __reduce_max_sync(FULL, b ? c : -1);
+    for (int t = c0; t <= c1 + 2 && t < SACC_CHUNKS; ++t) {
+        const uint32_t dg = b == 0ull ? 0u : t == c ? d0 : t == c + 1 ? d1 : t == c + 2 ? d2 : 0u;
+        const unsigned l16 = __reduce_add_sync(FULL, dg & 0xffffu), h16 = __reduce_add_sync(FULL, dg >> 16);
+        const unsigned long long sum = (unsigned long long)l16 + ((unsigned long long)h16 << 16);
+        if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&acc[t], sum);
+    }
+}
+
+// The accumulated signed value rounded to the nearest double (ties to even),
+// and the accumulator cleared: one warp, the result on every lane.  Only the
+// words between the lowest and the highest non-zero one are walked (the terms
+// of a gain reach over a handful), in place.
+static __device__ __noinline__ double ssacc_round_warp(unsigned long long *acc) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const unsigned m0 = __ballot_sync(FULL, acc[lane] != 0ull), m1 = __ballot_sync(FULL, acc[lane + 32] != 0ull);
+    const unsigned m2 = __ballot_sync(FULL, lane + 64 < SACC_CHUNKS && acc[min(lane + 64, SACC_CHUNKS - 1)] != 0ull);
+    if (!(m0 | m1 | m2)) return 0.0;
+    const int first = m0 ? __ffs(m0) - 1 : m1 ? 31 + __ffs(m1) : 63 + __ffs(m2);
+    const int last0 = m2 ? 95 - __clz(m2) : m1 ? 63 - __clz(m1) : 31 - __clz(m0);
+    double r = 0.0;
+    if (lane == 0) {
+        const int last = min(last0 + 1, SACC_CHUNKS - 1);   // the carry out of the top word
+        long long carry = 0;
+        for (int i = first; i <= last; ++i) {
+            const long long v = (long long)acc[i] + carry;
+            acc[i] = (unsigned long long)(uint32_t)v;
+            carry = v >> 32;   // rounds down: the digit just stored is v mod 2^32
+        }
+        const bool neg = carry < 0;   // the value is (digits) - 2^(32 (last + 1))
+        int top = -1;
+        uint32_t c = 1;
+        for (int i = first; i <= last; ++i) {
+            uint32_t d = (uint32_t)acc[i];
+            if (neg) {
+                const unsigned long long t = (unsigned long long)(uint32_t)~d + c;
+                d = (uint32_t)t;
+                c = (uint32_t)(t >> 32);
+                acc[i] = d;
+            }
+            if (d) top = i;
+        }
+        if (top >= 0) {
+            const uint32_t a2 = (uint32_t)acc[top], a1 = top >= 1 ? (uint32_t)acc[top - 1] : 0u,
+                           a0 = top >= 2 ? (uint32_t)acc[top - 2] : 0u;
+            const int z = __clz((int)a2), P = 32 * top + 31 - z;   // P: index of the leading bit
+            const unsigned long long h = ((unsigned long long)a2 << 32) | a1;
+            unsigned long long bits;
+            if (P <= 52) {   // fewer than 54 significant bits: exact
+                bits = top == 1 ? h : (unsigned long long)a2;
+            } else {
+                const unsigned long long w = z ? (h << z) | (a0 >> (32 - z)) : h;   // the leading 64 bits
+                bool sticky = (w & 0x3ffull) != 0ull || (z ? (a0 << z) != 0u : a0 != 0u);
+                for (int i = first; i < top - 2 && !sticky; ++i) sticky = acc[i] != 0ull;
+                unsigned long long mant = w >> 11;
+                long long biased = (long long)P - 51;
+                if (((w >> 10) & 1ull) && (sticky || (mant & 1ull))) ++mant;
+                if (mant == (1ull << 53)) {
+                    mant >>= 1;
+                    ++biased;
+                }
+                bits = biased >= 2047 ? 0x7ff0000000000000ull
+                                      : ((unsigned long long)biased << 52) | (mant & 0xfffffffffffffull);
+            }
+            r = __longlong_as_double((long long)bits);
+            if (neg) r = -r;
+        }
+        for (int i = first; i <= last; ++i) acc[i] = 0ull;
+    }
+    __syncwarp();
+    return __shfl_sync(FULL, r, 0);
+}
+
+// The value accumulated in global memory, rounded, and the accumulator cleared: one
+// warp, with SACC_CHUNKS words of shared memory of its own.  (One thread walking the
+// 68 words and a local copy of them took 6 us.)
+__device__ __forceinline__ double sacc_take_warp(unsigned long long *acc, unsigned long long *shared) {
+    for (int i = threadIdx.x & 31; i < SACC_CHUNKS; i += 32) {
+        shared[i] = acc[i];
         acc[i] = 0ull;
-        dg[i] = (uint32_t)(v & 0xffffffffull);
-        carry = v >> 32;
     }
-    int top = -1;
-    for (int i = SACC_CHUNKS - 1; i >= 0; --i)
-        if (dg[i]) { top = i; break; }
-    if (top < 0) return 0.0;
-    int P = 32 * top + (31 - __clz((int)dg[top]));   // index of the leading bit
-    auto bit = [&](int q) -> unsigned long long {
-        return q < 0 ? 0ull : (unsigned long long)((dg[q >> 5] >> (q & 31)) & 1u);
-    };
-    if (P <= 52) {   // fewer than 54 significant bits: exact (subnormal or smallest binade)
-        unsigned long long v = 0;
-        for (int q = P; q >= 0; --q) v = (v << 1) | bit(q);
-        return __longlong_as_double((long long)v);
-    }
-    unsigned long long mant = 0;
-    for (int q = P; q >= P - 52; --q) mant = (mant << 1) | bit(q);
-    int r = P - 53;                        // round bit position (>= 0)
-    bool round_bit = bit(r) != 0;
-    bool sticky = false;
-    for (int i = 0; i < (r >> 5) && !sticky; ++i) sticky = dg[i] != 0u;
-    if (!sticky && (r & 31)) sticky = (dg[r >> 5] & ((1u << (r & 31)) - 1u)) != 0u;
-    if (round_bit && (sticky || (mant & 1ull))) ++mant;
-    if (mant == (1ull << 53)) {
-        mant >>= 1;
-        ++P;
-    }
-    long long biased = (long long)P - 51;
-    if (biased >= 2047) return __longlong_as_double(0x7ff0000000000000ll);
-    unsigned long long bits = ((unsigned long long)biased << 52) | (mant & 0xfffffffffffffull);
-    return __longlong_as_double((long long)bits);
+    return ssacc_round_warp(shared);
 }
 
 __device__ __forceinline__ uint32_t hash32(uint32_t x) {

@@ -1905,71 +1905,6 @@ __device__ __forceinline__ void ssacc_add_warp(unsigned long long *acc, double v
     __syncwarp();
 }
 
-// The accumulated signed value rounded to the nearest double (ties to even),
-// and the accumulator cleared: one warp, the result on every lane.  Only the
-// words between the lowest and the highest non-zero one are walked (the terms
-// of a gain reach over a handful), in place.
-__device__ __noinline__ double ssacc_round_warp(unsigned long long *acc) {
-    const int lane = threadIdx.x & 31;
-    __syncwarp();
-    const unsigned m0 = __ballot_sync(FULL, acc[lane] != 0ull), m1 = __ballot_sync(FULL, acc[lane + 32] != 0ull);
-    const unsigned m2 = __ballot_sync(FULL, lane + 64 < SACC_CHUNKS && acc[min(lane + 64, SACC_CHUNKS - 1)] != 0ull);
-    if (!(m0 | m1 | m2)) return 0.0;
-    const int first = m0 ? __ffs(m0) - 1 : m1 ? 31 + __ffs(m1) : 63 + __ffs(m2);
-    const int last0 = m2 ? 95 - __clz(m2) : m1 ? 63 - __clz(m1) : 31 - __clz(m0);
-    double r = 0.0;
-    if (lane == 0) {
-        const int last = min(last0 + 1, SACC_CHUNKS - 1);   // the carry out of the top word
-        long long carry = 0;
-        for (int i = first; i <= last; ++i) {
-            const long long v = (long long)acc[i] + carry;
-            acc[i] = (unsigned long long)(uint32_t)v;
-            carry = v >> 32;   // rounds down: the digit just stored is v mod 2^32
-        }
-        const bool neg = carry < 0;   // the value is (digits) - 2^(32 (last + 1))
-        int top = -1;
-        uint32_t c = 1;
-        for (int i = first; i <= last; ++i) {
-            uint32_t d = (uint32_t)acc[i];
-            if (neg) {
-                const unsigned long long t = (unsigned long long)(uint32_t)~d + c;
-                d = (uint32_t)t;
-                c = (uint32_t)(t >> 32);
-                acc[i] = d;
-            }
-            if (d) top = i;
-        }
-        if (top >= 0) {
-            const uint32_t a2 = (uint32_t)acc[top], a1 = top >= 1 ? (uint32_t)acc[top - 1] : 0u,
-                           a0 = top >= 2 ? (uint32_t)acc[top - 2] : 0u;
-            const int z = __clz((int)a2), P = 32 * top + 31 - z;   // P: index of the leading bit
-            const unsigned long long h = ((unsigned long long)a2 << 32) | a1;
-            unsigned long long bits;
-            if (P <= 52) {   // fewer than 54 significant bits: exact
-                bits = top == 1 ? h : (unsigned long long)a2;
-            } else {
-                const unsigned long long w = z ? (h << z) | (a0 >> (32 - z)) : h;   // the leading 64 bits
-                bool sticky = (w & 0x3ffull) != 0ull || (z ? (a0 << z) != 0u : a0 != 0u);
-                for (int i = first; i < top - 2 && !sticky; ++i) sticky = acc[i] != 0ull;
-                unsigned long long mant = w >> 11;
-                long long biased = (long long)P - 51;
-                if (((w >> 10) & 1ull) && (sticky || (mant & 1ull))) ++mant;
-                if (mant == (1ull << 53)) {
-                    mant >>= 1;
-                    ++biased;
-                }
-                bits = biased >= 2047 ? 0x7ff0000000000000ull
-                                      : ((unsigned long long)biased << 52) | (mant & 0xfffffffffffffull);
-            }
-            r = __longlong_as_double((long long)bits);
-            if (neg) r = -r;
-        }
-        for (int i = first; i <= last; ++i) acc[i] = 0ull;
-    }
-    __syncwarp();
-    return __shfl_sync(FULL, r, 0);
-}
-
 // Bounds-checked mode (lf_options.debug_checks): a value read from device
 // state that is out of its range sets DERR_CHECK and the access is skipped
 // (never a trap; the call then fails with a message).
@@ -2233,16 +2168,21 @@ __device__ __forceinline__ MemberRange lit_member_range(const RunArgs &a, int32_
     return r;
 }
 
+// f gets two of them at a time (-1: none), so that their loads overlap.
 template <typename F>
-__device__ __forceinline__ void lit_members(const RunArgs &a, int32_t C, const MemberRange &r, int tid, int nthreads,
-                                            F &&f) {
+__device__ __forceinline__ void lit_members2(const RunArgs &a, int32_t C, const MemberRange &r, int tid, int nthreads,
+                                             F &&f) {
     const int64_t b0 = r.b0, cap = r.cap, used = r.used;
     const int64_t b1 = b0 + (used < cap ? used : cap);
-    for (int64_t p = b0 + tid; p < b1; p += nthreads) f(__ldcg(&a.cm_node[p]));
+    for (int64_t p = b0 + tid; p < b1; p += 2 * nthreads) {
+        const int32_t y0 = __ldcg(&a.cm_node[p]);
+        const int32_t y1 = p + nthreads < b1 ? __ldcg(&a.cm_node[p + nthreads]) : -1;
+        f(y0, y1);
+    }
     if (used > cap) {
         int idx = 0;
         for (int32_t e = __ldcg(&a.jl_head[C]); e >= 0; e = __ldcg(&a.jl_next[e]), ++idx)
-            if (idx % nthreads == tid) f(__ldcg(&a.jl_node[e]));
+            if (idx % nthreads == tid) f(__ldcg(&a.jl_node[e]), -1);
     }
 }
 
@@ -3844,12 +3784,27 @@ __device__ __forceinline__ void lit_g3(int32_t k, int32_t d, int32_t n, double &
     f2 = fma(q, lo * D, f2);
 }
 
-__device__ __forceinline__ void lit_fsum_member(const RunArgs &a, int32_t C, int32_t n, int32_t y, double &f0,
+struct FsumMember {   // what a member's terms need, on its way
+    RowHead ids, ks;
+    int32_t y, cy, dy;
+};
+
+__device__ __forceinline__ FsumMember lit_fsum_load(const RunArgs &a, int32_t y) {
+    FsumMember m;
+    m.y = y >= 0 && dbg_ok(a, y < a.nnodes) ? y : -1;
+    const int64_t at = m.y >= 0 ? m.y : 0;
+    m.ids = row_head8(a.mem, at, a.K);
+    m.ks = row_head8(a.kmem, at, a.K);
+    m.cy = __ldcg(&a.nmem[at]);
+    m.dy = a.deg[at];
+    return m;
+}
+
+__device__ __forceinline__ void lit_fsum_member(const RunArgs &a, int32_t C, int32_t n, const FsumMember &m, double &f0,
                                                 double &f1, double &f2) {
-    if (!dbg_ok(a, y >= 0 && y < a.nnodes)) return;
-    const RowHead ids = row_head8(a.mem, y, a.K), ks = row_head8(a.kmem, y, a.K);
-    const int32_t cy = __ldcg(&a.nmem[y]);
-    const int32_t dy = a.deg[y];
+    if (m.y < 0) return;
+    const RowHead &ids = m.ids, &ks = m.ks;
+    const int32_t y = m.y, cy = m.cy, dy = m.dy;
     if (!dbg_ok(a, cy >= 0 && cy <= a.K)) return;
     const int s = head_find(ids, a.mem + (int64_t)y * a.K, cy, C);
     if (s < 0) return;   // left C earlier in this iteration
@@ -3860,17 +3815,21 @@ __device__ __forceinline__ void lit_fsum_member(const RunArgs &a, int32_t C, int
 
 // The per-community values of the bracket from the member sums (rounded
 // to float; the bound E allows for it).  Lane t of the first three of a group
-// (all of which hold the sums) forms the t-th factor.
-__device__ __forceinline__ void lit_fsum_store(const RunArgs &a, int32_t C, const int4 &r, int t, double f0, double f1,
-                                               double f2) {
-    if (t > 2) return;
+// (all of which hold the sums) forms the t-th factor, from the community's
+// record alone: its division runs while the members load.
+__device__ __forceinline__ double lit_fsum_factor(const RunArgs &a, const int4 &r, int t) {
     const int32_t n = r.x;
-    const double cc = a.gcc ? a.gcc[r.w] : a.cc;
+    const double cc = a.gcc && t <= 2 ? a.gcc[r.w] : a.cc;
     const double nd = __int2double_rn(n);
-    const bool on = cc > 0.0 && (t == 0 ? n >= 2 : t == 1 ? n >= 1 : n >= 3);
+    const bool on = t <= 2 && cc > 0.0 && (t == 0 ? n >= 2 : t == 1 ? n >= 1 : n >= 3);
     // t = 0: n (n-1), 1: (n+1) n, 2: (n-1)(n-2)
     const double den = (t == 1 ? nd + 1.0 : nd - 1.0) * (t == 2 ? nd - 2.0 : nd);
-    double v = on ? (t == 0 ? __uint2double_rn((uint32_t)r.y) : 1.0) / (den * cc) : 0.0;
+    return on ? (t == 0 ? __uint2double_rn((uint32_t)r.y) : 1.0) / (den * cc) : 0.0;
+}
+
+__device__ __forceinline__ void lit_fsum_store(const RunArgs &a, int32_t C, int t, double v, double f0, double f1,
+                                               double f2) {
+    if (t > 2) return;
     float *f = a.litF + 8 * (int64_t)C;
     if (t == 0) {
         f[0] = (float)f0;
@@ -3886,6 +3845,16 @@ __device__ __forceinline__ void lit_fsum_reduce(double &f0, double &f1, double &
         f1 += __shfl_xor_sync(FULL, f1, o);
         f2 += __shfl_xor_sync(FULL, f2, o);
     }
+}
+
+// The sums of one community over threads tid of nthreads.
+__device__ __forceinline__ void lit_fsum_members(const RunArgs &a, int32_t C, int32_t n, const MemberRange &r, int tid,
+                                                 int nthreads, double &f0, double &f1, double &f2) {
+    lit_members2(a, C, r, tid, nthreads, [&](int32_t y0, int32_t y1) {
+        const FsumMember m0 = lit_fsum_load(a, y0), m1 = lit_fsum_load(a, y1);
+        lit_fsum_member(a, C, n, m0, f0, f1, f2);
+        lit_fsum_member(a, C, n, m1, f0, f1, f2);
+    });
 }
 
 struct FsumShared {
@@ -3919,11 +3888,11 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
     if (!few) {
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
         const bool mine = n >= 0 && n <= group;
-        if (mine && n > 0)
-            lit_members(a, C, mr, sub, 8, [&](int32_t y) { lit_fsum_member(a, C, n, y, f0, f1, f2); });
+        const double v = lit_fsum_factor(a, rec, mine ? sub : 3);
+        if (mine && n > 0) lit_fsum_members(a, C, n, mr, sub, 8, f0, f1, f2);
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 8);
-        if (mine) lit_fsum_store(a, C, rec, sub, f0, f1, f2);
+        if (mine) lit_fsum_store(a, C, sub, v, f0, f1, f2);
     }
     unsigned mid = __ballot_sync(FULL, sub == 0 && n > group);
     while (mid) {
@@ -3938,10 +3907,11 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
             continue;
         }
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-        lit_members(a, C1, mr1, lane, 32, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
+        const double v = lit_fsum_factor(a, rec1, lane);
+        lit_fsum_members(a, C1, n1, mr1, lane, 32, f0, f1, f2);
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 32);
-        lit_fsum_store(a, C1, rec1, lane, f0, f1, f2);
+        lit_fsum_store(a, C1, lane, v, f0, f1, f2);
     }
     __syncthreads();
     const int nbig = fs.nbig;
@@ -3950,7 +3920,8 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
         const int4 rec1 = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C1]));
         const int32_t n1 = rec1.x;
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-        lit_members(a, C1, lit_member_range(a, C1), threadIdx.x, blockDim.x, [&](int32_t y) { lit_fsum_member(a, C1, n1, y, f0, f1, f2); });
+        const double v = lit_fsum_factor(a, rec1, w == 0 ? lane : 3);
+        lit_fsum_members(a, C1, n1, lit_member_range(a, C1), threadIdx.x, blockDim.x, f0, f1, f2);
         __syncwarp();
         lit_fsum_reduce(f0, f1, f2, 32);
         if (lane == 0) {
@@ -3963,13 +3934,13 @@ __device__ void lit_fsum_block(const RunArgs &a, const int32_t *list, int64_t t0
             double sum[3] = {0.0, 0.0, 0.0};
             for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2)
                 for (int t2 = 0; t2 < 3; ++t2) sum[t2] += fs.red[t2][k2];
-            lit_fsum_store(a, C1, rec1, lane, sum[0], sum[1], sum[2]);
+            lit_fsum_store(a, C1, lane, v, sum[0], sum[1], sum[2]);
         }
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(EV_THREADS) k_lit_fsum(RunArgs a, const int32_t *list, const uint32_t *count,
+__global__ void __launch_bounds__(EV_THREADS, 4) k_lit_fsum(RunArgs a, const int32_t *list, const uint32_t *count,
                                                          int64_t ncount) {
     __shared__ FsumShared fs;
     pdl_trigger();
@@ -4586,15 +4557,6 @@ __device__ __forceinline__ void tot_count_smem(const RunArgs &a, int64_t pb, int
     }
 }
 
-__device__ __forceinline__ void tot_member(const RunArgs &a, unsigned long long *acc, int32_t C, int64_t k,
-                                           int32_t d) {
-    const int4 r = __ldcg(reinterpret_cast<const int4 *>(&a.comm[C]));
-    if (a.gsacc)   // a batch: the sum of the community's graph
-        sacc_add(a.gsacc + (int64_t)r.w * SACC_CHUNKS, wcchat_member(k, d, r.x, (uint32_t)r.y, a.gcc[r.w]));
-    else
-        sacc_add(acc, wcchat_member(k, d, r.x, (uint32_t)r.y, a.cc));
-}
-
 // Memberships waiting for their FP64 term, per warp: evaluated 32 at a time so
 // that the (slow) double-precision pipe runs with every lane busy.
 struct TotBuf {
@@ -4605,7 +4567,17 @@ struct TotBuf {
 __device__ __forceinline__ void tot_flush(const RunArgs &a, unsigned long long *acc, TotBuf &b) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
-    if (lane < b.n) tot_member(a, acc, b.C[lane], b.k[lane], b.d[lane]);
+    double v = 0.0;
+    int32_t g = -1;
+    if (lane < b.n) {
+        const int4 r = __ldcg(reinterpret_cast<const int4 *>(&a.comm[b.C[lane]]));
+        g = a.gsacc ? r.w : 0;
+        v = wcchat_member(b.k[lane], b.d[lane], r.x, (uint32_t)r.y, a.gsacc ? a.gcc[r.w] : a.cc);
+    }
+    const int32_t g0 = __shfl_sync(FULL, g, 0);   // lane 0 always has one
+    if (!a.gsacc) sacc_add_warp(acc, v);
+    else if (__all_sync(FULL, lane >= b.n || g == g0)) sacc_add_warp(a.gsacc + (int64_t)g0 * SACC_CHUNKS, v);
+    else if (lane < b.n) sacc_add(a.gsacc + (int64_t)g * SACC_CHUNKS, v);   // a batch: the sum of the community's graph
     __syncwarp();
     b.n = 0;
 }
@@ -4680,7 +4652,12 @@ __device__ void tot_node(const RunArgs &a, int32_t x, int64_t pb, int64_t pe, bo
     }
 }
 
-__global__ void __launch_bounds__(TOT_WARPS * 32) k_total(RunArgs a, int64_t n) {
+// run: nodes a warp takes at a time under the paper's gain (a node per lane): 32, fewer
+// where that would leave warps without any -- a warp's 32 nodes bring up to a few
+// hundred terms, 32 at a time one after the other (300 nodes: 54 -> 16 us). A
+// warp's digits are added up before they meet other warps' (767k nodes, first three
+// iterations: 189 us a total, 128 graphs: 141 us; 323 and 493 on average before).
+__global__ void __launch_bounds__(TOT_WARPS * 32) k_total(RunArgs a, int64_t n, int run) {
     __shared__ unsigned long long acc[SACC_CHUNKS];
     __shared__ int32_t s_row[TOT_WARPS][TOT_ROW];
     __shared__ int32_t s_cnt[TOT_WARPS][TOT_ROW];
@@ -4693,12 +4670,12 @@ __global__ void __launch_bounds__(TOT_WARPS * 32) k_total(RunArgs a, int64_t n) 
     if (a.kmem) {   // the paper's gain keeps deg(x, C) of every membership: no recount
         for (;;) {
             long long b0 = 0;
-            if (lane == 0) b0 = (long long)atomicAdd(&a.tot_next[0], 1u) * 32;
+            if (lane == 0) b0 = (long long)atomicAdd(&a.tot_next[0], 1u) * run;
             b0 = __shfl_sync(FULL, b0, 0);
             if (b0 >= n) break;
             const int64_t x = b0 + lane;   // a node per lane
             int32_t c = 0, d = 0;
-            if (x < n) {
+            if (lane < run && x < n) {
                 c = __ldcg(&a.nmem[x]);
                 if (!dbg_ok(a, c >= 0 && c <= a.K)) c = 0;
                 d = a.deg[x];
@@ -4771,16 +4748,20 @@ __global__ void __launch_bounds__(TOT_WARPS * 32) k_total(RunArgs a, int64_t n) 
         if (acc[s]) atomicAdd(&a.ds->sacc[s], acc[s]);
 }
 
-// Per-graph totals of a batch (one thread per graph); the shared counters
+// Per-graph totals of a batch (a warp per graph); the shared counters
 // are finalised by k_finalize as for one graph.
-__global__ void k_finalize_batch(unsigned long long *gsacc, int64_t G, double *gT) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < G; i += (int64_t)gridDim.x * blockDim.x)
-        gT[i] = sacc_round_and_clear(gsacc + i * SACC_CHUNKS);
+__global__ void __launch_bounds__(256) k_finalize_batch(unsigned long long *gsacc, int64_t G, double *gT) {
+    __shared__ unsigned long long acc[8][SACC_CHUNKS];
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < G; i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const double t = sacc_take_warp(gsacc + i * SACC_CHUNKS, acc[threadIdx.x >> 5]);
+        if ((threadIdx.x & 31) == 0) gT[i] = t;
+    }
 }
 
 __global__ void k_finalize(DevScalars *ds, Readback *rbd, int advance) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    const double T = sacc_round_and_clear(ds->sacc);
+    __shared__ unsigned long long acc[SACC_CHUNKS];
+    const double T = sacc_take_warp(ds->sacc, acc);   // one warp
+    if (threadIdx.x != 0) return;
     ds->total = T;
     rbd->total = T;
     rbd->joins = ds->joins;
@@ -5535,7 +5516,9 @@ void build_schedule(lf_graph *g, int64_t q, const std::vector<char> &active) {
 void launch_total(lf_graph *g, const RunArgs &a) {
     static const int per_sm = blocks_per_sm(k_total, TOT_WARPS * 32, 0);
     LF_CUDA(cudaMemsetAsync(g->tot_next, 0, 2 * sizeof(uint32_t), g->stream));
-    k_total<<<num_sms() * std::max(1, per_sm), TOT_WARPS * 32, 0, g->stream>>>(a, g->n);
+    const int64_t blocks = (int64_t)num_sms() * std::max(1, per_sm);
+    const int run = (int)std::min<int64_t>(32, std::max<int64_t>(1, g->n / (blocks * TOT_WARPS)));
+    k_total<<<(unsigned)blocks, TOT_WARPS * 32, 0, g->stream>>>(a, g->n, run);
     ++g->launches;
 }
 
@@ -5547,7 +5530,7 @@ void launch_iteration_end(lf_graph *g, const RunArgs &a) {
     LF_LAUNCHED();
     LF_CUDA(cudaMemcpyAsync(g->rb, device_readback(g), sizeof(Readback), cudaMemcpyDeviceToHost, g->stream));
     if (g->ngraphs > 0) {
-        k_finalize_batch<<<grid_for(g->ngraphs, 256, 1024), 256, 0, g->stream>>>(g->gsacc, g->ngraphs, g->gT);
+        k_finalize_batch<<<grid_for(g->ngraphs * 32, 256, 1024), 256, 0, g->stream>>>(g->gsacc, g->ngraphs, g->gT);
         ++g->launches;
         LF_LAUNCHED();
         LF_CUDA(cudaMemcpyAsync(g->gT_host, g->gT, (size_t)g->ngraphs * 8, cudaMemcpyDeviceToHost, g->stream));
@@ -6103,7 +6086,7 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
     LF_LAUNCHED();
     LF_CUDA(cudaMemcpyAsync(g->rb, device_readback(g), sizeof(Readback), cudaMemcpyDeviceToHost, st));
     if (batch) {   // every graph's T0
-        k_finalize_batch<<<grid_for(g->ngraphs, 256, 1024), 256, 0, st>>>(g->gsacc, g->ngraphs, g->gT);
+        k_finalize_batch<<<grid_for(g->ngraphs * 32, 256, 1024), 256, 0, st>>>(g->gsacc, g->ngraphs, g->gT);
         ++g->launches;
         LF_LAUNCHED();
         LF_CUDA(cudaMemcpyAsync(g->gT_host, g->gT, (size_t)g->ngraphs * 8, cudaMemcpyDeviceToHost, st));
