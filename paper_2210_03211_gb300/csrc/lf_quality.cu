@@ -265,9 +265,9 @@ __global__ void __launch_bounds__(F1_THREADS) k_cover_f1(const int64_t *off_a, c
 }
 
 __global__ void k_f1_final(unsigned long long *sacc, int64_t ka, double *out) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    const double s = sacc_round_and_clear(sacc);
-    *out = ka > 0 ? __ddiv_rn(s, (double)ka) : 0.0;
+    __shared__ unsigned long long acc[SACC_CHUNKS];
+    const double s = sacc_take_warp(sacc, acc);   // one warp
+    if (threadIdx.x == 0) *out = ka > 0 ? __ddiv_rn(s, (double)ka) : 0.0;
 }
 
 }  // namespace
@@ -297,19 +297,28 @@ extern "C" lf_status lf_cover_f1(const int64_t *det_offsets, const int32_t *det_
         const int64_t ea = det_offsets[num_det], eb = num_ref > 0 ? ref_offsets[num_ref] : 0;
         if (det_offsets[0] != 0 || (num_ref > 0 && ref_offsets[0] != 0)) fail(LF_ERR_INVALID, "offsets must start at 0");
         if ((ea > 0 && !det_members) || (eb > 0 && !ref_members)) fail(LF_ERR_INVALID, "members is NULL");
-        for (int64_t c = 0; c < num_det; ++c)
-            if (det_offsets[c + 1] <= det_offsets[c]) fail(LF_ERR_INVALID, "detected community %lld is empty", (long long)c);
-        for (int64_t c = 0; c < num_ref; ++c)
-            if (ref_offsets[c + 1] <= ref_offsets[c]) fail(LF_ERR_INVALID, "reference community %lld is empty", (long long)c);
-        uint32_t max_id = 0;
-        for (int64_t i = 0; i < ea; ++i) {
-            if (det_members[i] < 0) fail(LF_ERR_INVALID, "negative node id");
-            max_id = std::max(max_id, (uint32_t)det_members[i]);
-        }
-        for (int64_t i = 0; i < eb; ++i) {
-            if (ref_members[i] < 0) fail(LF_ERR_INVALID, "negative node id");
-            max_id = std::max(max_id, (uint32_t)ref_members[i]);
-        }
+        // whole passes without a branch (they vectorise); what is wrong is looked up afterwards
+        auto offsets_ok = [](const int64_t *off, int64_t k) {
+            bool ok = true;
+            for (int64_t c = 0; c < k; ++c) ok &= off[c + 1] > off[c];
+            return ok;
+        };
+        auto first_empty = [](const int64_t *off) {
+            int64_t c = 0;
+            while (off[c + 1] > off[c]) ++c;
+            return (long long)c;
+        };
+        if (!offsets_ok(det_offsets, num_det))
+            fail(LF_ERR_INVALID, "detected community %lld is empty", first_empty(det_offsets));
+        if (!offsets_ok(ref_offsets, num_ref))
+            fail(LF_ERR_INVALID, "reference community %lld is empty", first_empty(ref_offsets));
+        auto largest = [](const int32_t *m, int64_t n) {   // as unsigned: a negative id is above every other
+            uint32_t top = 0;
+            for (int64_t i = 0; i < n; ++i) top = std::max(top, (uint32_t)m[i]);
+            return top;
+        };
+        const uint32_t max_id = std::max(largest(det_members, ea), largest(ref_members, eb));
+        if (max_id > 0x7fffffffu) fail(LF_ERR_INVALID, "negative node id");
         auto alloc = [&](size_t bytes) {
             void *d = dalloc(&tmp, bytes > 0 ? bytes : 8);
             bufs.push_back(d);
