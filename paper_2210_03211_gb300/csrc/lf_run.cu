@@ -2417,15 +2417,13 @@ __device__ __forceinline__ bool lit_fill(const RunArgs &a, const LitNode &ln, in
         });
     }
     // a full table: the whole team starts over with more parts
+    ok = __all_sync(FULL, ok);
     if constexpr (T > 1) {
-        const bool all = __all_sync(FULL, ok);
-        if (lane == 0) ls.flag[w] = all ? 1 : 0;
+        if (lane == 0) ls.flag[w] = ok ? 1 : 0;
         team_sync<T>(tm);
         for (int k2 = 0; k2 < T; ++k2) ok &= ls.flag[tm * T + k2] != 0;
-        team_sync<T>(tm);
-    } else {
-        ok = __all_sync(FULL, ok);
     }
+    team_sync<T>(tm);   // the vote alone orders no memory: every lane's inserts before the table is read
     return ok;
 }
 
