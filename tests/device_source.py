@@ -10,10 +10,11 @@ import subprocess
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2210_03211_gb300", "csrc")
 
 SHIM = r"""
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
-using std::fma; using std::fmaf; using std::isfinite;
+using std::min; using std::max; using std::fma; using std::fmaf; using std::isfinite;
 #define __device__
 #define __forceinline__ inline
 struct int4 { int x, y, z, w; };
@@ -21,6 +22,7 @@ struct float4 { float x, y, z, w; };
 static inline float __uint2float_rn(uint32_t v) { return (float)v; }
 static inline double __uint2double_rn(uint32_t v) { return (double)v; }
 static inline double __int2double_rn(int32_t v) { return (double)v; }
+static inline uint32_t __umulhi(uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); }
 template <typename T> static inline T __ldcg(const T *p) { T v; std::memcpy(&v, p, sizeof v); return v; }
 struct CommRec { int32_t n; uint32_t m2, vol; int32_t gid; };   // sixteen bytes, read as an int4
 struct RunArgs { const CommRec *comm; float *litF; const double *gcc; double cc; };
@@ -34,6 +36,9 @@ def constant(text, name):
 def function(text, name):
     m = re.search(r"__device__ __forceinline__ [\w ]*\b%s\(" % name, text)
     start = m.start()
+    line = text[start:text.index("\n", start) + 1]
+    if line.rstrip().endswith("}"):   # on one line
+        return line
     return text[start:text.index("\n}\n", start) + 3]
 
 
