@@ -257,8 +257,9 @@ struct lf_graph {
     // and part items of all queues (offsets per queue on the host); the entries,
     // their groups' offsets and the candidate lists, shared by the queues
     int64_t lh_plan_q = -1, lh_plan_sched = -1;
-    int32_t lh_plan_K = 0;
+    int32_t lh_plan_K = 0, lh_plan_deg = 0;
     int64_t lh_n = 0;
+    bool lit_loop = false;                // this run's queues go through k_lit_iterate: no hub kernels
     std::vector<int64_t> lh_fq, lh_pq, lh_hq;
     int32_t *lh_pos = nullptr, *lh_fh = nullptr, *lh_fc = nullptr, *lh_ph = nullptr, *lh_pp = nullptr,
             *lh_lb = nullptr, *lh_ent = nullptr, *lh_cand = nullptr;

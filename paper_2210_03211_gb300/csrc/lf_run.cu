@@ -4351,8 +4351,8 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_iterate(RunArgs a, int64_t q,
 // boundaries to it, reload what a block has just had (a block applies the nodes it
 // evaluated, the next queue's static data load while a barrier completes) and
 // read lists to find their work.
-// Only for graphs without hubs (degree above LIT_HUB_DEG), which need the many-block
-// kernels.
+// Only for graphs without nodes of degree above LIT_HUB_DEG, which need the many-block
+// kernels; nodes up to it are a block's here, whatever the rows hold.
 // ---------------------------------------------------------------------------
 struct LitIterShared {
     LitScratch ls;
@@ -4905,7 +4905,7 @@ RunArgs make_args(lf_graph *g, Readback *rbd) {
     a.lg_keys = reinterpret_cast<int32_t *>(a.lg_dv + g->lg_cap);
     a.lg_vals = reinterpret_cast<uint32_t *>(a.lg_keys + g->lg_cap);
     a.lg_aux = reinterpret_cast<int32_t *>(a.lg_vals + g->lg_cap);
-    a.lit_hub_deg = g->lh_n > 0 ? (g->lh_plan_K <= 4 ? LIT_HUB_DEG : LIT_HUB_DEG_LONG) : 0x7fffffff;
+    a.lit_hub_deg = g->lh_n > 0 ? g->lh_plan_deg : 0x7fffffff;
     if (lit) a.screen = g->screen ? 1 : 0;   // brackets need no FP32 range condition
     return a;
 }
@@ -5137,7 +5137,11 @@ void launch_batches(lf_graph *g, const RunArgs &a, int64_t q, int64_t first, int
     LF_LAUNCHED();
 }
 
-int32_t lit_hub_degree(const lf_graph *g) { return g->K <= 4 ? LIT_HUB_DEG : LIT_HUB_DEG_LONG; }
+// Degree above which the hub kernels take a node; the persistent loop has none, so its
+// global tables are planned for every node.
+int32_t lit_hub_degree(const lf_graph *g) {
+    return g->lit_loop ? 0x7fffffff : g->K <= 4 ? LIT_HUB_DEG : LIT_HUB_DEG_LONG;
+}
 
 void free_lit_hub_plan(lf_graph *g) {
     auto drop = [&](auto *&p) {
@@ -5154,7 +5158,7 @@ void free_lit_hub_plan(lf_graph *g) {
     g->lh_pq.clear();
     g->lh_hq.clear();
     g->lh_plan_q = g->lh_plan_sched = -1;
-    g->lh_plan_K = 0;
+    g->lh_plan_K = g->lh_plan_deg = 0;
 }
 
 // Queues up to this size run in the persistent loop under the paper's gain: at
@@ -5199,7 +5203,9 @@ __global__ void k_lit_plan(const int32_t *order, const int32_t *deg, int64_t len
 // after the other, so they share the areas.  Also the global tables of the other
 // nodes (lg_area), sized for the largest queue.
 void build_lit_hub_plan(lf_graph *g, int64_t q, int64_t nb) {
-    if (g->lh_plan_q == q && g->lh_plan_K == g->K && g->lh_plan_sched == g->sched_version) return;
+    if (g->lh_plan_q == q && g->lh_plan_K == g->K && g->lh_plan_deg == lit_hub_degree(g) &&
+        g->lh_plan_sched == g->sched_version)
+        return;
     free_lit_hub_plan(g);
     drop_graph(g);
     g->lh_fq.assign((size_t)nb + 1, 0);
@@ -5308,6 +5314,7 @@ void build_lit_hub_plan(lf_graph *g, int64_t q, int64_t nb) {
     }
     g->lh_plan_q = q;
     g->lh_plan_K = g->K;
+    g->lh_plan_deg = lit_hub_degree(g);
     g->lh_plan_sched = g->sched_version;
 }
 
@@ -6099,6 +6106,12 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
     }
     g->ncomm = k0;
     const bool lit = g->gain_rule == LF_GAIN_LITERAL;
+    // measured on GB300: the persistent loop wins for small queues (grid
+    // barriers over few blocks), launches per queue for large ones
+    const bool loop_ok = !batch && (!lit || g->max_deg <= LIT_HUB_DEG);
+    const bool persistent =
+        loop_ok && (g->per_queue == 0 || (g->per_queue < 0 && q <= (lit ? LIT_LOOP_MAX_Q : 256)));
+    g->lit_loop = lit && persistent;
     if (lit && n > 0) {   // deg(x,C) of every membership of the starting state
         ensure_lit(g, batch ? max_queue(g, q) : q, num_queues(g, q));
         a = make_args(g, device_readback(g));
@@ -6129,11 +6142,6 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
     int64_t nb = num_queues(g, q);
     if (batch && !lit) ensure_dyn(g, max_queue(g, q), nb);
     else if (!lit && use_dyn(g, q)) ensure_dyn(g, q, nb);
-    // measured on GB300: the persistent loop wins for small queues (grid
-    // barriers over few blocks), launches per queue for large ones
-    const bool loop_ok = !batch && (!lit || g->max_deg <= LIT_HUB_DEG);
-    const bool persistent =
-        loop_ok && (g->per_queue == 0 || (g->per_queue < 0 && q <= (lit ? LIT_LOOP_MAX_Q : 256)));
     const int team = choose_team(g, q);
     const int grid_max = !persistent ? 0 : lit ? lit_persistent_grid_max(team) : persistent_grid_max(g, team);
     if (persistent) {

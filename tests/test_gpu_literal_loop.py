@@ -1,0 +1,42 @@
+"""The persistent queue loop under the paper's gain (one block at queue size 1): what
+it plans and how it compares with the oracle on graphs with nodes of 513 to 1,024
+neighbours and rows of more than four communities, which launches per queue give
+to the hub kernels and the loop evaluates in its own block."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def graph(nodes=900, busy=12, seed=0):
+    """`busy` nodes of 520 to 880 neighbours over a sparse random background."""
+    rng = np.random.default_rng(seed)
+    rest = np.arange(busy, nodes)
+    src, dst = [rng.choice(rest, 2000)], [rng.choice(rest, 2000)]
+    for i, d in enumerate(np.linspace(520, 880, busy).astype(int)):
+        src.append(np.full(d, i))
+        dst.append(rng.permutation(rest)[:d])
+    return np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+
+
+def test_loop_plans_no_hub_kernels():
+    """The hub plan is thirteen allocations; the loop makes none of them, keeps tables
+    in global memory for its own large nodes, and its run is the oracle's."""
+    import oracle
+    import torch
+    from paper_2210_03211_gb300 import lazyfox
+    src, dst = graph()
+    ref = oracle.OracleGraph(src, dst).run(1, -np.inf, 2, rule="literal")
+    made = {}
+    for per_queue in (None, True):
+        alloc = lazyfox.CountingAllocator(torch.device("cuda", torch.cuda.current_device()))
+        with lazyfox.Graph(src, dst, gain_rule="literal", member_slots=32, allocator=alloc,
+                           per_queue_launches=per_queue) as g:
+            before = alloc.calls
+            st = g.run(1, -np.inf, 2)
+            made[per_queue] = alloc.calls - before
+            assert np.array_equal(st.wcc_history, ref["T"])
+            assert np.array_equal(st.joins, ref["joins"]) and np.array_equal(st.leaves, ref["leaves"])
+        assert alloc.live == 0
+    # the loop's own: its barrier flags and one area of global tables
+    assert made[None] <= made[True] - 13 + 2, made
