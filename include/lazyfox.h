@@ -73,9 +73,12 @@ typedef struct lf_options {
                                 iteration captured in a CUDA graph; 2: one persistent
                                 cooperative kernel per iteration runs every queue
                                 (evaluate, grid barrier, apply, grid barrier); 0 (default):
-                                persistent for queues of at most 256 nodes (LF_GAIN_LITERAL: 1
-                                node, and never for graphs with nodes of degree above 1024 or
-                                batches), else per queue */
+                                persistent for queues of at most 256 nodes, else per queue.
+                                Batches always launch per queue.  LF_GAIN_LITERAL: the
+                                persistent kernel is the faster one for queues of 1 node only,
+                                so 0 and 2 take it for these and launch per queue otherwise; 2
+                                together with barrier_mode 1 or inject_barrier_stall takes it for
+                                any size; never for graphs with nodes of degree above 1024 */
     int32_t barrier_timeout_ms; /* bound on one grid-barrier wait (0: 2000 ms); a wait that
                                 runs out ends the call with LF_ERR_TIMEOUT */
     int32_t inject_barrier_stall; /* test hook: 1 makes one block of the persistent kernel
@@ -84,7 +87,8 @@ typedef struct lf_options {
                                 polls all arrival flags; 1 block 0 gathers them and
                                 publishes one release flag */
     int32_t warps_per_node;  /* warps that evaluate one node together: 1, 2, 4 or 8; 0 (default)
-                                picks by queue size (more warps per node for small queues) */
+                                picks by queue size (more warps per node for small queues); the
+                                persistent kernel of LF_GAIN_LITERAL always has 8 */
     int32_t hub_degree;      /* nodes of higher degree are evaluated with a table in global
                                 memory, in blocks of their own (per-queue launches: on a second
                                 stream); 0 (default) = 384 */

@@ -4344,9 +4344,10 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_iterate(RunArgs a, int64_t q,
 
 // ---------------------------------------------------------------------------
 // Persistent queue loop under the paper's gain: one cooperative launch runs
-// queues first .. first + count - 1 of an iteration, each evaluate | apply | member
-// sums of the touched communities, with a grid barrier after each step (a
-// __syncthreads when one block holds the queue: Fox).  A short queue's time is
+// queues first .. first + count - 1 of an iteration, a block per queued node, each
+// evaluate | apply | member sums of the touched communities, with a grid barrier
+// after each step (a __syncthreads when one block holds the queue: Fox, the one case
+// it is chosen for; see LIT_LOOP_MAX_Q).  A short queue's time is
 // the latency of its chain of dependent loads; per-queue launches add four launch
 // boundaries to it, reload what a block has just had (a block applies the nodes it
 // evaluated, the next queue's static data load while a barrier completes) and
@@ -4357,12 +4358,10 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_iterate(RunArgs a, int64_t q,
 struct LitIterShared {
     LitScratch ls;
     FsumShared fs;
-    int2 over[EV_WARPS];
-    int nover, ok;
+    int ok;
     long long base;
 };
 
-template <int T>
 __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, int64_t q, int64_t first, int64_t count,
                                                               uint32_t *ctr, unsigned long long *used,
                                                               long long spin_limit, int inject_stall, unsigned *flags,
@@ -4371,9 +4370,6 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, int64_
     __shared__ LitIterShared sh;
     const LitTables t = lit_tables(lit_dyn);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tm = w / T, w_in = w % T;
-    constexpr int TEAMS = EV_WARPS / T;
-    const int64_t round = (int64_t)gridDim.x * TEAMS;
     unsigned long long nj = 0, nl = 0;
     if (inject_stall && blockIdx.x == 0 && gridDim.x > 1) return;   // test hook: a block that never arrives
     auto bounds = [&](int64_t b, int64_t &start, int32_t &len) {
@@ -4391,44 +4387,35 @@ __global__ void __launch_bounds__(EV_THREADS, 2) k_lit_iterate(RunArgs a, int64_
     int32_t blen;
     bounds(first, bstart, blen);
     NodePrefetch pf;
-    const int base0 = (int)blockIdx.x * TEAMS;
-    prefetch_node(a, bstart, blen, base0 + tm, w_in, pf);
+    const int i0 = (int)blockIdx.x, step = (int)gridDim.x;
+    prefetch_node(a, bstart, blen, i0, w, pf);
     if (a.qtimes && blockIdx.x == 0 && threadIdx.x == 0) a.qtimes[0] = global_ns();
     for (int64_t b = first; b < first + count; ++b) {
         const uint32_t serial = (uint32_t)queue_serial(a, b);
         a.ntouched = ctr + 8 * b + 2;
         // evaluate
         NodePrefetch cur = pf;
-        for (int64_t base = base0; base < blen; base += round) {
-            const int i = (int)base + tm;
-            if (base != base0) prefetch_node(a, bstart, blen, i, w_in, cur);
-            if (threadIdx.x == 0) sh.nover = 0;
-            __syncthreads();
-            long long bound = 0;
-            if (i < blen && !lit_eval_team<T>(a, i, cur, t, sh.ls, tm, w_in, bound) && w_in == 0 && lane == 0)
-                sh.over[atomicAdd(&sh.nover, 1)] = make_int2(i, (int)min(bound, 0x7fffffffll));
-            __syncthreads();
-            const int nover = sh.nover;
-            for (int h = 0; h < nover; ++h)
-                lit_big_node(a, bstart, sh.over[h].x, sh.over[h].y, t, sh.ls, sh.base, used + b);
+        for (int64_t i = i0; i < blen; i += step) {
+            if (i != i0) prefetch_node(a, bstart, blen, (int)i, w, cur);
+            long long bound = 0;   // the same on all warps, as is the answer
+            if (!lit_eval_team<EV_WARPS>(a, (int)i, cur, t, sh.ls, 0, w, bound))
+                lit_big_node(a, bstart, (int)i, bound, t, sh.ls, sh.base, used + b);
         }
         if (!meet()) return;
-        // apply: each team's first warp, its own nodes
-        for (int64_t base = base0; base < blen; base += round) {
-            const int i = (int)base + tm;
-            if (base != base0) prefetch_node(a, bstart, blen, i, w_in, cur);
+        // apply: the first warp, the block's own nodes
+        for (int64_t i = i0; w == 0 && i < blen; i += step) {
+            if (i != i0) prefetch_node(a, bstart, blen, (int)i, w, cur);
             else cur = pf;
-            if (i >= blen || w_in != 0) continue;
             ApplyPrefetch ap{cur.x, cur.y0, cur.beg, cur.end, -1};
             if (cur.beg + lane < cur.end) ap.py0 = a.pos[cur.y0];
             for (int piece = 0; piece == 0 || piece * AP_CHUNK < cur.d; ++piece)
-                lit_apply_piece(a, bstart, blen, i, piece, ap, serial, nj, nl);
+                lit_apply_piece(a, bstart, blen, (int)i, piece, ap, serial, nj, nl);
         }
         // the next queue's static data load while the barrier completes
         const bool more = b + 1 < first + count;
         if (more) {
             bounds(b + 1, bstart, blen);
-            prefetch_node(a, bstart, blen, base0 + tm, w_in, pf);
+            prefetch_node(a, bstart, blen, i0, w, pf);
         }
         if (!meet()) return;
         const int64_t total = __ldcg(a.ntouched);
@@ -5164,7 +5151,10 @@ void free_lit_hub_plan(lf_graph *g) {
 // Queues up to this size run in the persistent loop under the paper's gain: at
 // queue size 1 one block holds it, with no grid barrier.  Measured, us a queue, loop /
 // launches: 1,000 nodes (planted) q 1 13.3 / 16.9, q 2 19.2 / 17.8, q 8 21.0 / 21.1, q 16
-// 23.2 / 22.4; 84k nodes q 64 25.0 / 21.9, q 256 36.4 / 27.6.
+// 23.2 / 22.4; 84k nodes q 64 25.0 / 21.9, q 256 36.4 / 27.6; q 1 on 20,000 nodes
+// (planted) 13.9 / 17.2, on 33k (power law) 8.4 / 10.3, on 20,000 of which 400 have 520-880
+// neighbours 6.3 / 8.1.  So longer queues are launched also where the caller prefers
+// the loop, unless an option of its barrier is set with it.
 constexpr int64_t LIT_LOOP_MAX_Q = 1;
 
 // The nodes of degree > hub_deg by position in the order the queues take,
@@ -5656,30 +5646,18 @@ void launch_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int64_t
     if (e1) LF_CUDA(cudaEventRecord(e1, g->stream));
 }
 
-const void *lit_iterate_kernel_for(int T) {
-    switch (T) {
-    case 1: return (const void *)k_lit_iterate<1>;
-    case 2: return (const void *)k_lit_iterate<2>;
-    case 4: return (const void *)k_lit_iterate<4>;
-    default: return (const void *)k_lit_iterate<8>;
-    }
-}
-
-int lit_persistent_grid_max(int T) {
+int lit_persistent_grid_max() {
     int per_sm = 0;
-    const void *k = lit_iterate_kernel_for(T);
-    LF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
-    LF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, EV_THREADS, LIT_SMEM));
+    LF_CUDA(cudaFuncSetAttribute(k_lit_iterate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIT_SMEM));
+    LF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lit_iterate, EV_THREADS, LIT_SMEM));
     return std::max(1, per_sm) * num_sms();
 }
 
 // One cooperative launch runs queues first .. first+count-1 under the paper's gain.
-void launch_lit_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int64_t count, int grid_max, int T,
+void launch_lit_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int64_t count, int grid_max,
                            cudaEvent_t e0, cudaEvent_t e1) {
     if (count <= 0) return;
-    const int64_t teams = EV_WARPS / T;
-    const int64_t want = (q + teams - 1) / teams;
-    unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, grid_max));
+    unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(q, grid_max));
     long long spin = (long long)g->barrier_timeout_ms * 4000ll;   // >= ~250 ns per poll of the flags
     int inject = g->inject_stall;
     unsigned *flags = g->bar_flags;
@@ -5693,7 +5671,7 @@ void launch_lit_persistent(lf_graph *g, RunArgs a, int64_t q, int64_t first, int
     LF_CUDA(cudaMemsetAsync(used + first, 0, (size_t)count * sizeof(unsigned long long), g->stream));
     void *args[] = {&a, &q, &first, &count, &ctr, &used, &spin, &inject, &flags, &epoch, &bar_mode};
     if (e0) LF_CUDA(cudaEventRecord(e0, g->stream));
-    LF_CUDA(cudaLaunchCooperativeKernel(lit_iterate_kernel_for(T), dim3(grid), dim3(EV_THREADS), args, LIT_SMEM,
+    LF_CUDA(cudaLaunchCooperativeKernel((const void *)k_lit_iterate, dim3(grid), dim3(EV_THREADS), args, LIT_SMEM,
                                         g->stream));
     ++g->launches;
     if (e1) LF_CUDA(cudaEventRecord(e1, g->stream));
@@ -6109,8 +6087,8 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
     // measured on GB300: the persistent loop wins for small queues (grid
     // barriers over few blocks), launches per queue for large ones
     const bool loop_ok = !batch && (!lit || g->max_deg <= LIT_HUB_DEG);
-    const bool persistent =
-        loop_ok && (g->per_queue == 0 || (g->per_queue < 0 && q <= (lit ? LIT_LOOP_MAX_Q : 256)));
+    const bool asked = g->per_queue == 0 && (!lit || g->barrier_mode == 1 || g->inject_stall);
+    const bool persistent = loop_ok && (asked || (g->per_queue <= 0 && q <= (lit ? LIT_LOOP_MAX_Q : 256)));
     g->lit_loop = lit && persistent;
     if (lit && n > 0) {   // deg(x,C) of every membership of the starting state
         ensure_lit(g, batch ? max_queue(g, q) : q, num_queues(g, q));
@@ -6143,7 +6121,7 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
     if (batch && !lit) ensure_dyn(g, max_queue(g, q), nb);
     else if (!lit && use_dyn(g, q)) ensure_dyn(g, q, nb);
     const int team = choose_team(g, q);
-    const int grid_max = !persistent ? 0 : lit ? lit_persistent_grid_max(team) : persistent_grid_max(g, team);
+    const int grid_max = !persistent ? 0 : lit ? lit_persistent_grid_max() : persistent_grid_max(g, team);
     if (persistent) {
         if (g->bar_flags_cap < grid_max + 1) {
             if (g->bar_flags) dfree(g, g->bar_flags);
@@ -6186,7 +6164,7 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
         const bool partial = max_batches >= 0 && batches + nb > max_batches;
         if (partial) {
             if (persistent && lit)
-                launch_lit_persistent(g, a, q, 0, max_batches - batches, grid_max, team, nullptr, nullptr);
+                launch_lit_persistent(g, a, q, 0, max_batches - batches, grid_max, nullptr, nullptr);
             else if (persistent) launch_persistent(g, a, q, 0, max_batches - batches, grid_max, team, nullptr, nullptr);
             else if (lit) launch_batches_lit(g, a, q, 0, max_batches - batches);
             else launch_batches(g, a, q, 0, max_batches - batches);
@@ -6198,7 +6176,7 @@ void run_impl(lf_graph *g, int32_t q_in, double thr, int32_t max_iters, int64_t 
             break;
         }
         if (persistent) {
-            if (lit) launch_lit_persistent(g, a, q, 0, nb, grid_max, team, pev[0], pev[1]);
+            if (lit) launch_lit_persistent(g, a, q, 0, nb, grid_max, pev[0], pev[1]);
             else launch_persistent(g, a, q, 0, nb, grid_max, team, pev[0], pev[1]);
             launch_iteration_end(g, a);
         } else if (g->use_graphs > 0 && max_batches < 0) {

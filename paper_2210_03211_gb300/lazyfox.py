@@ -273,7 +273,7 @@ class Graph:
         opt.use_graphs = 0 if use_graphs else -1
         opt.profile = 1 if profile else 0
         opt.exhaustive_fp64 = 1 if exhaustive_fp64 else 0
-        # True: launches per queue; False: persistent loop; None: by queue size
+        # True: launches per queue; False: persistent loop (the literal rule: one-node queues); None: by queue size
         opt.per_queue_launches = 0 if per_queue_launches is None else (1 if per_queue_launches else 2)
         opt.barrier_timeout_ms = int(barrier_timeout_ms)
         opt.inject_barrier_stall = 1 if inject_barrier_stall else 0

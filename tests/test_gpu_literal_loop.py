@@ -40,3 +40,18 @@ def test_loop_plans_no_hub_kernels():
         assert alloc.live == 0
     # the loop's own: its barrier flags and one area of global tables
     assert made[None] <= made[True] - 13 + 2, made
+
+
+@pytest.mark.parametrize("q", [2, 64, 300])
+def test_longer_queues_are_launched_where_the_loop_is_preferred(q):
+    """Above one node the loop's grid barriers cost more than launches: preferring it
+    launches every queue all the same (the loop is one launch an iteration), and the
+    run is the same."""
+    from paper_2210_03211_gb300 import lazyfox
+    src, dst = graph()
+    runs = []
+    for per_queue in (False, True):
+        with lazyfox.Graph(src, dst, gain_rule="literal", profile=True, per_queue_launches=per_queue) as g:
+            runs.append(g.run(q, -np.inf, 3))
+        assert runs[-1].prof_move_launches == runs[-1].num_batches, per_queue
+    assert np.array_equal(runs[0].wcc_history, runs[1].wcc_history)
