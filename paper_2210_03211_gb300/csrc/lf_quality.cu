@@ -349,11 +349,18 @@ extern "C" lf_status lf_cover_f1(const int64_t *det_offsets, const int32_t *det_
         RefIndex ref{keys, eb, nullptr};
         const int64_t ids = (int64_t)max_id + 1;
         if (eb > 0 && ids <= 16 * (ea + eb) + (1 << 20)) {   // a table per id, unless the ids are far sparser than the covers
-            auto *range = static_cast<uint2 *>(alloc((size_t)ids * sizeof(uint2)));
-            LF_CUDA(cudaMemsetAsync(range, 0, (size_t)ids * sizeof(uint2), st));
-            k_ref_ranges<<<grid_for(eb, 256, 1 << 16), 256, 0, st>>>(keys, eb, range);
-            LF_LAUNCHED();
-            ref.range = range;
+            uint2 *range = nullptr;
+            try {
+                range = static_cast<uint2 *>(alloc((size_t)ids * sizeof(uint2)));
+            } catch (const Error &e) {   // no room: the keys are searched, which needs none
+                if (e.status != LF_ERR_OOM) throw;
+            }
+            if (range) {
+                LF_CUDA(cudaMemsetAsync(range, 0, (size_t)ids * sizeof(uint2), st));
+                k_ref_ranges<<<grid_for(eb, 256, 1 << 16), 256, 0, st>>>(keys, eb, range);
+                LF_LAUNCHED();
+                ref.range = range;
+            }
         }
         k_cover_f1<<<grid_for(num_det, F1_THREADS / 32, 152 * 5), F1_THREADS, 0, st>>>(oa, ma, num_det, ob, ref, sacc,
                                                                                        bst);
