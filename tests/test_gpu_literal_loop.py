@@ -1,7 +1,8 @@
-"""The persistent queue loop under the paper's gain (one block at queue size 1): what
-it plans and how it compares with the oracle on graphs with nodes of 513 to 1,024
-neighbours and rows of more than four communities, which launches per queue give
-to the hub kernels and the loop evaluates in its own block."""
+"""The persistent queue loop under the paper's gain: which queues take it, what it
+plans (on graphs with nodes of 513 to 1,024 neighbours and rows of more than four
+communities, which launches per queue give to the hub kernels and the loop evaluates
+in its own block), its central barrier over many blocks, and a handle's runs after a
+barrier ran out of time.  Compared with the oracle exactly."""
 import numpy as np
 import pytest
 
@@ -55,3 +56,43 @@ def test_longer_queues_are_launched_where_the_loop_is_preferred(q):
             runs.append(g.run(q, -np.inf, 3))
         assert runs[-1].prof_move_launches == runs[-1].num_batches, per_queue
     assert np.array_equal(runs[0].wcc_history, runs[1].wcc_history)
+
+
+@pytest.mark.parametrize("rule", ["literal", "meanfield"])
+@pytest.mark.parametrize("q", [2, 40, 700])
+def test_loop_of_many_blocks_with_the_central_barrier(rule, q):
+    """Several blocks meet at grid barriers that block 0 gathers and releases: the
+    oracle's run."""
+    import oracle
+    from paper_2210_03211_gb300 import lazyfox
+    src, dst = graph()
+    og = oracle.OracleGraph(src, dst)
+    ref = og.run(q, -np.inf, 3, rule=rule)
+    with lazyfox.Graph(src, dst, gain_rule=rule, barrier_mode=1, per_queue_launches=False, profile=True) as g:
+        st = g.run(q, -np.inf, 3)
+        assert st.prof_move_launches == st.iterations   # the loop: one launch an iteration
+        assert np.array_equal(st.wcc_history, ref["T"])
+        assert np.array_equal(st.joins, ref["joins"]) and np.array_equal(st.leaves, ref["leaves"])
+        s, o = g.state(), og.state()
+        for key in ("mem_off", "mem_ids", "n", "m", "vol"):
+            assert np.array_equal(s[key], o[key]), key
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_handle_is_usable_after_a_timeout(mode):
+    """A block that never arrives ends the run with LF_ERR_TIMEOUT in either barrier
+    mode.  The same handle then runs at queue size 1, where one block meets nobody:
+    nothing of the abandoned run is left over."""
+    import oracle
+    from paper_2210_03211_gb300 import lazyfox
+    src, dst = graph()
+    ref = oracle.OracleGraph(src, dst).run(1, 0.01, 3, rule="literal")
+    with lazyfox.Graph(src, dst, gain_rule="literal", inject_barrier_stall=True, barrier_timeout_ms=50,
+                       barrier_mode=mode, per_queue_launches=False) as g:
+        for _ in range(2):
+            with pytest.raises(lazyfox.LazyFoxError) as e:
+                g.run(64, 0.01, 3)
+            assert e.value.status == lazyfox.LF_ERR_TIMEOUT
+            st = g.run(1, 0.01, 3)
+            assert np.array_equal(st.wcc_history, ref["T"])
+            assert np.array_equal(st.joins, ref["joins"]) and np.array_equal(st.leaves, ref["leaves"])
