@@ -316,15 +316,20 @@ __device__ __forceinline__ int warp_scan_inclusive(int x, int lane) {
     return x;
 }
 
+// The lowest n of 32 bits (n below 0: none, above 32: all).
+__device__ __forceinline__ unsigned bits_below(int n) { return n <= 0 ? 0u : n >= 32 ? FULL : (1u << n) - 1u; }
+
 // Nodes with 2 <= d+(u) <= TRI_FLAT_MAX.  Their streams are a few elements
 // long, so a warp per node spends its time in the node's chain of dependent
 // loads and in clearing a hash table.  Here a warp lays the out-edges of up to
 // 32 consecutive nodes end to end over its lanes, then the out-lists of 32 such
 // edges, so every lane has an element whatever the lists' lengths, and tests it
-// by a binary search of N+(u) (at most five loads, in the first-level cache: the
-// warp has just read that row).  Triangles are credited by global atomics; the
-// rows are short, so there are few per element.
-// 335k nodes, 0.93M edges: 133 (a warp and a hash table per node) -> 39 us.
+// by a binary search of N+(u) (at most six loads, in the first-level cache: the
+// warp has just read that row).  Triangles are credited by global atomics, one for
+// all of a warp's 32 elements (edges) with the same node: few nodes that close most
+// triangles would queue them up on a few addresses.
+// 335k nodes, 0.93M edges: 133 (a warp and a hash table per node) -> 39 us.  A million
+// nodes joined to the same two: 1.33 (an atomic per triangle) -> 0.14 ms.
 constexpr int TRI_FLAT_MAX = 32;
 
 __global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int32_t *__restrict__ oadj, int64_t n,
@@ -356,31 +361,44 @@ __global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int
             }
             const int inc2 = warp_scan_inclusive(len, lane);
             const int total = __shfl_sync(FULL, inc2, 31);
-            int mine = 0;   // triangles closed by this lane's elements
+            int mine = 0;   // triangles closed on this lane's edge
             for (int f0 = 0; f0 < total; f0 += 32) {
                 const int f = f0 + lane;
                 const int q = flat_owner(inc2, f);
                 const int64_t at = __shfl_sync(FULL, vs, q) + (f - (__shfl_sync(FULL, inc2, q) - __shfl_sync(FULL, len, q)));
                 const int64_t rs = __shfl_sync(FULL, us, q);
                 const int rd = __shfl_sync(FULL, ud, q);
-                const int rk = __shfl_sync(FULL, k, q);
-                const int32_t rv = __shfl_sync(FULL, v, q);
-                const int64_t ru = u0 + __shfl_sync(FULL, j, q);
+                bool hit = false;
+                int32_t x = 0;
                 if (f < total) {
-                    const int32_t x = oadj[at];
+                    x = oadj[at];
                     const int idx = find_sorted(oadj + rs, rd, x);
                     if (idx >= 0) {
-                        atomicAdd(&tri[ru], 1ull);
-                        atomicAdd(&tri[rv], 1ull);
-                        atomicAdd(&tri[x], 1ull);
+                        hit = true;
                         sup[at] = 1;
-                        sup[rs + rk] = 1;
                         sup[rs + idx] = 1;
-                        ++mine;
                     }
                 }
-                __syncwarp();
+                const unsigned hits = __ballot_sync(FULL, hit);
+                if (hits) {
+                    mine += __popc(hits & bits_below(inc2 - f0) & ~bits_below(inc2 - len - f0));
+                    if (hit) {
+                        const unsigned same = __match_any_sync(hits, x);
+                        if (lane == __ffs(same) - 1) atomicAdd(&tri[x], (unsigned long long)__popc(same));
+                    }
+                }
             }
+            const unsigned has = __ballot_sync(FULL, mine > 0);
+            if (mine > 0) {
+                sup[us + k] = 1;
+                const unsigned sv = __match_any_sync(has, v);
+                const int cv = __reduce_add_sync(sv, mine);
+                if (lane == __ffs(sv) - 1) atomicAdd(&tri[v], (unsigned long long)cv);
+                const unsigned su = __match_any_sync(has, j);
+                const int cu = __reduce_add_sync(su, mine);
+                if (lane == __ffs(su) - 1) atomicAdd(&tri[u0 + j], (unsigned long long)cu);
+            }
+            __syncwarp();
             found += (unsigned long long)__reduce_add_sync(FULL, mine);
         }
     }
