@@ -410,11 +410,13 @@ __global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int
     }
 }
 
-// One warp per node u with TRI_FLAT_MAX < d+(u) <= TRI_WARP_MAX; warps of a
-// resident grid take runs of up to 32 consecutive nodes, whose offsets load
-// together and of which one ballot picks the ones to do.
+// One warp per node u with above < d+(u) <= TRI_WARP_MAX.  Warps take runs of up to 32
+// consecutive nodes, in a fixed order or, where their streams differ widely and there
+// are many, from a counter (100k nodes, m/n 80: 3.25 -> 2.54 ms); a run's offsets load
+// together and one ballot picks the nodes to do.  A table has four slots an id as
+// far as it goes: with two, lookups walk longer than clearing costs (m/n 40: 0.93 -> 0.77 ms).
 __global__ void __launch_bounds__(256) k_tri_warp(const int64_t *ooff, const int32_t *__restrict__ oadj, int64_t n,
-                                                  int run, unsigned long long *tri, uint8_t *sup, DevScalars *ds) {
+                                                  int run, int above, uint32_t *next, unsigned long long *tri, uint8_t *sup, DevScalars *ds) {
     __shared__ long long s_base[8][TRI_WARP_MAX];
     __shared__ int32_t s_list[8][TRI_WARP_MAX];
     __shared__ int32_t s_pre[8][TRI_WARP_MAX + 1];
@@ -426,19 +428,25 @@ __global__ void __launch_bounds__(256) k_tri_warp(const int64_t *ooff, const int
     int32_t *list = s_list[w], *pre = s_pre[w], *cnt = s_cnt[w], *hk = s_hk[w];
     long long *base = s_base[w];
     uint8_t *hp = s_hp[w];
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     unsigned long long found = 0;
-    for (int64_t u0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * run; u0 < n; u0 += warps * run) {
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t at = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;; at += warps) {
+        int64_t u0 = at * run;
+        if (next) {
+            if (lane == 0) u0 = (int64_t)atomicAdd(next, 1u) * run;
+            u0 = __shfl_sync(FULL, u0, 0);
+        }
+        if (u0 >= n) break;
         const int64_t ul = min(n, u0 + lane);
         const int64_t sl = ooff[ul], dl = ooff[min(n, ul + 1)] - sl;
-        unsigned todo = __ballot_sync(FULL, lane < run && dl > TRI_FLAT_MAX && dl <= TRI_WARP_MAX);
+        unsigned todo = __ballot_sync(FULL, lane < run && dl > above && dl <= TRI_WARP_MAX);
         while (todo) {
             const int src = __ffs(todo) - 1;
             todo &= todo - 1;
             const int64_t u = u0 + src;
             const int64_t s = __shfl_sync(FULL, sl, src);
             const int du = (int)__shfl_sync(FULL, dl, src);
-            const uint32_t hs = max(32u, 2u << (31 - __clz(2 * du - 1)));   // pow2 >= 2 du
+            const uint32_t hs = min((uint32_t)TW_HASH, 2u << (31 - __clz(4 * du - 1)));   // pow2 >= 4 du, or all (>= 2 du)
             for (uint32_t k = lane; k < hs; k += 32) hk[k] = -1;
             int carry = 0;
             for (int k0 = 0; k0 < du; k0 += 32) {
@@ -677,31 +685,45 @@ void set_triangle_attrs() {
 
 // lf_graph_create takes this path up to this mean out-degree m / n, the
 // middle-vertex kernels above it.  Measured (ms; this path / the other):
-// m/n 2.8 and 335k nodes 0.06 / 0.19, 7.9 and 300k nodes 0.23 / 0.34, 9.1
-// (planted) and 300k nodes 0.21 / 0.30, 11.6 and 200k nodes 0.30 / 0.40, 15 and
-// 100k nodes 0.76 / 0.64, 19 (planted) and 61k nodes 0.22 / 0.25, 28 and 100k nodes
-// 1.82 / 1.04: the streams of the lowest vertices grow faster with the mean
-// degree and its spread.
-constexpr int64_t FLAT_MAX_MEAN = 10;
+// m/n 2.8 and 335k nodes 0.07 / 0.25, 9 and 300k nodes 0.20 / 0.36, 9.5 (cliques of 20) and
+// 40k nodes 0.07 / 0.29.
+constexpr int64_t SOURCE_MAX_MEAN = 10;
 
-// Triangle counts and support marks of an oriented graph with n > 0 nodes.
-// `hubs` holds n ints of scratch and `nh` two counters that start at zero.
+// On it, the flat kernel takes the short rows up to this mean, and k_tri_warp all rows
+// above: a binary search per element is the cheaper test while streams are short,
+// a hash table once they are long, which a few high degrees are enough for.
+// lf_triangles_noalloc, ms, flat / hash: 100k nodes of even degrees m/n 3 0.071 / 0.093,
+// 6 0.090 / 0.114, 10 0.128 / 0.136; of skewed degrees m/n 4 0.16 / 0.14, 7 0.45 / 0.19, 10 0.69 /
+// 0.23; cliques of 33 0.15 / 0.08, of 100 0.87 / 0.51; 335k nodes m/n 2.8 0.116 / 0.139.
+constexpr int64_t FLAT_MAX_MEAN = 6;
+
+// Triangle counts and support marks of an oriented graph with n > 0 nodes and m edges.
+// `hubs` holds n ints of scratch and `nh` three counters that start at zero.
 // Returns the number of kernels launched.
-int launch_triangles(const int64_t *ooff, const int32_t *oadj, int64_t n, int32_t *hubs, uint32_t *nh,
+int launch_triangles(const int64_t *ooff, const int32_t *oadj, int64_t n, int64_t m, int32_t *hubs, uint32_t *nh,
                      unsigned long long *tri, uint8_t *sup, DevScalars *ds, cudaStream_t st) {
     const int sms = 152;
+    const bool flat = m <= FLAT_MAX_MEAN * n;
     k_select_hubs<<<grid_for(n, 256, 8192), 256, 0, st>>>(ooff, n, hubs, nh);
     LF_LAUNCHED();
-    const int run = (int)std::min<int64_t>(32, std::max<int64_t>(1, n / (2 * 8 * 6 * sms)));
-    k_tri_flat<<<grid_for(n, 8 * run, 6 * sms), 256, 0, st>>>(ooff, oadj, n, run, tri, sup, ds);
-    LF_LAUNCHED();
-    k_tri_warp<<<grid_for(n, 8 * run, 6 * sms), 256, 0, st>>>(ooff, oadj, n, run, tri, sup, ds);
+    const int64_t blocks = 6 * sms, warps = 8 * blocks;   // resident
+    if (flat) {   // leaves few rows to k_tri_warp: fixed runs
+        const int run = (int)std::min<int64_t>(32, std::max<int64_t>(1, n / (2 * warps)));
+        k_tri_flat<<<grid_for(n, 8 * run, blocks), 256, 0, st>>>(ooff, oadj, n, run, tri, sup, ds);
+        LF_LAUNCHED();
+        k_tri_warp<<<grid_for(n, 8 * run, blocks), 256, 0, st>>>(ooff, oadj, n, run, TRI_FLAT_MAX, nullptr, tri, sup, ds);
+    } else if (n < 4 * warps) {   // a node a warp: the counter's atomics would cost more than they balance
+        k_tri_warp<<<grid_for(n, 8, 4 * blocks), 256, 0, st>>>(ooff, oadj, n, 1, 1, nullptr, tri, sup, ds);
+    } else {
+        const int run = (int)std::min<int64_t>(32, n / (4 * warps));
+        k_tri_warp<<<(unsigned)blocks, 256, 0, st>>>(ooff, oadj, n, run, 1, nh + 2, tri, sup, ds);
+    }
     LF_LAUNCHED();
     k_tri_mid<<<sms * 8, TRI_MID_THREADS, TRI_MID_SMEM, st>>>(ooff, oadj, hubs, nh, tri, sup, ds);
     LF_LAUNCHED();
     k_tri_block<<<2 * sms, TRI_BLOCK_THREADS, TRI_BIG_SMEM, st>>>(ooff, oadj, hubs + n, nh + 1, tri, sup, ds);
     LF_LAUNCHED();
-    return 5;
+    return flat ? 5 : 4;
 }
 
 
@@ -1306,16 +1328,17 @@ int launch_tv(const int64_t *off, const int32_t *adj, const int32_t *deg, const 
 int64_t tv_item_cap(int64_t m) { return 2 * m / (TV_WARP_DPLUS + 1) + 2 * m / TV_ITEM + 2; }
 
 // ---- a4 --------------------------------------------------------------------
-// vt: groups of eight lanes take a node each (mean out-degrees are small), on a
-// resident grid.  The merge-stream byte count leaves a block as one atomic:
+// vt: groups of LANES lanes take a node each, on a resident grid (eight; a whole warp
+// where rows are long).  The merge-stream byte count leaves a block as one atomic:
 // one per node's warp queued hundreds of thousands of atomics on one address,
 // which was nearly all of the kernel's time (335k nodes: 231 -> 23 us).
+template <int LANES>
 __global__ void __launch_bounds__(256) k_vt(const int64_t *ooff, const int32_t *oadj, const uint8_t *sup, int64_t n,
                                             int32_t *vt, DevScalars *ds) {
     __shared__ unsigned long long s_mb[8];
-    const int sub = threadIdx.x & 7, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> 3;
-    const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int sub = threadIdx.x & (LANES - 1), lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t groups = (int64_t)gridDim.x * (blockDim.x / LANES);
+    const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
     unsigned long long mb = 0;
     for (int64_t b = 0; b < n; b += groups) {   // the whole warp stays together for the shuffles
         const int64_t u = b + g0;
@@ -1323,7 +1346,7 @@ __global__ void __launch_bounds__(256) k_vt(const int64_t *ooff, const int32_t *
         if (u < n) {
             const int64_t s = ooff[u], e = ooff[u + 1];
             const int64_t du = e - s;
-            for (int64_t p = s + sub; p < e; p += 8) {
+            for (int64_t p = s + sub; p < e; p += LANES) {
                 const int32_t v = oadj[p];
                 mb += 4ull * (unsigned long long)(du + (ooff[v + 1] - ooff[v]));
                 if (sup[p]) {
@@ -1333,7 +1356,7 @@ __global__ void __launch_bounds__(256) k_vt(const int64_t *ooff, const int32_t *
             }
         }
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
+        for (int o = LANES / 2; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
         if (sub == 0 && cnt) atomicAdd(&vt[u], cnt);
     }
 #pragma unroll
@@ -1344,6 +1367,16 @@ __global__ void __launch_bounds__(256) k_vt(const int64_t *ooff, const int32_t *
         for (int k = 1; k < 8; ++k) mb += s_mb[k];
         if (mb) atomicAdd(&ds->merge_bytes, mb);
     }
+}
+
+// us, 8 lanes / 32: 100k nodes, m/n 28 24 / 35, 80 65 / 74; 22k nodes, m/n 215 120 / 97.
+constexpr int64_t VT_WARP_MEAN = 128;
+
+void launch_vt(const int64_t *ooff, const int32_t *oadj, const uint8_t *sup, int64_t n, int64_t m, int32_t *vt,
+               DevScalars *ds, cudaStream_t st) {
+    if (m <= VT_WARP_MEAN * n) k_vt<8><<<grid_for(n * 8, 256, 8 * sm_count()), 256, 0, st>>>(ooff, oadj, sup, n, vt, ds);
+    else k_vt<32><<<grid_for(n * 32, 256, 8 * sm_count()), 256, 0, st>>>(ooff, oadj, sup, n, vt, ds);
+    LF_LAUNCHED();
 }
 
 // ---- a5 --------------------------------------------------------------------
@@ -1662,12 +1695,12 @@ void build_graph(lf_graph *g, const int32_t *src, const int32_t *dst, int64_t E,
     LF_CUDA(cudaMemsetAsync(g->vt, 0, (size_t)(n > 0 ? n : 1) * 4, st));
     LF_CUDA(cudaMemsetAsync(sup, 0, (size_t)(m > 0 ? m : 1), st));
     unsigned long long *utri = reinterpret_cast<unsigned long long *>(g->tri);
-    if (n > 0 && m <= FLAT_MAX_MEAN * n) {
+    if (n > 0 && m <= SOURCE_MAX_MEAN * n) {
         int32_t *hubs = dalloc_n<int32_t>(g, n);
         uint32_t *nh = reinterpret_cast<uint32_t *>(tmp64);
-        LF_CUDA(cudaMemsetAsync(nh, 0, 2 * sizeof(uint32_t), st));
+        LF_CUDA(cudaMemsetAsync(nh, 0, 3 * sizeof(uint32_t), st));
         set_triangle_attrs();
-        g->launches += launch_triangles(g->ooff, g->oadj, n, hubs, nh, utri, sup, ds, st);
+        g->launches += launch_triangles(g->ooff, g->oadj, n, m, hubs, nh, utri, sup, ds, st);
         dfree(g, hubs);
     } else if (n > 0) {
         const int64_t cap = tv_item_cap(m);
@@ -1685,8 +1718,7 @@ void build_graph(lf_graph *g, const int32_t *src, const int32_t *dst, int64_t E,
     }
     pt.mark();   // 3
     if (n > 0) {
-        k_vt<<<grid_for(n * 8, 256, 8 * sm_count()), 256, 0, st>>>(g->ooff, g->oadj, sup, n, g->vt, ds); ++g->launches;
-        LF_LAUNCHED();
+        launch_vt(g->ooff, g->oadj, sup, n, m, g->vt, ds, st); ++g->launches;
     }
     dfree(g, sup);
     pt.mark();   // 4
@@ -1857,7 +1889,7 @@ void triangles_noalloc(const int64_t *ooff, const int32_t *oadj, int64_t n, int6
     uint8_t *sup = base + round256(sizeof(DevScalars)) + 256 + round256((size_t)n * sizeof(int32_t));
     // the array keeps the previous call's contents: clear what must start at zero
     LF_CUDA(cudaMemsetAsync(ds, 0, sizeof(DevScalars), st));
-    LF_CUDA(cudaMemsetAsync(nh, 0, 2 * sizeof(uint32_t), st));
+    LF_CUDA(cudaMemsetAsync(nh, 0, 3 * sizeof(uint32_t), st));
     if (m > 0) LF_CUDA(cudaMemsetAsync(sup, 0, (size_t)m, st));
     if (n == 0) return;
     // validate the input first (its flag is a word of the array; the host
@@ -1873,9 +1905,8 @@ void triangles_noalloc(const int64_t *ooff, const int32_t *oadj, int64_t n, int6
     LF_CUDA(cudaMemsetAsync(t, 0, (size_t)n * sizeof(int64_t), st));
     LF_CUDA(cudaMemsetAsync(vt, 0, (size_t)n * sizeof(int32_t), st));
     unsigned long long *utri = reinterpret_cast<unsigned long long *>(t);
-    launch_triangles(ooff, oadj, n, hubs, nh, utri, sup, ds, st);
-    k_vt<<<grid_for(n * 8, 256, 8 * sm_count()), 256, 0, st>>>(ooff, oadj, sup, n, vt, ds);
-    LF_LAUNCHED();
+    launch_triangles(ooff, oadj, n, m, hubs, nh, utri, sup, ds, st);
+    launch_vt(ooff, oadj, sup, n, m, vt, ds, st);
 }
 
 }  // namespace lf
