@@ -229,7 +229,8 @@ __device__ __forceinline__ int find_sorted(const int32_t *list, int len, int32_t
 // (prefix sums of their lengths in shared memory) and consumed 32 elements
 // per lane group whatever the v boundaries, so short lists leave no lanes
 // idle; each lane issues TRI_UNROLL independent loads before it uses any.
-// Membership in N+(u) goes through a shared-memory hash table of the ids.
+// Membership in N+(u) goes through a shared-memory hash table of the ids (k_tri_flat,
+// for short rows, searches N+(u) itself).
 
 constexpr int TRI_UNROLL = 4;
 constexpr int TW_HASH = 2 * TRI_WARP_MAX;   // slots of a warp's table (load <= 1/2)

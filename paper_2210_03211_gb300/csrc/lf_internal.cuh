@@ -230,8 +230,9 @@ struct lf_graph {
     // the paper's gain (gain_rule == LF_GAIN_LITERAL): deg(x,C) beside each
     // membership, the member index of the current iteration (members at its
     // start, by community; its joiners as per-community lists), per-community
-    // sums F(n-1), F(n), F(n+1), per-queue counters (overflow count, overflow
-    // next, touched count, apply items), the overflow list, the touched list and stamps
+    // sums F(n-1), F(n), F(n+1), per-queue counters (of eight: [0] nodes listed for a
+    // block, [1] taken, [2] communities touched, [3] apply items, [4] nodes listed for
+    // two warps, [5] taken), the two lists, the touched list and stamps
     int32_t *kmem = nullptr;              // n*K
     unsigned long long *cm_off = nullptr; // n+1
     unsigned long long *cm_cur = nullptr; // n+1

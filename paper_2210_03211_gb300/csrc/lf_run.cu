@@ -1839,7 +1839,7 @@ __global__ void __launch_bounds__(AP_THREADS) k_apply(RunArgs a, int64_t bstart,
 // of the real one (M: the same expression with every term's magnitude; the
 // FP64 sums are at most 2n + k + 40 roundings of non-negative terms, the
 // float path about ten roundings of 2^-24 on terms bounded by M (1.5e-6 is
-// 25 of them), a correction about ten roundings plus one per addition --
+// 25 of them), a correction at most ten roundings plus one per addition --
 // every count taken about twice over).  Per kind, candidates whose upper end cannot reach
 // the best lower end (or 0) are dropped; one surviving candidate with a
 // positive lower end is the answer; otherwise the survivors' gains are
@@ -1928,7 +1928,7 @@ __device__ __forceinline__ int row_find(const int32_t *row, int32_t cnt, int32_t
 }
 
 // The first eight ids of node y's membership row (rows start on 16-byte
-// boundaries; K is 4 or a multiple of 8): loads that do not wait for the row's
+// boundaries; K is a multiple of 4): loads that do not wait for the row's
 // count, so that count, ids and whatever else of y is wanted arrive together.
 struct RowHead {
     int4 a, b;
@@ -1997,9 +1997,9 @@ __device__ __forceinline__ bool adj_has(const int32_t *adj, int64_t beg, int64_t
 //        (a neighbour y of a joining x; y is not x, so k <= d - 1 and D - 1 >= n >= 1),
 //   h- = g(n-1; k-1) - g(n-1; k) = -d (C(k-1,2) + (k-1)(D+1)) / (C(d,2) D (D+1)),
 //        D = n - 2 + d - k (used only when n - 1 >= 2, so D >= 1),
-// and x's own g, in FP32 (about ten roundings each, relative error
-// < 16 x 2^-24; a sum of k of them adds k roundings): used only in the
-// bracket, whose bound E carries a term for them.
+// and x's own g, in FP32 (relative error < 16 x 2^-24; a sum of k of them
+// adds k roundings): used only in the bracket, whose bound E carries a term for
+// them.
 // With kk = k, E = n + d - k for a join and kk = k - 1, E = n - 1 + d - k for a leave
 // both corrections are one expression up to the sign,
 //   h = kk (2 E + kk - 1) / ((d - 1) E (E - 1)),
@@ -2028,7 +2028,7 @@ __device__ __forceinline__ float lit_g32(uint32_t k, uint32_t d, uint32_t nu) {
     return (kf * (kf - 1.f)) / (__uint2float_rn(d - 1u) * __uint2float_rn(den1 - 1));
 }
 
-// Bracket of one candidate: FP64 value X of the expression above and a bound
+// Bracket of one candidate: FP32 value X of the expression above and a bound
 // E on its distance from the exactly summed, once rounded gain.
 __device__ __forceinline__ void lit_screen(const RunArgs &a, int32_t C, uint32_t v, int32_t d, float Hs, float &X,
                                            float &E) {
@@ -2374,12 +2374,10 @@ __device__ __forceinline__ void lit_screen_table(const RunArgs &a, int32_t d, in
     team_sync<T>(tm);
 }
 
-// One pass over the node's candidates of part p (of P): the table gets x's
-// own communities (own flag), then every neighbour membership (y, C) adds
-// one to C's count and its correction h(y) (by C's size before the queue and
-// whether C is x's own) to C's sum (dv); then each candidate's bracket:
-// dv <- X, aux <- E (as a float rounded up).  Per lane: the largest lower
-// ends of the two kinds.  Returns false (team-wide) if the table overflowed.
+// The node's candidates of part p (of P) in the table: x's own communities (own
+// flag), then every neighbour membership (y, C) adds one to C's count and its
+// correction h(y) (by C's size before the queue and whether C is x's own) to C's
+// sum.  Returns false (team-wide) if the table overflowed.
 template <int T>
 __device__ __forceinline__ bool lit_fill(const RunArgs &a, const LitNode &ln, int P, int p, int32_t *keys, uint32_t *vals,
                                          int32_t *aux, uint32_t H, LitScratch &ls, int tm, int w_in,
@@ -2427,6 +2425,8 @@ __device__ __forceinline__ bool lit_fill(const RunArgs &a, const LitNode &ln, in
     return ok;
 }
 
+// One pass over a part: filled, then each candidate's bracket: dv <- X, aux <- E (as a
+// float rounded up).  Per lane: the largest lower ends of the two kinds.
 template <int T>
 __device__ bool lit_pass(const RunArgs &a, const LitNode &ln, int P, int p, int32_t *keys, uint32_t *vals,
                          int32_t *aux, float *dv, uint32_t H, LitScratch &ls, int tm, int w_in, float &lbj,
@@ -2622,7 +2622,7 @@ __device__ __forceinline__ void lit_finish(const RunArgs &a, int i, const LitNod
 }
 
 // One shared table that holds all candidates, screened and decided over the
-// list of its used slots: tables are at most half full and mostly far emptier, and
+// list of its used slots: tables are at most three quarters full and mostly far emptier, and
 // a scan of the slots left most lanes idle and, worse, gave a warp one dependent
 // gather of the communities' records per 32 slots; over the list it is one per 32
 // candidates.
@@ -3122,7 +3122,7 @@ __global__ void __launch_bounds__(EV_THREADS, 3) k_lit_big(RunArgs a, int64_t bs
 }
 
 // ---------------------------------------------------------------------------
-// Hubs under the paper's gain: a queued node of degree > LIT_HUB_DEG has more
+// Hubs under the paper's gain: a queued node of degree > lit_hub_degree() has more
 // entries than a block's table holds.  Its entries are partitioned by community
 // instead of meeting in one table in global memory (three global atomics per
 // entry on three sectors, then two scans of a table sized for the worst case):
@@ -5331,9 +5331,9 @@ LitHubPlan lit_hub_plan(lf_graph *g) {
 }
 
 // Per-queue launches under the paper's gain: teams evaluate the queue's nodes
-// (k_lit_eval), blocks take the nodes too large for a team (k_lit_big), then
-// the apply, the neighbours' deg(y,C) updates and the touched communities'
-// sums.
+// (k_lit_eval), in long queues teams of two warps and blocks take the nodes too
+// large for theirs (k_lit_mid, k_lit_big), the hub kernels the hubs, then the apply and
+// the touched communities' sums.
 void launch_batches_lit(lf_graph *g, const RunArgs &a, int64_t q, int64_t first, int64_t count,
                         bool capturing = false) {
     const bool sched = !g->sched.empty();
