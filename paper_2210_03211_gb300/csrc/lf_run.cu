@@ -3780,8 +3780,8 @@ __global__ void __launch_bounds__(AP_THREADS) k_lit_apply(RunArgs a, int64_t bst
 // members, and the block those above LIT_FSUM_WARP; a member's count, ids,
 // deg(y,C) and degree load together, not one after another; its three terms
 // share one division; and the stored factors are formed by three lanes at once.
-// Mean over the queues: 767k nodes, q 16,384: 112 -> 59 us; 3.07M nodes, q 65,536:
-// 460 -> 111 us; 335k nodes, q 1,024: 23 -> 20 us (cold caches).
+// Mean over the queues: 767k nodes, q 16,384: 112 -> 56 us; 3.07M nodes, q 65,536:
+// 460 -> 141 us (cold caches; 45 and 112 us of it without lit_g3's corrections).
 constexpr int LIT_FSUM_GROUP = 64;
 constexpr int LIT_FSUM_WARP = 512;
 constexpr int LIT_FSUM_FEW = 128;    // the same where entries are few
