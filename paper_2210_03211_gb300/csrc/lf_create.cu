@@ -326,12 +326,15 @@ __device__ __forceinline__ unsigned bits_below(int n) { return n <= 0 ? 0u : n >
 // 32 consecutive nodes end to end over its lanes, then the out-lists of 32 such
 // edges, so every lane has an element whatever the lists' lengths, and tests it
 // by a binary search of N+(u) (at most six loads, in the first-level cache: the
-// warp has just read that row).  Triangles are credited by global atomics, one for
-// all of a warp's 32 elements (edges) with the same node: few nodes that close most
-// triangles would queue them up on a few addresses.
+// warp has just read that row).  Triangles are credited by global atomics: an edge's
+// own nodes once per edge, and, where TRI_FLAT_MATCH of a warp's elements (edges) have a
+// credit, equal nodes among them once, as few nodes that close most triangles would
+// queue the atomics up on a few addresses (looked for always,
+// 335k nodes take 2% longer; from 24 lanes, a million pages joined to two nodes miss it).
 // 335k nodes, 0.93M edges: 133 (a warp and a hash table per node) -> 39 us.  A million
 // nodes joined to the same two: 1.33 (an atomic per triangle) -> 0.14 ms.
 constexpr int TRI_FLAT_MAX = 32;
+constexpr int TRI_FLAT_MATCH = 16;
 
 __global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int32_t *__restrict__ oadj, int64_t n,
                                                   int run, unsigned long long *tri, uint8_t *sup, DevScalars *ds) {
@@ -384,7 +387,7 @@ __global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int
                 if (hits) {
                     mine += __popc(hits & bits_below(inc2 - f0) & ~bits_below(inc2 - len - f0));
                     if (hit) {
-                        const unsigned same = __match_any_sync(hits, x);
+                        const unsigned same = __popc(hits) < TRI_FLAT_MATCH ? 1u << lane : __match_any_sync(hits, x);
                         if (lane == __ffs(same) - 1) atomicAdd(&tri[x], (unsigned long long)__popc(same));
                     }
                 }
@@ -392,12 +395,14 @@ __global__ void __launch_bounds__(256) k_tri_flat(const int64_t *ooff, const int
             const unsigned has = __ballot_sync(FULL, mine > 0);
             if (mine > 0) {
                 sup[us + k] = 1;
-                const unsigned sv = __match_any_sync(has, v);
-                const int cv = __reduce_add_sync(sv, mine);
-                if (lane == __ffs(sv) - 1) atomicAdd(&tri[v], (unsigned long long)cv);
-                const unsigned su = __match_any_sync(has, j);
-                const int cu = __reduce_add_sync(su, mine);
-                if (lane == __ffs(su) - 1) atomicAdd(&tri[u0 + j], (unsigned long long)cu);
+                atomicAdd(&tri[u0 + j], (unsigned long long)mine);
+                if (__popc(has) < TRI_FLAT_MATCH) {
+                    atomicAdd(&tri[v], (unsigned long long)mine);
+                } else {
+                    const unsigned sv = __match_any_sync(has, v);
+                    const int cv = __reduce_add_sync(sv, mine);
+                    if (lane == __ffs(sv) - 1) atomicAdd(&tri[v], (unsigned long long)cv);
+                }
             }
             __syncwarp();
             found += (unsigned long long)__reduce_add_sync(FULL, mine);
